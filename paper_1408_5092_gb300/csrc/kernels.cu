@@ -1,5 +1,5 @@
-// CUDA-core kernels of the MPS-PT hot path (sm_103a): grouped block GEMM
-// (float64 / float32) driven by task lists, Jacobi diagonal, batched Jacobi
+// CUDA-core kernels of the MPS-PT hot path (sm_103a): grouped block GEMM in
+// float32 arithmetic driven by task lists, Jacobi diagonal, batched Jacobi
 // eigensolver for the density-matrix blocks, block copies, and the CG vector
 // kernels with deterministic (fixed-order) reductions.
 #include "kernels.h"
@@ -44,54 +44,47 @@ __device__ __forceinline__ float d2f_rn(double v) {
     if (rem > 0x10000000u || (rem == 0x10000000u && (mant & 1u))) f += 1u;
     return __uint_as_float(f);
 }
-template <class U>
-__device__ __forceinline__ U conv(double v);
-template <>
-__device__ __forceinline__ double conv<double>(double v) { return v; }
-template <>
-__device__ __forceinline__ float conv<float>(double v) { return d2f_rn(v); }
-
 // Grouped GEMM: one CTA per output tile, looping over the tile's K-list.
 // 16x16 threads; thread (tx, ty) owns rows ty + 16 i (i < TM/16) and
-// cols tx + 16 j (j < TN/16).  T: storage type, U: arithmetic type.
+// cols tx + 16 j (j < TN/16).  Operands and results are float64.
 // Persistent: the grid is at most the resident CTAs of the GPU, and CTA b
 // takes tasks b, b + gridDim.x, ... (the planner orders tasks longest first).
-template <int TM, int TN, class T, class Task, class Op, class U = T>
-__global__ void __launch_bounds__(NT) k_gemm(const Task* __restrict__ tasks, int ntask,
-                                             const Op* __restrict__ ops,
+template <int TM, int TN>
+__global__ void __launch_bounds__(NT) k_gemm(const GemmTask* __restrict__ tasks, int ntask,
+                                             const GemmOp* __restrict__ ops,
                                              const int* __restrict__ skip) {
     if (skip && *skip) return;
     constexpr int RI = TM / 16, RJ = TN / 16;
-    __shared__ U As[TK][TM + 1];
-    __shared__ U Bs[TK][TN + 1];
+    __shared__ float As[TK][TM + 1];
+    __shared__ float Bs[TK][TN + 1];
     const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
   for (int ti = blockIdx.x; ti < ntask; ti += gridDim.x) {
-    const Task t = tasks[ti];
-    U acc[RI][RJ];
+    const GemmTask t = tasks[ti];
+    float acc[RI][RJ];
 #pragma unroll
     for (int i = 0; i < RI; ++i)
 #pragma unroll
-        for (int j = 0; j < RJ; ++j) acc[i][j] = U(0);
+        for (int j = 0; j < RJ; ++j) acc[i][j] = 0.f;
     const int mrem = min(TM, t.m - t.r0);
     const int nrem = min(TN, t.n - t.c0);
     int kbase = 0;   // position of op o's first K index in the concatenated K-list
     for (int o = t.op0; o < t.op1; ++o) {
-        const Op op = ops[o];
+        const GemmOp op = ops[o];
         const int kb = max(0, t.kb - kbase), ke = min(op.k, t.ke - kbase);
         kbase += op.k;
         if (kb >= ke) continue;
         const bool ta = op.trans & 1, tb = op.trans & 2;
-        const U alpha = conv<U>(op.alpha);
+        const float alpha = d2f_rn(op.alpha);
         for (int k0 = kb; k0 < ke; k0 += TK) {
             const int krem = min(TK, ke - k0);
             for (int e = threadIdx.x; e < TM * TK; e += NT) {
                 int i, kk;
                 if (ta) { i = e % TM; kk = e / TM; }
                 else { kk = e % TK; i = e / TK; }
-                U v = U(0);
+                float v = 0.f;
                 if (i < mrem && kk < krem) {
                     const int row = t.r0 + i, kg = k0 + kk;
-                    v = conv<U>(ta ? op.A[(size_t)kg * op.lda + row] : op.A[(size_t)row * op.lda + kg]) * alpha;
+                    v = d2f_rn(ta ? op.A[(size_t)kg * op.lda + row] : op.A[(size_t)row * op.lda + kg]) * alpha;
                 }
                 As[kk][i] = v;
             }
@@ -99,17 +92,17 @@ __global__ void __launch_bounds__(NT) k_gemm(const Task* __restrict__ tasks, int
                 int j, kk;
                 if (tb) { kk = e % TK; j = e / TK; }
                 else { j = e % TN; kk = e / TN; }
-                U v = U(0);
+                float v = 0.f;
                 if (j < nrem && kk < krem) {
                     const int col = t.c0 + j, kg = k0 + kk;
-                    v = conv<U>(tb ? op.B[(size_t)col * op.ldb + kg] : op.B[(size_t)kg * op.ldb + col]);
+                    v = d2f_rn(tb ? op.B[(size_t)col * op.ldb + kg] : op.B[(size_t)kg * op.ldb + col]);
                 }
                 Bs[kk][j] = v;
             }
             __syncthreads();
 #pragma unroll
             for (int kk = 0; kk < TK; ++kk) {
-                U a[RI], b[RJ];
+                float a[RI], b[RJ];
 #pragma unroll
                 for (int i = 0; i < RI; ++i) a[i] = As[kk][ty + 16 * i];
 #pragma unroll
@@ -117,7 +110,7 @@ __global__ void __launch_bounds__(NT) k_gemm(const Task* __restrict__ tasks, int
 #pragma unroll
                 for (int i = 0; i < RI; ++i)
 #pragma unroll
-                    for (int j = 0; j < RJ; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+                    for (int j = 0; j < RJ; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
             }
             __syncthreads();
         }
@@ -130,13 +123,13 @@ __global__ void __launch_bounds__(NT) k_gemm(const Task* __restrict__ tasks, int
         for (int j = 0; j < RJ; ++j) {
             const int c = tx + 16 * j;
             if (c >= nrem) continue;
-            if (t.part) { t.part[r * TN + c] = (T)acc[i][j]; continue; }
+            if (t.part) { t.part[r * TN + c] = (double)acc[i][j]; continue; }
             const int gr = t.r0 + r, gc = t.c0 + c;
-            T* dst;
+            double* dst;
             if (t.cmap == nullptr) dst = t.C + (size_t)gr * t.ldc + gc;
             else if (t.cmap_rows) dst = t.C + t.cmap[2 * gr] + (size_t)gc * t.cmap[2 * gr + 1];
             else dst = t.C + t.cmap[2 * gc] + (size_t)gr * t.cmap[2 * gc + 1];
-            *dst = t.accumulate ? *dst + (T)acc[i][j] : (T)acc[i][j];
+            *dst = t.accumulate ? *dst + (double)acc[i][j] : (double)acc[i][j];
         }
     }
   }
@@ -601,9 +594,9 @@ int resident_ctas(const void* func, int threads, size_t smem) {
     return mine[{func, dev}] = cache[{func, dev}] = nb * sms;
 }
 
-template <int TM, int TN, class U>
+template <int TM, int TN>
 void launch_tile(const GemmTask* tasks, int ntask, const GemmOp* ops, cudaStream_t st, const int* skip) {
-    auto* f = k_gemm<TM, TN, double, GemmTask, GemmOp, U>;
+    auto* f = k_gemm<TM, TN>;
     const int grid = std::min(ntask, resident_ctas(reinterpret_cast<const void*>(f), NT, 0));
     counted();
     f<<<grid, NT, 0, st>>>(tasks, ntask, ops, skip);
@@ -619,14 +612,13 @@ void launch_splitk_reduce(const SplitRed* tasks, int ntask, cudaStream_t st, con
     if (ntask > 0) { counted(); k_splitk_reduce<<<ntask, 256, 0, st>>>(tasks, skip); }
 }
 
-void launch_gemm_tile(int tm, int tn, bool f32, const GemmTask* tasks, int ntask, const GemmOp* ops, cudaStream_t st,
+void launch_gemm_tile(int tm, int tn, const GemmTask* tasks, int ntask, const GemmOp* ops, cudaStream_t st,
                       const int* skip) {
     if (ntask <= 0) return;
-#define MPSPT_TILE(A, B)                                                          \
-    if (tm == A && tn == B) {                                                     \
-        if (f32) launch_tile<A, B, float>(tasks, ntask, ops, st, skip);           \
-        else launch_tile<A, B, double>(tasks, ntask, ops, st, skip);              \
-        return;                                                                   \
+#define MPSPT_TILE(A, B)                                    \
+    if (tm == A && tn == B) {                               \
+        launch_tile<A, B>(tasks, ntask, ops, st, skip);     \
+        return;                                             \
     }
     MPSPT_TILE(64, 64)
     MPSPT_TILE(32, 64)
@@ -634,29 +626,12 @@ void launch_gemm_tile(int tm, int tn, bool f32, const GemmTask* tasks, int ntask
     MPSPT_TILE(16, 128)
     MPSPT_TILE(32, 32)
 #undef MPSPT_TILE
-    launch_tile<64, 64, double>(tasks, 0, ops, st, skip);   // unreachable for planned tiles
 }
 
-void launch_gemm_f64in_f32(const GemmTask* tasks, int ntask, const GemmOp* ops, cudaStream_t st,
-                           const int* skip) {
-    launch_gemm_tile(64, 64, true, tasks, ntask, ops, st, skip);
-}
-void launch_gemm_f64_skinny(const GemmTask* tasks, int ntask, const GemmOp* ops, cudaStream_t st,
-                            const int* skip) {
-    launch_gemm_tile(16, 128, false, tasks, ntask, ops, st, skip);
-}
-void launch_gemm_f64in_f32_skinny(const GemmTask* tasks, int ntask, const GemmOp* ops, cudaStream_t st,
-                                  const int* skip) {
-    launch_gemm_tile(16, 128, true, tasks, ntask, ops, st, skip);
-}
 void launch_mix(const MixTask* tasks, int ntask, const MixSrc* srcs, cudaStream_t st, const int* skip) {
     if (ntask > 0) { counted(); k_mix<<<ntask, 128, 0, st>>>(tasks, srcs, skip); }
 }
 
-void launch_gemm_f64(const GemmTask* tasks, int ntask, const GemmOp* ops, cudaStream_t st,
-                     const int* skip) {
-    launch_gemm_tile(64, 64, false, tasks, ntask, ops, st, skip);
-}
 void launch_diag(const DiagTask* tasks, int ntask, const DiagTerm* terms, cudaStream_t st) {
     if (ntask > 0) { counted(); k_diag<<<ntask, 256, 0, st>>>(tasks, terms); }
 }

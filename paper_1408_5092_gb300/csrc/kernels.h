@@ -46,6 +46,23 @@ struct SplitRed {
     int accumulate, cmap_rows;
 };
 
+// One output block of the float64 grouped GEMM (kernels_dgemm.cu): an m x n
+// block C = sum of its K-list ops[op0, op1), addressed as GemmTask's.  Its
+// units are numbered u0, u0 + 1, ...: tiles row by row, `nt` to a row, the S
+// pieces of a tile's K-list together.  The K-list counts q steps of four K
+// (each entry rounded up), a piece has qs of them.  With S > 1 the pieces of
+// tile t meet at part + part_off + t * S * tile and tick + tick_off + t.
+struct GemmBlk {
+    double* C;
+    const int* cmap;
+    size_t part;
+    int tick;
+    int ldc, m, n;
+    int op0, op1;
+    int accumulate, cmap_rows;
+    int q, qs, S, nt, u0;
+};
+
 constexpr int GEMM_TM = 64;
 constexpr int GEMM_TN = 64;
 
@@ -138,24 +155,18 @@ int tc_tile_m();
 int tc_tile_n();
 void launch_gemm_tc(const GemmTask* tasks, int ntask, const GemmOp* ops, int* err, cudaStream_t st,
                     const int* skip = nullptr, bool f16 = false);
-// Float32-arithmetic variant of the float64 grouped GEMM (float64 in/out).
-void launch_gemm_f64in_f32(const GemmTask* tasks, int ntask, const GemmOp* ops, cudaStream_t st,
-                           const int* skip = nullptr);
-
-void launch_gemm_f64(const GemmTask* tasks, int ntask, const GemmOp* ops, cudaStream_t st,
-                     const int* skip = nullptr);
-// Grouped GEMM with output tile tm x tn (64x64, 32x64, 64x32, 16x128, 32x32),
-// float64 or float32 arithmetic (f32) on float64 data.  Persistent: at most
-// the resident CTAs are launched and each walks a stride of the task list.
+// Float64 grouped GEMM over the units of a block list (see GemmBlk), output
+// tile 16 x 16 or 32 x 32; unit_blk[u] is the block of unit u.  part holds the
+// partial tiles and tick one zeroed counter per split tile (left at zero).
+void launch_dgemm(int tile, const GemmBlk* blks, const unsigned* unit_blk, int nunit, const GemmOp* ops, double* part,
+                  unsigned* tick, cudaStream_t st, const int* skip = nullptr);
+// Float32 arithmetic on float64 data: grouped GEMM with output tile tm x tn
+// (64x64, 32x64, 64x32, 16x128, 32x32).  Persistent: at most the resident
+// CTAs are launched and each walks a stride of the task list.
 bool gemm_tile_supported(int tm, int tn);
 void launch_splitk_reduce(const SplitRed* tasks, int ntask, cudaStream_t st, const int* skip = nullptr);
-void launch_gemm_tile(int tm, int tn, bool f32, const GemmTask* tasks, int ntask, const GemmOp* ops, cudaStream_t st,
+void launch_gemm_tile(int tm, int tn, const GemmTask* tasks, int ntask, const GemmOp* ops, cudaStream_t st,
                       const int* skip = nullptr);
-// Skinny-tile (16 x 128) float64 variant for panels with few rows.
-void launch_gemm_f64_skinny(const GemmTask* tasks, int ntask, const GemmOp* ops, cudaStream_t st,
-                            const int* skip = nullptr);
-void launch_gemm_f64in_f32_skinny(const GemmTask* tasks, int ntask, const GemmOp* ops, cudaStream_t st,
-                                  const int* skip = nullptr);
 void launch_mix(const MixTask* tasks, int ntask, const MixSrc* srcs, cudaStream_t st,
                 const int* skip = nullptr);
 void launch_diag(const DiagTask* tasks, int ntask, const DiagTerm* terms, cudaStream_t st);

@@ -2,6 +2,7 @@
 #include "plans.h"
 
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <map>
 #include <tuple>
@@ -58,7 +59,75 @@ void GemmPlan::split(int tm_, int tn_, std::vector<GemmTask>& out, std::vector<l
     if (part_elems) *part_elems = pe;
 }
 
+// Float64 units.  A block's K-list counts steps of four K per entry, rounded
+// up; a 16 x 16 tile of a full block costs 4 DMMAs a step.  The work is cut so
+// that 1216 units (eight a SM) of equal cost would cover it, but into no
+// piece of fewer than eight steps (two per warp: 2.4 us on its
+// sub-partition, about what a unit costs to start) nor a tile into more than
+// 64 pieces.  The cut depends on the block list only, not on the tile, and so
+// do the results.
+void GemmPlan::units(int tile, std::vector<GemmBlk>& gb, std::vector<unsigned>& ub,
+                     std::vector<long long>* cm, size_t* part_elems, size_t* ticks) const {
+    const int nb = (int)blocks.size();
+    std::vector<int> q(nb), cost(nb), ord(nb);
+    double total = 0.0;
+    for (int i = 0; i < nb; ++i) {
+        const Blk& b = blocks[i];
+        long long s = 0;
+        for (int o = b.op0; o < b.op1; ++o) s += (ops[o].k + 3) / 4;
+        require(s < (1LL << 30), "gemm K-list too long");
+        q[i] = (int)s;
+        total += (double)((b.m + 7) / 8) * ((b.n + 7) / 8) * s;
+        ord[i] = i;
+    }
+    const double target = std::max(32.0, total / 1216.0);
+    std::vector<int> qs(nb);
+    for (int i = 0; i < nb; ++i) {
+        const Blk& b = blocks[i];
+        const double tc = (double)std::min(2, (b.m + 7) / 8) * std::min(2, (b.n + 7) / 8) * q[i];
+        int S = (int)std::min(64.0, std::ceil(tc / target));
+        S = std::max(1, std::min(S, q[i] / 8));
+        qs[i] = std::max(1, (q[i] + S - 1) / S);
+        cost[i] = (int)std::min(1e9, std::min(tile / 8, (b.m + 7) / 8) * (double)std::min(tile / 8, (b.n + 7) / 8) * qs[i]);
+    }
+    // costliest units first: the persistent CTAs take units in strides of the grid
+    std::stable_sort(ord.begin(), ord.end(), [&](int x, int y) { return cost[x] > cost[y]; });
+    gb.clear();
+    ub.clear();
+    if (cm) cm->clear();
+    size_t pe = 0, tk = 0;
+    for (int k = 0; k < nb; ++k) {
+        const int i = ord[k];
+        const Blk& b = blocks[i];
+        const int mt = (b.m + tile - 1) / tile, nt = (b.n + tile - 1) / tile;
+        const int S = std::max(1, (q[i] + qs[i] - 1) / qs[i]);
+        gb.push_back({b.C, nullptr, pe, (int)tk, b.ldc, b.m, b.n, b.op0, b.op1, b.accumulate, b.cmap_rows, q[i], qs[i], S,
+                      nt, (int)ub.size()});
+        if (cm) cm->push_back(b.cmap_off);
+        const size_t tiles = (size_t)mt * nt;
+        if (S > 1) {
+            pe += tiles * S * tile * tile;
+            tk += tiles;
+        }
+        require(ub.size() + tiles * S < (1ULL << 31) && tk < (1ULL << 31), "gemm unit list too long");
+        ub.insert(ub.end(), tiles * S, (unsigned)k);
+    }
+    *part_elems = pe;
+    *ticks = tk;
+}
+
 namespace {
+// 32 x 32 units when there are enough of them to keep every SM busy for two
+// rounds of its eight (fewer unit starts, half the operand traffic), the
+// narrow 16 x 16 ones below that.  Both give the same bits and nearly the same
+// time near the line (the float64 pipe bounds both); in the M = 256 sweep the
+// tuner takes 32 x 32 for a third of the launches.
+int dgemm_tile(const GemmPlan& g) {
+    size_t n = 0;
+    for (const auto& b : g.blocks) n += (size_t)((b.m + 31) / 32) * ((b.n + 31) / 32);
+    return n >= 2432 ? 32 : 16;
+}
+
 // longest K-list first: the persistent kernels hand out tasks in strides of
 // the grid, so this order balances the CTAs (each output tile has exactly
 // one task, so the order does not change any result)
@@ -96,20 +165,37 @@ void GemmPlan::upload(cudaStream_t st) {
         tm = t.first;
         tn = t.second;
     }
-    size_t pe = 0;
-    split(tm, tn, tasks, &task_cmap, &reds, &red_cmap, &pe);
-    if (pe) dpart.ensure(pe * sizeof(double) + 16, st);
-    double* pbase = dpart.as<double>();
-    for (auto& t : tasks)   // partial offsets (stored as byte offsets + 8) become pointers
-        if (t.part) t.part = pbase + ((reinterpret_cast<uintptr_t>(t.part) - 8) / sizeof(double));
-    for (auto& r : reds) r.part = pbase + ((reinterpret_cast<uintptr_t>(r.part) - 8) / sizeof(double));
-    order_tasks(tasks, &task_cmap, ops);
     if (!cmaps.empty()) mpspt::upload(dcmaps, cmaps, st);
     const int* cbase = dcmaps.as<int>();
-    for (size_t i = 0; i < tasks.size(); ++i)
-        tasks[i].cmap = task_cmap[i] >= 0 ? cbase + task_cmap[i] : nullptr;
-    for (size_t i = 0; i < reds.size(); ++i) reds[i].cmap = red_cmap[i] >= 0 ? cbase + red_cmap[i] : nullptr;
-    if (!reds.empty()) mpspt::upload(dreds, reds, st);
+    size_t pe = 0;
+    if (kind == GEMM_F64) {
+        size_t tk = 0;
+        std::vector<long long> cm;
+        tile64 = tuner && !blocks.empty() ? (tm == 32 ? 32 : 16) : dgemm_tile(*this);
+        units(tile64, gblk, unit_blk, &cm, &pe, &tk);
+        for (size_t i = 0; i < gblk.size(); ++i) gblk[i].cmap = cm[i] >= 0 ? cbase + cm[i] : nullptr;
+        if (pe) dpart.ensure(pe * sizeof(double) + 16, st);
+        if (tk) {   // the kernel leaves the counters at zero; new ones are set here
+            const size_t had = dtick.bytes();
+            dtick.ensure(tk * sizeof(unsigned), st);
+            if (dtick.bytes() != had) MPSPT_CUDA(cudaMemsetAsync(dtick.get(), 0, dtick.bytes(), st));
+        }
+        mpspt::upload(dgblk, gblk, st);
+        mpspt::upload(dunit, unit_blk, st);
+    } else {
+        split(tm, tn, tasks, &task_cmap, &reds, &red_cmap, &pe);
+        if (pe) dpart.ensure(pe * sizeof(double) + 16, st);
+        double* pbase = dpart.as<double>();
+        for (auto& t : tasks)   // partial offsets (stored as byte offsets + 8) become pointers
+            if (t.part) t.part = pbase + ((reinterpret_cast<uintptr_t>(t.part) - 8) / sizeof(double));
+        for (auto& r : reds) r.part = pbase + ((reinterpret_cast<uintptr_t>(r.part) - 8) / sizeof(double));
+        order_tasks(tasks, &task_cmap, ops);
+        for (size_t i = 0; i < tasks.size(); ++i)
+            tasks[i].cmap = task_cmap[i] >= 0 ? cbase + task_cmap[i] : nullptr;
+        for (size_t i = 0; i < reds.size(); ++i) reds[i].cmap = red_cmap[i] >= 0 ? cbase + red_cmap[i] : nullptr;
+        if (!reds.empty()) mpspt::upload(dreds, reds, st);
+        mpspt::upload(dtasks, tasks, st);
+    }
     if (checks_enabled()) {
         // per planned block (all tiles of a block share its output and its
         // K-list): the output range, or the span of its mapped addresses,
@@ -143,7 +229,6 @@ void GemmPlan::upload(cudaStream_t st) {
             }
         }
     }
-    mpspt::upload(dtasks, tasks, st);
 }
 
 void Autotuner::RawBuf::ensure(size_t bytes) {
@@ -190,11 +275,14 @@ std::pair<int, int> Autotuner::choose(const GemmPlan& g, cudaStream_t st) {
                   bucket((long long)g.blocks.size())};
     std::lock_guard<std::mutex> lk(mu);
     auto it = best.find(key);
-    if (it != best.end()) { ++reused; return it->second; }
+    // (a float64 entry of another tile, from an older file, is timed again)
+    if (it != best.end() && (g.kind != GEMM_F64 || it->second.first <= 32)) { ++reused; return it->second; }
     static const int cand_wide[][2] = {{64, 64}, {32, 64}, {64, 32}, {32, 32}};
     static const int cand_skinny[][2] = {{16, 128}, {32, 64}, {32, 32}};
-    const int (*cand)[2] = g.skinny ? cand_skinny : cand_wide;
-    const int nc = g.skinny ? 3 : 4;
+    static const int cand_f64[][2] = {{32, 32}, {16, 128}};
+    const bool f64 = g.kind == GEMM_F64;
+    const int (*cand)[2] = f64 ? cand_f64 : g.skinny ? cand_skinny : cand_wide;
+    const int nc = f64 ? 2 : g.skinny ? 3 : 4;
     if (!ev[0]) {
         MPSPT_CUDA(cudaEventCreate(&ev[0]));
         MPSPT_CUDA(cudaEventCreate(&ev[1]));
@@ -203,23 +291,51 @@ std::pair<int, int> Autotuner::choose(const GemmPlan& g, cudaStream_t st) {
     std::pair<int, int> win{cand[0][0], cand[0][1]};
     float tbest = 1e30f;
     std::vector<GemmTask> tt;
+    std::vector<GemmBlk> gb;
+    std::vector<unsigned> ub;
     for (int c = 0; c < nc; ++c) {
-        g.split(cand[c][0], cand[c][1], tt, nullptr);
-        order_tasks(tt, nullptr, g.ops);
-        for (auto& t : tt) {   // outputs go to scratch: dense m x n, no map; operands are the plan's
-            t.C = static_cast<double*>(scratch.p);
-            t.ldc = t.n;
-            t.cmap = nullptr;
-            t.cmap_rows = 0;
+        // outputs go to scratch: dense m x n, no map; operands are the plan's
+        size_t pe = 0, tk = 0;
+        if (f64) {
+            g.units(cand[c][0] == 32 ? 32 : 16, gb, ub, nullptr, &pe, &tk);
+            for (auto& b : gb) {
+                b.C = static_cast<double*>(scratch.p);
+                b.ldc = b.n;
+                b.accumulate = b.cmap_rows = 0;
+            }
+            dpart.ensure(pe * sizeof(double) + 16);
+            dtick.ensure(tk * sizeof(unsigned) + 16);
+            MPSPT_CUDA(cudaMemsetAsync(dtick.p, 0, tk * sizeof(unsigned) + 16, st));
+            dtasks.ensure(gb.size() * sizeof(GemmBlk) + 16);
+            dunits.ensure(ub.size() * sizeof(unsigned) + 16);
+            if (!ub.empty()) {
+                copy_h2d(dtasks.p, gb.data(), gb.size() * sizeof(GemmBlk), st);
+                copy_h2d(dunits.p, ub.data(), ub.size() * sizeof(unsigned), st);
+            }
+        } else {
+            g.split(cand[c][0], cand[c][1], tt, nullptr);
+            order_tasks(tt, nullptr, g.ops);
+            for (auto& t : tt) {
+                t.C = static_cast<double*>(scratch.p);
+                t.ldc = t.n;
+                t.cmap = nullptr;
+                t.cmap_rows = 0;
+            }
+            dtasks.ensure(tt.size() * sizeof(GemmTask) + 16);
+            if (!tt.empty()) copy_h2d(dtasks.p, tt.data(), tt.size() * sizeof(GemmTask), st);
         }
-        dtasks.ensure(tt.size() * sizeof(GemmTask) + 16);
-        const GemmTask* dt = static_cast<const GemmTask*>(dtasks.p);
-        if (!tt.empty()) copy_h2d(dtasks.p, tt.data(), tt.size() * sizeof(GemmTask), st);
-        const bool f32 = g.kind == GEMM_F32;
-        launch_gemm_tile(cand[c][0], cand[c][1], f32, dt, (int)tt.size(), g.dops.as<GemmOp>(), st);
+        auto run = [&] {
+            if (f64)
+                launch_dgemm(cand[c][0] == 32 ? 32 : 16, static_cast<const GemmBlk*>(dtasks.p),
+                             static_cast<const unsigned*>(dunits.p), (int)ub.size(), g.dops.as<GemmOp>(),
+                             static_cast<double*>(dpart.p), static_cast<unsigned*>(dtick.p), st);
+            else
+                launch_gemm_tile(cand[c][0], cand[c][1], static_cast<const GemmTask*>(dtasks.p), (int)tt.size(),
+                                 g.dops.as<GemmOp>(), st);
+        };
+        run();
         MPSPT_CUDA(cudaEventRecord(ev[0], st));
-        for (int r = 0; r < 3; ++r)
-            launch_gemm_tile(cand[c][0], cand[c][1], f32, dt, (int)tt.size(), g.dops.as<GemmOp>(), st);
+        for (int r = 0; r < 3; ++r) run();
         MPSPT_CUDA(cudaEventRecord(ev[1], st));
         MPSPT_CUDA(cudaEventSynchronize(ev[1]));
         float ms_ = 0.f;
@@ -254,12 +370,17 @@ void Autotuner::save(const std::string& path) {
 }
 
 void GemmPlan::run(cudaStream_t st) const {
+    if (kind == GEMM_F64) {
+        launch_dgemm(tile64, dgblk.as<GemmBlk>(), dunit.as<unsigned>(), (int)unit_blk.size(), dops.as<GemmOp>(),
+                     dpart.as<double>(), dtick.as<unsigned>(), st, skip);
+        return;
+    }
     const int nt = (int)tasks.size();
     if (nt == 0) return;
     const GemmTask* t = dtasks.as<GemmTask>();
     const GemmOp* o = dops.as<GemmOp>();
     if (is_tc(kind)) launch_gemm_tc(t, nt, o, err, st, skip, kind == GEMM_TC16);
-    else launch_gemm_tile(tm, tn, kind == GEMM_F32, t, nt, o, st, skip);
+    else launch_gemm_tile(tm, tn, t, nt, o, st, skip);
     if (!reds.empty()) launch_splitk_reduce(dreds.as<SplitRed>(), (int)reds.size(), st, skip);
 }
 
@@ -461,7 +582,7 @@ void TwoSitePlan::build(const Omega& om, const TwoT& bra, const TwoT& ket, const
             g2.op(Vp + voff[sl], W, Lpp + lp_off[sl], K, K, 1 | 2, 1.0);
             g2.block(out, 0, W, dl, 0, m0, co, 1);
         } else {
-            GemmPlan& g = (dl <= 16) ? g2s : g2;
+            GemmPlan& g = (kind == GEMM_F32 && dl <= 16) ? g2s : g2;
             const long long co = g.add_cmap(cm);
             int m0 = g.mark();
             g.op(Lpp + lp_off[sl], K, Vp + voff[sl], W, K, 0, 1.0);

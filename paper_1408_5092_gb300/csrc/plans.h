@@ -18,12 +18,14 @@ inline bool is_tc(int kind) { return kind == GEMM_TC || kind == GEMM_TC16; }
 
 struct GemmPlan;
 
-// Tile-shape autotuner of the CUDA-core grouped GEMM.  A plan's shape class
-// is (arithmetic, skinny, and log2 buckets of the median block rows, columns
-// and K-length and of the block count).  The first plan of a class times
-// every candidate tile on its own operands (outputs redirected to scratch,
-// so no result changes), keeps the fastest, and later plans of the class
-// reuse it.  The table can be read from and written to a text file.
+// Tile-shape autotuner of the float64 and float32 grouped GEMMs.  A plan's
+// shape class is (arithmetic, skinny, and log2 buckets of the median block
+// rows, columns and K-length and of the block count).  The first plan of a
+// class times every candidate tile on its own operands (outputs redirected to
+// scratch, so no result changes), keeps the fastest, and later plans of the
+// class reuse it.  The table can be read from and written to a text file; in
+// it the float64 kernel's 32 x 32 units are "32 32" and its narrow 16 x 16
+// units "16 128" (the narrow form's name since the file's first version).
 struct Autotuner {
     using Key = std::tuple<int, int, int, int, int, int>;
     std::mutex mu;
@@ -41,10 +43,11 @@ struct Autotuner {
         void ensure(size_t bytes);
         ~RawBuf();
     };
-    RawBuf scratch, dtasks;
+    RawBuf scratch, dtasks, dunits, dpart, dtick;
     cudaEvent_t ev[2] = {nullptr, nullptr};
     ~Autotuner();
-    // (tm, tn) for the plan (its blocks recorded, its ops uploaded)
+    // (tm, tn) for the plan (its blocks recorded, its ops uploaded); float64
+    // plans: (32, 32) or the narrow (16, 128)
     std::pair<int, int> choose(const GemmPlan& g, cudaStream_t st);
     void load(const std::string& path);
     void save(const std::string& path);
@@ -82,8 +85,18 @@ struct GemmPlan {
     std::vector<SplitRed> reds;
     std::vector<long long> red_cmap;
     DBuf dreds, dpart;
+    // float64: block and unit lists of k_dgemm
+    int tile64 = 32;
+    std::vector<GemmBlk> gblk;
+    std::vector<unsigned> unit_blk;
+    DBuf dgblk, dunit, dtick;
+    // block and unit lists for a tile of 16 or 32 (no map pointers yet; cm, if
+    // given: each block's map offset); partial-tile elements and split tiles
+    void units(int tile, std::vector<GemmBlk>& gb, std::vector<unsigned>& ub, std::vector<long long>* cm,
+               size_t* part_elems, size_t* ticks) const;
     void clear() {
         blocks.clear(); tasks.clear(); ops.clear(); cmaps.clear(); task_cmap.clear(); reds.clear(); red_cmap.clear();
+        gblk.clear(); unit_blk.clear();
         flops = 0.0;
     }
     // K-chunks of a block: blocks with a small output and a long K-list are
@@ -134,7 +147,7 @@ struct Omega {
 //   g2:  out(sl, :) = Lpack(sl) V_stack(sl)  one long-K GEMM per bra left
 //        sector, scattered into the two-site layout by a column map
 struct TwoSitePlan {
-    GemmPlan g1, g2, g2s;            // g2: wide rows, g2s: few rows (skinny tiles)
+    GemmPlan g1, g2, g2s;            // g2s: the float32 blocks of few rows (skinny tiles)
     std::vector<MixTask> mtasks;
     std::vector<MixSrc> msrc;
     DBuf dmt, dms;
@@ -210,7 +223,8 @@ struct EnvPlan {
     // lists, mix tasks and sources)
     size_t plan_bytes() const {
         return mt.size() * sizeof(MixTask) + ms.size() * sizeof(MixSrc) +
-               (g1.tasks.size() + g2.tasks.size()) * sizeof(GemmTask) +
+               (g1.gblk.size() + g2.gblk.size()) * sizeof(GemmBlk) +
+               (g1.unit_blk.size() + g2.unit_blk.size()) * sizeof(unsigned) +
                (g1.ops.size() + g2.ops.size()) * sizeof(GemmOp);
     }
 
