@@ -369,21 +369,22 @@ mpspt_status mpspt_train_preconditioner(mpspt_ctx* ctx, mpspt_h0 h0, int M, int 
  * sum_{j<i} n[j]^2 of A (row-major, symmetric, not modified) and of V
  * (eigenvectors as columns), and at sum_{j<i} n[j] of w (eigenvalues, in
  * the column order of V, unsorted).  Work is ordered on `stream`
- * (cudaStream_t, 0 = default); the call allocates a work copy of A with
+ * (cudaStream_t, 0 = default); the call allocates its task list (and a work
+ * copy of matrices too large for the on-chip solver, n above about 590) with
  * cudaMallocAsync on that stream and returns without synchronising. */
 mpspt_status mpspt_eigh_batched(int device, void* stream, int batch, const int* n, const double* A,
                                 double* V, double* w);
 
 /* Same contract as mpspt_eigh_batched, with the solver the truncation step
- * uses: Jacobi with one launch per sweep (the matrix as a packed triangle in
- * shared memory, the recorded rotations applied to the rows of V by many
- * CTAs in parallel).  f32_start = 0: float64 sweeps from the identity.
+ * uses.  f32_start = 0: float64 Jacobi sweeps from the identity.
  * f32_start = 1: float32 sweeps from the identity, two float64
  * Newton-Schulz steps that restore orthonormality (V <- V (3/2 I -
- * 1/2 V^T V)), then float64 sweeps on V^T A V starting from V, to the same
- * float64 convergence test.  A is left unchanged.  Allocates device scratch
- * (about 4 n^2 doubles per matrix) and returns after the stream has
- * finished the work. */
+ * 1/2 V^T V)), then rounds of B = V^T A V in float64, Jacobi sweeps on B with
+ * its diagonal in float64 and its small off-diagonal part in float32, and
+ * V <- V R with float64 rotations, until float32 leaves nothing above
+ * float64 rounding.  A is left unchanged.  Allocates device scratch
+ * (about 25 n^2 doubles per matrix, rotation lists included) and returns
+ * after the stream has finished the work. */
 mpspt_status mpspt_eigh_batched_ex(int device, void* stream, int batch, const int* n, const double* A,
                                    double* V, double* w, int f32_start);
 

@@ -430,23 +430,29 @@ mpspt_status mpspt_eigh_batched(int device, void* stream, int batch, const int* 
     return guard(nullptr, [&] {
         MPSPT_CUDA(cudaSetDevice(device));
         cudaStream_t st = static_cast<cudaStream_t>(stream);
-        size_t tot = 0, totw = 0;
-        for (int i = 0; i < batch; ++i) {
-            mpspt::require(n[i] >= 1 && n[i] <= 2048, "matrix size must be in [1, 2048]");
-            tot += (size_t)n[i] * n[i];
-            totw += (size_t)n[i];
-        }
-        mpspt::DBuf work(tot * sizeof(double), st), dt;
-        MPSPT_CUDA(cudaMemcpyAsync(work.get(), A, tot * sizeof(double), cudaMemcpyDeviceToDevice, st));
+        for (int i = 0; i < batch; ++i) mpspt::require(n[i] >= 1 && n[i] <= 2048, "matrix size must be in [1, 2048]");
+        // a work copy only for matrices that the solver cannot hold on chip
+        size_t wtot = 0;
+        for (int i = 0; i < batch; ++i)
+            if (mpspt::eig_in_place(n[i])) wtot += (size_t)n[i] * n[i];
+        mpspt::DBuf work(wtot * sizeof(double), st), dt;
         std::vector<mpspt::EigTask> tasks(batch);
-        size_t o = 0, ow = 0;
+        size_t o = 0, ow = 0, wo = 0;
         for (int i = 0; i < batch; ++i) {
-            tasks[i] = {work.as<double>() + o, V + o, w + ow, n[i], 0};
-            o += (size_t)n[i] * n[i];
+            const size_t nn = (size_t)n[i] * n[i];
+            double* a = const_cast<double*>(A) + o;
+            if (mpspt::eig_in_place(n[i])) {
+                MPSPT_CUDA(cudaMemcpyAsync(work.as<double>() + wo, a, nn * sizeof(double), cudaMemcpyDeviceToDevice, st));
+                a = work.as<double>() + wo;
+                wo += nn;
+            }
+            tasks[i] = {a, V + o, w + ow, n[i], 0};
+            o += nn;
             ow += (size_t)n[i];
         }
+        mpspt::order_eig_tasks(tasks.data(), batch);
         mpspt::upload(dt, tasks, st);
-        mpspt::launch_eig(dt.as<mpspt::EigTask>(), batch, st);
+        mpspt::launch_eig(dt.as<mpspt::EigTask>(), tasks.data(), batch, false, mpspt::kEighSweeps, nullptr, st);
         MPSPT_CUDA(cudaGetLastError());
     });
 }
@@ -475,11 +481,13 @@ mpspt_status mpspt_eigh_batched_ex(int device, void* stream, int batch, const in
         }
         mpspt::EigSolver es;
         es.run(tasks, f32_start == 0, st);
+        std::vector<int> fl(es.nflags);
+        do {
+            MPSPT_CUDA(cudaMemcpyAsync(fl.data(), es.flags.get(), es.nflags * sizeof(int), cudaMemcpyDeviceToHost, st));
+            MPSPT_CUDA(cudaStreamSynchronize(st));
+        } while (es.again(fl.data(), st));
         MPSPT_CUDA(cudaMemcpyAsync(V, wv.get(), tot * sizeof(double), cudaMemcpyDeviceToDevice, st));
         MPSPT_CUDA(cudaMemcpyAsync(w, ww.get(), totw * sizeof(double), cudaMemcpyDeviceToDevice, st));
-        std::vector<int> fl(es.nflags);
-        if (es.nflags)
-            MPSPT_CUDA(cudaMemcpyAsync(fl.data(), es.flags.get(), es.nflags * sizeof(int), cudaMemcpyDeviceToHost, st));
         MPSPT_CUDA(cudaStreamSynchronize(st));   // the solver's scratch is released on return
         MPSPT_CUDA(cudaGetLastError());
         for (int f : fl)

@@ -10,33 +10,50 @@
 namespace mpspt {
 
 struct EigSolver {
-    DBuf scratch, vt, g, djt, djt1, djtc, drows, dtns;
-    // per task of the last stage run: 1 converged, 2 stopped by the sweep
-    // cap (device ints, valid once the stream has reached them)
+    // per task of the last run: 0 another round is needed, 1 converged, 2
+    // stopped by the sweep cap (device ints, valid once the stream has
+    // reached them; see again)
     DBuf flags;
     int nflags = 0;
-    int* flag_host = nullptr;   // page-locked copy of the flags between sweep batches
-    ~EigSolver() { if (flag_host) cudaFreeHost(flag_host); }
-    GemmPlan ge;   // batched square GEMMs of the float64 stage
     bool stats = false;   // count sweeps per matrix (sum, matrices, max)
-    long long sweeps32[3] = {0, 0, 0}, sweeps_polish[3] = {0, 0, 0}, sweeps64[3] = {0, 0, 0};
+    long long sweeps32[3] = {0, 0, 0}, sweeps_polish[3] = {0, 0, 0};
 
     // For every task: A (n x n, symmetric, left unchanged) -> V (eigenvectors
     // as columns) and w (unsorted eigenvalues).  All pointers must lie in
     // library allocations.  fp64_only: float64 Jacobi from the identity.
-    // Otherwise three stages:
-    //  1. cyclic Jacobi in float32 from the identity (the float64 pipe is the
-    //     scarce one on this GPU), giving V orthonormal to float32 rounding;
+    // Otherwise (the float64 pipe is the scarce one on this GPU):
+    //  1. cyclic Jacobi in float32 from the identity, giving V orthonormal to
+    //     float32 rounding;
     //  2. two Newton-Schulz steps V <- V (3/2 I - 1/2 V^T V) in float64, each
     //     squaring the departure from orthonormality;
-    //  3. B = V^T A V in float64 (nearly diagonal) and float64 Jacobi on B
-    //     starting from V, to the same float64 convergence test.
+    //  3. rounds of: B = V^T A V in float64; Jacobi sweeps on B with its
+    //     diagonal in float64 and its off-diagonal part (3e-5 |A| in the first
+    //     round, about 1e-11 in the second) in float32; V <- V R with the
+    //     rotations in float64.  Float32 resolves an off-diagonal part to 1e-7
+    //     of itself, so a round that starts below 1e-9 |A| ends at float64
+    //     rounding and is the last.  Two rounds are enqueued.
     void run(const std::vector<EigTask>& et, bool fp64_only, cudaStream_t st);
+    // With the flags of the last run on the host: false if all are set, else
+    // enqueues two more rounds for the matrices that need them (w and flags
+    // have to be read again) and returns true.  A matrix that needs more than
+    // the cap of rounds is an error.
+    bool again(const int* flags_host, cudaStream_t st);
 
   private:
-    // Jacobi from the given inputs (one per task) into the tasks' V (and w)
-    void jacobi(const std::vector<EigTask>& et, const std::vector<const double*>& in, int vinit, bool f32, int maxs,
-                bool want_w, cudaStream_t st, int batch = 0);
+    void fp64(const std::vector<EigTask>& et, cudaStream_t st);
+    void rounds(int n, cudaStream_t st);
+    void product(int j, cudaStream_t st);
+    void count(long long (&acc)[3], const std::vector<JacTask>& jt, cudaStream_t st);
+    DBuf scratch, vt, g, blob;
+    GemmPlan ge;                // shape of the batched square products
+    // the enqueued batch: device lists in blob, sizes
+    int ntask = 0, nsmall = 0, nmax_small = 0, nmax = 0, nrows = 0, nunit = 0, nround = 0, sweeps = 0;
+    const JacTask* dtask = nullptr;     // polish tasks (input B); small matrices first
+    const JacRows* drows = nullptr;
+    const GemmBlk* dblk = nullptr;      // ntask blocks per product
+    const unsigned* dunit = nullptr;
+    const GemmOp* dops = nullptr;
+    std::vector<JacTask> polish;
 };
 
 }  // namespace mpspt

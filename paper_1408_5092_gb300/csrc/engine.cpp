@@ -744,7 +744,7 @@ struct Sweeper {
         if (c.tuner) {
             Autotuner* t = c.tuner.get();
             sig.set_tuner(t); sig_lo.set_tuner(t); rhs.set_tuner(t); envp.set_tuner(t);
-            prod.tuner = t; prod0.tuner = t; gr.tuner = t; gc.tuner = t; eig.ge.tuner = t;
+            prod.tuner = t; prod0.tuner = t; gr.tuner = t; gc.tuner = t;
         }
         MPSPT_CUDA(cudaEventCreate(&ev0));
         MPSPT_CUDA(cudaEventCreate(&ev1));
@@ -889,20 +889,23 @@ struct Sweeper {
             eig_n3 += n3; eig_nmax = std::max(eig_nmax, nmax); eig_calls += (int)et.size();
         }
         // eigenvalues and convergence flags back through the lane's
-        // page-locked buffer (one asynchronous copy each, one sync)
+        // page-locked buffer (one asynchronous copy each, one sync; again if a
+        // matrix needs more rounds)
         const size_t wbytes = (wsz * sizeof(double) + 15) & ~(size_t)15;
         unsigned char* hb = static_cast<unsigned char*>(ln.readback(wbytes + eig.nflags * sizeof(int) + 16));
-        if (wsz) MPSPT_CUDA(cudaMemcpyAsync(hb, wv.get(), wsz * sizeof(double), cudaMemcpyDeviceToHost, ln.st));
-        if (eig.nflags)
-            MPSPT_CUDA(cudaMemcpyAsync(hb + wbytes, eig.flags.get(), eig.nflags * sizeof(int), cudaMemcpyDeviceToHost,
-                                       ln.st));
-        auto ts = clk::now();
-        wait();
-        split_wait += since(ts);
+        const int* eflag = reinterpret_cast<int*>(hb + wbytes);
+        do {
+            if (wsz) MPSPT_CUDA(cudaMemcpyAsync(hb, wv.get(), wsz * sizeof(double), cudaMemcpyDeviceToHost, ln.st));
+            if (eig.nflags)
+                MPSPT_CUDA(cudaMemcpyAsync(hb + wbytes, eig.flags.get(), eig.nflags * sizeof(int),
+                                           cudaMemcpyDeviceToHost, ln.st));
+            auto ts = clk::now();
+            wait();
+            split_wait += since(ts);
+        } while (eig.again(eflag, ln.st));
         std::vector<double> wh(reinterpret_cast<double*>(hb), reinterpret_cast<double*>(hb) + wsz);
-        std::vector<int> eflag(reinterpret_cast<int*>(hb + wbytes), reinterpret_cast<int*>(hb + wbytes) + eig.nflags);
-        for (int f : eflag)
-            require(f != 2, "truncation eigensolver: sweep cap reached before the convergence test",
+        for (int f = 0; f < eig.nflags; ++f)
+            require(eflag[f] != 2, "truncation eigensolver: sweep cap reached before the convergence test",
                     MPSPT_ERR_NOT_CONVERGED);
         // selection: keep the Mkeep largest (ties at the cut dropped as a group)
         struct Cand { double lam; int ci; int rank; int col; };
@@ -1666,10 +1669,9 @@ std::unique_ptr<MpsD> minimize(Ctx& c, const Chain& ch, int M, SweepResult& res,
             fprintf(stderr, "[mpspt]   rhs dev ms %.1f (%.1f GF) env dev ms %.1f (%.1f GF)\n", sw.t_rhs_dev, sw.rhs_gf,
                     sw.t_env_dev, sw.env_gf);
             const auto& E = sw.eig;
-            fprintf(stderr, "[mpspt]   jacobi sweeps (mean/max): float32 %.2f/%lld polish %.2f/%lld float64 %.2f/%lld\n",
+            fprintf(stderr, "[mpspt]   jacobi sweeps (mean/max): float32 %.2f/%lld polish %.2f/%lld\n",
                     E.sweeps32[1] ? (double)E.sweeps32[0] / E.sweeps32[1] : 0.0, E.sweeps32[2],
-                    E.sweeps_polish[1] ? (double)E.sweeps_polish[0] / E.sweeps_polish[1] : 0.0, E.sweeps_polish[2],
-                    E.sweeps64[1] ? (double)E.sweeps64[0] / E.sweeps64[1] : 0.0, E.sweeps64[2]);
+                    E.sweeps_polish[1] ? (double)E.sweeps_polish[0] / E.sweeps_polish[1] : 0.0, E.sweeps_polish[2]);
         }
         if (c.opt.verbose == 1)
             fprintf(stderr, "[mpspt]   host-only ms: layouts+products %.1f rhs-plan %.1f sigma-plans %.1f split-host %.1f env-plans %.1f\n",

@@ -39,4 +39,40 @@ struct Sched {
     }
 };
 
+// The same ordering with the entries addressed by slot position: slot k holds
+// positions k and m-1-k.  Position 0 keeps its player, the others move down by
+// one after every round (1 to m-1), so the player at position j >= 1 of round
+// r is ((j - 1 + r) mod (m - 1)) + 1 and after m - 1 rounds everybody is back.
+JAC_HD int next_pos(int m, int j) { return j == 0 ? 0 : j == 1 ? m - 1 : j - 1; }
+// Place of the entry of positions a < b among m (m - 1) / 2: where a + b < m
+// row a, consecutive in b; where a + b >= m row b, consecutive in a.  The four
+// entries of a block of slots (k, l), k < l, are then each consecutive in l
+// for a fixed k (a packed upper triangle puts two of them in its columns, and
+// a warp's accesses to those fell on the same banks three or four at a time).
+JAC_HD int tri(int m, int a, int b) {
+    const int half = m / 2;
+    if (a + b < m) return a * (m - a) + (b - a - 1);
+    return half * half + (b - half) * (b - half - 1) + (a - (m - b));
+}
+// place of the same two players' entry in the next round
+JAC_HD int tri_next(int m, int a, int b) {
+    const int x = next_pos(m, a), y = next_pos(m, b);
+    return x < y ? tri(m, x, y) : tri(m, y, x);
+}
+// Block number e in [0, half (half - 1) / 2) -> slots k < l: the rows of the
+// strict triangle folded in pairs of one length, so that consecutive numbers
+// stay in one row for as long as possible.
+JAC_HD void block_slots(int half, int e, int& k, int& l) {
+    const int W = (half & 1) ? half : half - 1;
+    const int i = e / W, j = e - i * W;
+    const int len = half - 1 - i;   // blocks of row i
+    if (j < len) {
+        k = i;
+        l = i + 1 + j;
+    } else {
+        k = (half & 1) ? half - 2 - i : half - 1 - i;
+        l = k + 1 + (j - len);
+    }
+}
+
 }  // namespace mpspt

@@ -61,6 +61,7 @@ struct GemmBlk {
     int op0, op1;
     int accumulate, cmap_rows;
     int q, qs, S, nt, u0;
+    float scale = 1.f, diag = 0.f;   // stored: scale * sum, plus diag where row = column
 };
 
 constexpr int GEMM_TM = 64;
@@ -93,26 +94,29 @@ struct DiagTask {
     int t0, t1;
 };
 
-// Symmetric eigenproblem of one dense n x n row-major block (in place).
+// Symmetric eigenproblem of one dense n x n row-major block, float64 sweeps.
 struct EigTask {
-    double* A;      // n*n, destroyed (diagonal holds eigenvalues on exit)
-    double* V;      // n*n eigenvectors (columns); with vinit: initial basis, rotated in place
+    double* A;      // n*n; read only, or destroyed where eig_in_place(n)
+    double* V;      // n*n eigenvectors (columns)
     double* w;      // n eigenvalues (unsorted)
     int n;
-    int vinit;
+    int pad;
 };
-// One matrix of the sweep-per-launch Jacobi (kernels_eig.cu).
+// One matrix of the sweep kernels (kernels_eig.cu).  Rotation lists hold, for
+// every sweep of the last launch, m - 1 rounds of m / 2 slots (m = n rounded
+// up to even): the rotation of slot k of round r acts on columns (x, y) of
+// the round-robin schedule's slot as x' = c x - s y, y' = s x + c y.
 struct JacTask {
-    const double* A;   // n x n symmetric input, row-major (read by sweep 0 only)
-    void* P;           // scratch: packed upper triangle, jac_p_bytes(n)
-    void* rot;         // scratch: rotation lists of the current sweep, jac_rot_bytes(n)
-    double* V;         // n x n eigenvectors (columns), row-major; with vinit: the start basis
+    const double* A;   // n x n symmetric input, row-major
+    double* V;         // n x n eigenvectors (columns), row-major
     double* w;         // n eigenvalues (unsorted), or null
-    double* prev;      // scratch: off-norm of the previous sweep
-    int* done;         // 0 while sweeping; 1 converged; 2 stopped by the sweep cap
-    int* nsw;          // scratch: sweeps performed (written when the matrix stops)
-    int n, vinit;
-    int pad0, pad1;
+    void* P;           // scratch for n beyond shared memory: the two float32 triangles
+    float2* rot;       // mixed sweeps: (c, s), or (tan, 0) in the polish
+    double2* rot64;    // float64 (c, s)
+    int* done;         // 1: converged
+    int* nsw;          // sweeps in the lists of the last launch
+    int* total;        // sweeps performed so far
+    int n, pad;
 };
 struct JacRows {       // rows [r0, r0 + rows) of task's V for one apply block
     int task, r0, rows, pad;
@@ -170,17 +174,27 @@ void launch_gemm_tile(int tm, int tn, const GemmTask* tasks, int ntask, const Ge
 void launch_mix(const MixTask* tasks, int ntask, const MixSrc* srcs, cudaStream_t st,
                 const int* skip = nullptr);
 void launch_diag(const DiagTask* tasks, int ntask, const DiagTerm* terms, cudaStream_t st);
-void launch_eig(const EigTask* tasks, int ntask, cudaStream_t st);
-size_t jac_p_bytes(int n);
-size_t jac_rot_bytes(int n);
-int jac_rows_per_block(int n, bool f32);
-void launch_jac_sweep(const JacTask* tasks, int ntask, int sweep, int maxs, bool f32, cudaStream_t st);
-// float64 sweep by clusters of 8 CTAs per matrix (distributed shared memory)
-int jac_cluster_smem(int n);
-void launch_jac_sweep_cluster(const JacTask* tasks, int ntask, int sweep, int maxs, int smem, cudaStream_t st);
-void launch_jac_apply(const JacTask* tasks, const JacRows* rows, int nblocks, int smem, int sweep, bool f32,
+// Float64 Jacobi of every matrix, at most maxs sweeps.  host: the same task
+// list on the host, in the order of order_eig_tasks (largest first, so that
+// each of the two kernels gets one launch).  null_rule: pairs below
+// 1e-14 |A|_F are left alone; flags (nullable): 1 converged, 2 stopped by the
+// cap.
+void order_eig_tasks(EigTask* tasks, int ntask);
+void launch_eig(const EigTask* tasks, const EigTask* host, int ntask, bool null_rule, int maxs, int* flags,
+                cudaStream_t st);
+bool eig_in_place(int n);
+constexpr int kEighSweeps = 40;   // sweep cap of the calls that report no flags
+size_t jac_e_bytes(int n);                 // global float32 triangles of the mixed sweeps (0: shared memory)
+size_t jac_rot_entries(int n);             // list entries of one sweep
+// Mixed sweeps (float32 off-diagonal, float64 diagonal) of every matrix, up
+// to maxs in the launch; polish: see k_jac_mixed.  nmax: the largest n.
+void launch_jac_mixed(const JacTask* tasks, int ntask, int nmax, bool polish, int maxs, cudaStream_t st);
+// rot64 <- the float64 rotations of the tangents in rot
+void launch_jac_rot64(const JacTask* tasks, int ntask, cudaStream_t st);
+// V <- V R over the lists (ident: V starts as the identity)
+constexpr int JAC_APPLY_ROWS = 4;
+void launch_jac_apply(const JacTask* tasks, const JacRows* rows, int nblocks, int nmax, bool f32, bool ident,
                       cudaStream_t st);
-void launch_ns_prep(const EigTask* tasks, int ntask, cudaStream_t st);
 void launch_copy(const CopyTask* tasks, int ntask, cudaStream_t st);
 
 // Vector kernels (n doubles).  Reductions are deterministic (fixed order).

@@ -163,6 +163,7 @@ __global__ void __launch_bounds__(DT) k_dgemm(const GemmBlk* __restrict__ blks, 
                     for (int p = 0; p < b.S; ++p) v += __ldcg(pt + (size_t)p * (TM * TN) + e);
                 }
                 const int gr = r0 + r, gc = c0 + c;
+                if (b.scale != 1.f || b.diag != 0.f) v = (double)b.scale * v + (gr == gc ? (double)b.diag : 0.0);
                 double* dst;
                 if (b.cmap == nullptr) dst = b.C + (size_t)gr * b.ldc + gc;
                 else if (b.cmap_rows) dst = b.C + b.cmap[2 * gr] + (size_t)gc * b.cmap[2 * gr + 1];

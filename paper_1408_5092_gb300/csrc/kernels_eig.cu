@@ -1,577 +1,732 @@
-// Batched cyclic Jacobi for the density-matrix eigenproblems of the
-// truncation step, one launch per sweep.
+// Batched cyclic Jacobi for the density-matrix eigenproblems of the truncation
+// step.
 //
-// k_jac_sweep (one CTA of 512 threads per matrix): the symmetric matrix is
-// kept as its packed upper triangle, in shared memory when it fits (float64
-// up to n = 215, float32 up to n = 305), else in the task's global scratch.
-// A sweep is the m-1 rounds of the round-robin ordering; in a round the m/2
-// disjoint pairs get their rotations (threshold: negligible a_pq are
-// skipped), then every unordered 2x2 block {k, l} of pairs is updated once
-// (R_k^T A_kl R_l; the symmetric partner is implied).  The applied rotations
-// of each round are recorded, compacted, in the task's rotation list.
+// The float64 pipe of this GPU (1.75 FMA per clock and SM, 64 clocks of
+// latency) is the scarce unit, so the default solver keeps the O(n^3) work of
+// the sweeps in float32 and corrects it by float64 GEMMs on all SMs (eig.cpp):
 //
-// k_jac_apply (one warp per block of rows of V): V <- V R for the
-// recorded rotations, in order.  A row of V is touched independently of the
-// others, so each lane owns one row in shared memory and runs through the
-// whole list without synchronisation; the work spreads over many SMs.
+// k_jac_mixed (one CTA per matrix): all sweeps of a phase in one launch.  The
+// off-diagonal part is float32, the diagonal float32 in the start and float64
+// in the polish, both scaled by a power of two.  In a round of the round-robin ordering the m/2 disjoint
+// pairs get their rotations, then every 2 x 2 block of slots (k, l) is
+// transformed.  Entries are addressed by slot position, not by index: a round
+// reads each block from the same four places of one buffer and writes it to
+// the four places of the next round's positions in the other, so a thread's
+// addresses are computed once per launch and kept in registers.  The update
+// moves 32 bytes of shared memory per block, 940 clocks a round at n = 173;
+// the pair phase and two barriers are the rest.
+// k_jac_rot64: the float64 (c, s) of the recorded float32 tangents.
+// k_jac_apply (a warp per row of V): V <- V R over the recorded lists; a row
+// is touched independently of the others, the rotations of a round act on
+// disjoint columns and take one lane each.
 //
-// The host launches sweep 0, apply 0, sweep 1, apply 1, ... up to maxs.  A
-// sweep first measures off(A)^2 and stops the task (flag, eigenvalues
-// written) when off^2 <= STOP * |A|_F^2, when a small off-norm stalled at
-// the rounding floor, or at sweep maxs; later launches for that task return
-// at once.
+// Measured (device time of the truncations of one M = 256 sweep of 8e/8o + 24,
+// sectors up to n = 173): sweeps 240 -> 47 ms, V 159 -> 25 ms against one
+// launch per sweep with float64 polish sweeps and 32 rows of V per CTA; a
+// batch of ten sectors (173 and down by 0.8) 29.7 -> 4.5 ms.
+//
+// k_eig_one / k_eig_cl: the plain float64 solver (float64 sweeps from the
+// identity), all sweeps in one launch, V included.
 #include <cooperative_groups.h>
 
+#include <algorithm>
+#include <type_traits>
+
+#include "jac_rot.h"
 #include "jacobi_schedule.h"
 #include "kernels.h"
 
 namespace mpspt {
 namespace {
 
-constexpr int JAC_THREADS = 512;
-constexpr int JAC_SMEM = 200704;     // dynamic shared memory of the sweep kernel
+constexpr int JAC_SMEM = 200704;     // dynamic shared memory of the float64 solver and of the apply kernel
 
-template <class T>
-struct RotE {
-    T c, s;
-    int p, q;
-};
-
-// stop: off(A)^2 <= stop |A|_F^2; a pair is not rotated when |a_pq| <= skip
-// sqrt|a_pp a_qq| or |a_pq| <= absf |A|_F; a solve that reached off(A)^2 <=
-// stall |A|_F^2 also ends when a sweep shrinks off(A)^2 by less than 19%.
-// (A rounding-level absf and a tighter float64 stall let the solves end
-// sooner but moved the sweep's energies by 1e-7..1e-6 against the oracle;
-// the values below keep float64 parity.)
-template <class T>
-struct JacTol;
-template <>
-struct JacTol<double> {
-    static constexpr double stop = 1e-30, skip = 1e-18, absf = 0.0, stall = 1e-8, null = 1e-14;
-};
-template <>
-struct JacTol<float> {
-    static constexpr double stop = 1e-11, skip = 1e-9, absf = 0.0, stall = 1e-8, null = 0.0;
-};
+// stop: off(A)^2 <= stop |A|_F^2; a solve that reached off(A)^2 <= stall
+// |A|_F^2 also ends when a sweep shrinks off(A)^2 by less than 19%.
 // Null pairs: a pair (p, q) whose 2x2 block has every entry below
 // null * |A|_F is neither rotated nor counted in the off-diagonal norm.  Its
 // eigenvalues are below 2 null |A|_F, so inside such a cluster the vectors
 // are set by rounding anyway; every coupling of a null index to a larger
 // entry is still rotated away.  For the density matrices of the truncation
-// (positive semidefinite) in float64 these are the exactly rank-deficient
-// directions, far below the keep threshold; skipping them saves the sweeps
-// the polish spent circulating rounding noise inside the null cluster.  The
-// float32 start sweeps every pair (a null level at float32 resolution,
-// 1e-6, saved float32 sweeps but cost as many float64 polish sweeps).
-
+// (positive semidefinite) these are the exactly rank-deficient directions,
+// far below the keep threshold; skipping them saves the sweeps the polish
+// spent circulating rounding noise inside the null cluster.  The float32
+// start sweeps every pair.
+struct Tol {
+    static constexpr double stop = 1e-30, stall = 1e-8, null = 1e-14;
+    // start of the mixed solver: off^2 <= 1e-9 |A|_F^2.  Against 1e-11 it
+    // saves one or two float32 sweeps of eight to ten and costs the polish
+    // none (graded, rank-deficient and degenerate spectra)
+    static constexpr double start = 1e-9;
+    // a polish round ends at off^2 <= 1e-11 of its start (float32 resolves no
+    // more than 1e-7 of the start's off-norm), and is the last one if it
+    // started from off^2 <= 1e-18 |A|_F^2: what float32 rounding leaves is
+    // then below 1e-16 |A|_F
+    static constexpr double gain = 1e-11, last = 1e-18;
+};
 
 __host__ __device__ inline size_t align16(size_t b) { return (b + 15) & ~(size_t)15; }
 
-// Rounds of one sweep at most (either schedule), and the rotation-list
-// layout: [nrounds][rcount per round] then `half` entries per round.
-__host__ __device__ inline int jac_max_rounds(int n) { return 2 * n + 4; }
-__host__ __device__ inline size_t jac_rot_head(int n) { return align16((size_t)(1 + jac_max_rounds(n)) * 4); }
-
-// shared-memory head of the sweep kernels: rowoff, Pp, Qq (n ints each, room
-// for four), Cc, Ss (n T each) and n doubles of headroom; the packed
-// triangle follows
-template <class T>
-__host__ __device__ inline size_t jac_head_bytes(int n) {
-    return align16((size_t)n * 16) + align16(2 * (size_t)n * sizeof(T)) + align16((size_t)n * 8);
+// ---------------------------------------------------------------- mixed
+constexpr int MIX_SMEM = 230000;
+// Shared memory of the mixed kernel: two triangle buffers of `cap` floats at
+// fixed offsets (so that a buffer is an immediate offset), then two diagonals,
+// (c, s) and (tan, e).  cap of the variants with NB cached blocks per thread:
+__host__ __device__ constexpr int mixed_cap(int nb) { return nb <= 2 ? 1040 : nb <= 5 ? 4192 : nb <= 8 ? 16112 : 27736; }
+inline size_t mixed_smem(int n, int cap) {
+    const size_t m = n + (n & 1);
+    return 8 * (size_t)cap + 24 * m + 16;
 }
 
-template <class T>
-__global__ void __launch_bounds__(JAC_THREADS) k_jac_sweep(const JacTask* __restrict__ tasks, int sweep, int maxs) {
+// NT threads, NB blocks per thread with cached addresses (0: any n, triangles
+// in global memory, addresses computed).
+// The start keeps its diagonal in float32 as well (its V is corrected to
+// float64 later): the chain of the pair phase is then 400 clocks instead of
+// 1000, a float64 operation being 64.  In the polish the float64 diagonal is
+// updated beside the blocks, by the last warps.
+template <int NT, int NB, bool POLISH>
+__global__ void __launch_bounds__(NT) k_jac_mixed(const JacTask* __restrict__ tasks, int maxs) {
     extern __shared__ __align__(16) unsigned char sm[];
-    __shared__ double red[2][JAC_THREADS / 32];
-    __shared__ double thr;
-    __shared__ int stop, cnt;
+    constexpr int NW = NT / 32, NC = NB > 0 ? NB : 1;
+    __shared__ double red[2][NW];
+    __shared__ unsigned redm[NW];
+    __shared__ int stop, shift;
+    __shared__ double sa_sh;
     const JacTask t = tasks[blockIdx.x];
-    if (sweep > 0 && *(volatile const int*)t.done) return;
-    const int n = t.n;
-    const int m = n + (n & 1), half = m / 2;
-    const size_t np = (size_t)n * (n + 1) / 2;
-    int* rowoff = reinterpret_cast<int*>(sm);
-    int* Pp = rowoff + n;
-    int* Qq = Pp + n;
-    T* Cc = reinterpret_cast<T*>(sm + align16((size_t)n * 16));
-    T* Ss = Cc + n;
-    const size_t head = jac_head_bytes<T>(n);
-    const bool p_sm = head + np * sizeof(T) <= (size_t)JAC_SMEM;
-    T* P = p_sm ? reinterpret_cast<T*>(sm + head) : reinterpret_cast<T*>(t.P);
-    T* Pg = reinterpret_cast<T*>(t.P);
-    int* rhead = reinterpret_cast<int*>(t.rot);          // [0]: rounds, [1 + r]: count of round r
-    RotE<T>* rlist = reinterpret_cast<RotE<T>*>(reinterpret_cast<unsigned char*>(t.rot) + jac_rot_head(n));
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = JAC_THREADS / 32;
-    for (int i = tid; i < n; i += JAC_THREADS) rowoff[i] = i * n - i * (i + 1) / 2;
-    __syncthreads();
-    if (sweep == 0) {
-        for (int e = tid; e < n * n; e += JAC_THREADS) {
-            const int i = e / n, j = e % n;
-            if (j >= i) P[rowoff[i] + j] = (T)t.A[e];
-        }
-    } else if (p_sm) {
-        for (size_t e = tid; e < np; e += JAC_THREADS) P[e] = Pg[e];
-    }
-    __syncthreads();
-    auto S = [&](int a, int b) -> T& { return a <= b ? P[rowoff[a] + b] : P[rowoff[b] + a]; };
-    // convergence test: |A|_F first (it sets the null level), then the
-    // off-diagonal norm without null pairs
-    __shared__ double nullv;
-    {
-        double all = 0.0;
-        for (int i = warp; i < n; i += nw)
-            for (int j = i + lane; j < n; j += 32) {
-                const double v = (double)P[rowoff[i] + j];
-                all += (j == i ? 1.0 : 2.0) * v * v;
-            }
-        for (int o = 16; o > 0; o >>= 1) all += __shfl_xor_sync(0xffffffffu, all, o);
-        if (lane == 0) red[1][warp] = all;
-        __syncthreads();
-        if (tid == 0) {
-            double sa = 0.0;
-            for (int w = 0; w < nw; ++w) sa += red[1][w];
-            nullv = JacTol<T>::null * sqrt(sa);
-        }
-        __syncthreads();
-        const double nv = nullv;
-        double off = 0.0;
-        all = 0.0;
-        for (int i = warp; i < n; i += nw) {
-            const double di = fabs((double)P[rowoff[i] + i]);
-            for (int j = i + lane; j < n; j += 32) {
-                const double v = (double)P[rowoff[i] + j];
-                if (j == i) { all += v * v; continue; }
-                if (fabs(v) < nv && di < nv && fabs((double)P[rowoff[j] + j]) < nv) all += 2.0 * v * v;
-                else off += 2.0 * v * v;
-            }
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            off += __shfl_xor_sync(0xffffffffu, off, o);
-            all += __shfl_xor_sync(0xffffffffu, all, o);
-        }
-        __syncthreads();
-        if (lane == 0) { red[0][warp] = off; red[1][warp] = all; }
-        __syncthreads();
-        if (tid == 0) {
-            double so = 0.0, sd = 0.0;
-            for (int w = 0; w < nw; ++w) { so += red[0][w]; sd += red[1][w]; }
-            const double sa = so + sd;
-            const double prev = sweep == 0 ? 1e300 : *t.prev;
-            const int conv = (so <= JacTol<T>::stop * sa) || sa == 0.0 ||
-                             (so <= JacTol<T>::stall * sa && so > 0.81 * prev) || n < 2;
-            const int s = conv || sweep >= maxs;
-            *t.prev = so;
-            *t.done = s ? (conv ? 1 : 2) : 0;   // 2: stopped by the sweep cap
-            if (s) *t.nsw = sweep;
-            stop = s;
-            thr = JacTol<T>::absf * sqrt(sa);
-        }
-        __syncthreads();
-    }
-    if (stop) {
-        if (t.w)
-            for (int i = tid; i < n; i += JAC_THREADS) t.w[i] = (double)P[rowoff[i] + i];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (POLISH && *(volatile const int*)t.done) {
+        if (tid == 0) *t.nsw = 0;
         return;
     }
-    Sched sc;
-    sc.init(n);
-    const int nr = sc.rounds();
-    if (tid == 0) rhead[0] = nr;
-    constexpr T SKIP = (T)JacTol<T>::skip;
-    for (int r = 0; r < nr; ++r) {
-        const int ns = sc.slots(r);
-        if (tid == 0) cnt = 0;
+    const int n = t.n, m = n + (n & 1), half = m / 2, rounds = m - 1;
+    const int np = m * (m - 1) / 2, nblk = half * (half - 1) / 2;
+    constexpr int CAP = NB > 0 ? mixed_cap(NB) : 0;
+    float* E = NB > 0 ? reinterpret_cast<float*>(sm) : static_cast<float*>(t.P);
+    unsigned char* rest = sm + (size_t)8 * CAP;
+    const int half2 = NB > 0 ? CAP : np;   // the second buffer
+    using DT = std::conditional_t<POLISH, double, float>;
+    DT* D = reinterpret_cast<DT*>(rest);              // two of m
+    float2* cs = reinterpret_cast<float2*>(rest + 16 * (size_t)m);
+    float2* te = cs + half;                            // (tan, e) of the round's pairs
+    // scale: the exponent of the largest |a_ij| (over the float64 bits)
+    {
+        unsigned mx = 0;
+        for (int i = warp; i < n; i += NW)
+            for (int j = i + lane; j < n; j += 32) mx = max(mx, (unsigned)dexp(t.A[(size_t)i * n + j]));
+        mx = __reduce_max_sync(0xffffffffu, mx);
+        if (lane == 0) redm[warp] = mx;
         __syncthreads();
-        for (int k = tid; k < ns; k += JAC_THREADS) {
-            int p, q;
-            sc.slot(r, k, p, q);
-            T c = T(1), s = T(0);
-            if (q >= 0) {
-                const T apq = P[rowoff[p] + q];
-                const T app = P[rowoff[p] + p], aqq = P[rowoff[q] + q];
-                const bool null_pair = (double)fabs(apq) < nullv && (double)fabs(app) < nullv &&
-                                       (double)fabs(aqq) < nullv;
-                if (!null_pair && fabs(apq) > SKIP * sqrt(fabs(app * aqq)) && (double)fabs(apq) > thr &&
-                    apq != T(0)) {
-                    const T th = (aqq - app) / (T(2) * apq);
-                    const T tt = (th >= T(0) ? T(1) : T(-1)) / (fabs(th) + sqrt(th * th + T(1)));
-                    c = T(1) / sqrt(tt * tt + T(1));
-                    s = tt * c;
-                }
-            }
-            Pp[k] = p; Qq[k] = q; Cc[k] = c; Ss[k] = s;
-            if (s != T(0)) {
-                const int slot = atomicAdd(&cnt, 1);   // pairs of a round commute: order is free
-                rlist[(size_t)r * half + slot] = RotE<T>{c, s, p, q};
-            }
-        }
-        __syncthreads();
-        if (tid == 0) rhead[1 + r] = cnt;
-        for (int k = warp; k < ns; k += nw) {
-            const int p = Pp[k], q = Qq[k];
-            const T ck = Cc[k], sk = Ss[k];
-            for (int l = k + lane; l < ns; l += 32) {
-                const T cl = Cc[l], sl = Ss[l];
-                if (sk == T(0) && sl == T(0)) continue;
-                if (l == k) {
-                    const T app = S(p, p), apq = S(p, q), aqq = S(q, q);
-                    const T r_pp = ck * app - sk * apq, r_pq = ck * apq - sk * aqq;
-                    const T r_qp = sk * app + ck * apq, r_qq = sk * apq + ck * aqq;
-                    S(p, p) = ck * r_pp - sk * r_pq;
-                    S(q, q) = sk * r_qp + ck * r_qq;
-                    S(p, q) = T(0);
-                    continue;
-                }
-                const int u = Pp[l], v = Qq[l];
-                const bool hq = q >= 0, hv = v >= 0;
-                const T a_pu = S(p, u);
-                const T a_pv = hv ? S(p, v) : T(0);
-                const T a_qu = hq ? S(q, u) : T(0);
-                const T a_qv = (hq && hv) ? S(q, v) : T(0);
-                const T r_pu = ck * a_pu - sk * a_qu, r_qu = sk * a_pu + ck * a_qu;
-                const T r_pv = ck * a_pv - sk * a_qv, r_qv = sk * a_pv + ck * a_qv;
-                S(p, u) = cl * r_pu - sl * r_pv;
-                if (hv) S(p, v) = sl * r_pu + cl * r_pv;
-                if (hq) S(q, u) = cl * r_qu - sl * r_qv;
-                if (hq && hv) S(q, v) = sl * r_qu + cl * r_qv;
-            }
+        if (tid == 0) {
+            for (int w = 1; w < NW; ++w) mx = max(mx, redm[w]);
+            shift = mx == 0 ? 0 : (int)mx - 1022;   // largest entry in [1/2, 1)
         }
         __syncthreads();
     }
-    if (p_sm)
-        for (size_t e = tid; e < np; e += JAC_THREADS) Pg[e] = P[e];
+    const int sh = shift;
+    for (int e = tid; e < np; e += NT) E[e] = 0.f;
+    for (int e = tid; e < m; e += NT) D[e] = DT(0);
+    __syncthreads();
+    for (int i = warp; i < n; i += NW)
+        for (int j = i + lane; j < n; j += 32) {
+            const double a = t.A[(size_t)i * n + j];
+            if (j == i) {
+                if constexpr (POLISH) D[i] = ldexp(a, -sh);
+                else D[i] = d2f_scaled(a, sh);
+            }
+            else E[tri(m, i, j)] = d2f_scaled(a, sh);
+        }
+    // places of this thread's pair and blocks in a buffer (16 bits each)
+    int kl[NC];
+    unsigned rd[2][NC], wr[2][NC];
+    int pr = 0, pw = 0, pk = 0, pkb = 0;
+    if (NB > 0) {
+#pragma unroll
+        for (int i = 0; i < NC; ++i) {
+            const int e = tid + i * NT;
+            kl[i] = rd[0][i] = rd[1][i] = wr[0][i] = wr[1][i] = 0;
+            if (e < nblk) {
+                int k, l;
+                block_slots(half, e, k, l);
+                const int kb = m - 1 - k, lb = m - 1 - l;
+                kl[i] = k | (l << 16);
+                rd[0][i] = (unsigned)tri(m, k, l) | ((unsigned)tri(m, k, lb) << 16);
+                rd[1][i] = (unsigned)tri(m, l, kb) | ((unsigned)tri(m, lb, kb) << 16);
+                wr[0][i] = (unsigned)tri_next(m, k, l) | ((unsigned)tri_next(m, k, lb) << 16);
+                wr[1][i] = (unsigned)tri_next(m, l, kb) | ((unsigned)tri_next(m, lb, kb) << 16);
+            }
+        }
+        if (tid < half) {
+            pr = tri(m, tid, m - 1 - tid);
+            pw = tri_next(m, tid, m - 1 - tid);
+            pk = next_pos(m, tid);
+            pkb = next_pos(m, m - 1 - tid);
+        }
+    }
+    __syncthreads();
+    float* cur = E;
+    float* nxt = E + half2;
+    DT* Dc = D;
+    DT* Dn = D + m;
+    double off0 = 0.0, prev = 1e300;   // thread 0
+    float nv = 0.f;
+    int s = 0;
+    for (;; ++s) {
+        // |A|_F^2 and the off-diagonal norm without null pairs
+        double dd = 0.0;
+        for (int i = tid; i < n; i += NT) dd = fma((double)Dc[i], (double)Dc[i], dd);
+        float ee = 0.f;
+        for (int i = warp; i < n; i += NW)
+            for (int j = i + 1 + lane; j < n; j += 32) {
+                const float v = cur[tri(m, i, j)];
+                ee = fmaf(v, v, ee);
+            }
+        double e2 = (double)ee;
+        for (int o = 16; o > 0; o >>= 1) {
+            dd += __shfl_xor_sync(0xffffffffu, dd, o);
+            e2 += __shfl_xor_sync(0xffffffffu, e2, o);
+        }
+        if (lane == 0) { red[0][warp] = dd; red[1][warp] = e2; }
+        __syncthreads();
+        if (tid == 0) {
+            double a = 0.0, b = 0.0;
+            for (int w = 0; w < NW; ++w) { a += red[0][w]; b += red[1][w]; }
+            sa_sh = a + 2.0 * b;
+            red[0][0] = 2.0 * b;
+        }
+        __syncthreads();
+        const double sa = sa_sh;
+        double so = red[0][0];
+        if constexpr (POLISH) {   // take the null pairs out
+            nv = (float)Tol::null * sqrtf((float)sa);
+            float nn = 0.f;
+            for (int i = warp; i < n; i += NW)
+                if (fabsf(d2f_trunc(Dc[i])) < nv)
+                    for (int j = i + 1 + lane; j < n; j += 32) {
+                        const float v = cur[tri(m, i, j)];
+                        if (fabsf(v) < nv && fabsf(d2f_trunc(Dc[j])) < nv) nn = fmaf(v, v, nn);
+                    }
+            double n2 = (double)nn;
+            for (int o = 16; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+            __syncthreads();
+            if (lane == 0) red[1][warp] = n2;
+            __syncthreads();
+            if (tid == 0) {
+                double b = 0.0;
+                for (int w = 0; w < NW; ++w) b += red[1][w];
+                so = fmax(0.0, so - 2.0 * b);
+            }
+        }
+        if (tid == 0) {
+            if (s == 0) off0 = so;
+            int conv;
+            if (POLISH) conv = so <= Tol::stop * sa || so <= Tol::gain * off0;
+            else conv = so <= Tol::start * sa;
+            conv = conv || sa == 0.0 || (so <= Tol::stall * sa && so > 0.81 * prev) || n < 2;
+            prev = so;
+            stop = conv || s >= maxs;
+            if (stop) {
+                *t.nsw = s;
+                *t.total = (POLISH ? *t.total : 0) + s;
+                *t.done = POLISH && conv && (off0 <= Tol::last * sa || sa == 0.0 || n < 2) ? 1 : 0;
+            }
+        }
+        __syncthreads();
+        if (stop) break;
+        float2* list = t.rot + (size_t)s * rounds * half;
+        for (int r = 0; r < rounds; ++r) {
+            auto pair = [&](int k, int kb, int from, int to, int tok, int tokb) {
+                const float e = cur[from];
+                const DT dx = Dc[k], dy = Dc[kb];
+                float d;
+                if constexpr (POLISH) d = d2f_trunc(dy - dx);
+                else d = dy - dx;
+                bool on = fabsf(e) >= 0x1p-126f;   // (a subnormal entry is left alone)
+                if constexpr (POLISH) on = on && !(fabsf(e) < nv && fabsf(d2f_trunc(dx)) < nv && fabsf(d2f_trunc(dy)) < nv);
+                const float tn = on ? jac_tan(d, e) : 0.f;
+                const float x = fmaf(tn, tn, 1.f);
+                float c = rsqrtf(x);
+                c = fmaf(0.5f * c, fmaf(-x * c, c, 1.f), c);
+                const float sn = tn * c;
+                cs[k] = make_float2(c, sn);
+                nxt[to] = on ? 0.f : e;
+                if constexpr (POLISH) {
+                    te[k] = make_float2(tn, e);
+                    list[k] = make_float2(tn, 0.f);
+                } else {
+                    Dn[tok] = fmaf(-tn, e, dx);
+                    Dn[tokb] = fmaf(tn, e, dy);
+                    list[k] = make_float2(c, sn);
+                }
+            };
+            if (NB > 0) {
+                if (tid < half) pair(tid, m - 1 - tid, pr, pw, pk, pkb);
+            } else {
+                for (int k = tid; k < half; k += NT) {
+                    const int kb = m - 1 - k;
+                    pair(k, kb, tri(m, k, kb), tri_next(m, k, kb), next_pos(m, k), next_pos(m, kb));
+                }
+            }
+            __syncthreads();
+            auto block = [&](int k, int l, int r0, int r1, int r2, int r3, int w0, int w1, int w2, int w3) {
+                const float2 a = cs[k], b = cs[l];
+                const float kl_ = cur[r0], kL = cur[r1], Kl = cur[r2], KL = cur[r3];
+                const float x0 = a.x * kl_ - a.y * Kl, y0 = a.y * kl_ + a.x * Kl;
+                const float x1 = a.x * kL - a.y * KL, y1 = a.y * kL + a.x * KL;
+                nxt[w0] = b.x * x0 - b.y * x1;
+                nxt[w1] = b.y * x0 + b.x * x1;
+                nxt[w2] = b.x * y0 - b.y * y1;
+                nxt[w3] = b.y * y0 + b.x * y1;
+            };
+            if (NB > 0) {
+#pragma unroll
+                for (int i = 0; i < NC; ++i)
+                    if (tid + i * NT < nblk)
+                        block(kl[i] & 0xffff, kl[i] >> 16, rd[0][i] & 0xffff, rd[0][i] >> 16, rd[1][i] & 0xffff,
+                              rd[1][i] >> 16, wr[0][i] & 0xffff, wr[0][i] >> 16, wr[1][i] & 0xffff, wr[1][i] >> 16);
+            } else {
+                for (int e = tid; e < nblk; e += NT) {
+                    int k, l;
+                    block_slots(half, e, k, l);
+                    const int kb = m - 1 - k, lb = m - 1 - l;
+                    block(k, l, tri(m, k, l), tri(m, k, lb), tri(m, l, kb), tri(m, lb, kb), tri_next(m, k, l),
+                          tri_next(m, k, lb), tri_next(m, l, kb), tri_next(m, lb, kb));
+                }
+            }
+            if constexpr (POLISH)
+                for (int k = NT - 1 - tid; k < half; k += NT) {
+                    const double u = f2d_exact(te[k].x) * f2d_exact(te[k].y);
+                    Dn[next_pos(m, k)] = Dc[k] - u;
+                    Dn[next_pos(m, m - 1 - k)] = Dc[m - 1 - k] + u;
+                }
+            __syncthreads();
+            float* x = cur; cur = nxt; nxt = x;
+            DT* d = Dc; Dc = Dn; Dn = d;
+            list += half;
+        }
+    }
+    if (t.w)
+        for (int i = tid; i < n; i += NT) t.w[i] = ldexp((double)Dc[i], sh);
 }
 
-// Float64 sweep of one matrix by a cluster of JC CTAs (distributed shared
-// memory).  Packed entry e lives in CTA e mod JC at slot e / JC.  Every CTA
-// computes all rotations of a round from the distributed entries; the 2x2
-// blocks {k, l} (k <= l) are split by k mod JC, so each CTA does 1/JC of the
-// float64 update work on its own SM.  Two cluster barriers per round keep
-// the pair phase and the update phase apart.  The arithmetic per entry is
-// the single-CTA kernel's; only rank 0 records rotations and flags.
-constexpr int JC = 8;
-
-template <class T>
-__global__ void __cluster_dims__(JC, 1, 1) __launch_bounds__(JAC_THREADS)
-    k_jac_sweep_cl(const JacTask* __restrict__ tasks, int sweep, int maxs) {
-    namespace cg = cooperative_groups;
-    cg::cluster_group cl = cg::this_cluster();
-    extern __shared__ __align__(16) unsigned char sm[];
-    __shared__ double red[2][JAC_THREADS / 32];
-    __shared__ double part[2][JC];
-    __shared__ double thr;
-    __shared__ int stop, cnt;
-    const int rank = (int)cl.block_rank();
-    const JacTask t = tasks[blockIdx.x / JC];
-    if (sweep > 0 && *(volatile const int*)t.done) return;   // same value in every CTA of the cluster
-    const int n = t.n;
-    const int m = n + (n & 1), half = m / 2;
-    const size_t np = (size_t)n * (n + 1) / 2;
-    const size_t nloc = (np + JC - 1) / JC;
-    int* rowoff = reinterpret_cast<int*>(sm);
-    int* Pp = rowoff + n;
-    int* Qq = Pp + n;
-    T* Cc = reinterpret_cast<T*>(sm + align16((size_t)n * 16));
-    T* Ss = Cc + n;
-    T* Ploc = reinterpret_cast<T*>(sm + jac_head_bytes<T>(n));
-    T* Pg = reinterpret_cast<T*>(t.P);
-    int* rhead = reinterpret_cast<int*>(t.rot);
-    RotE<T>* rlist = reinterpret_cast<RotE<T>*>(reinterpret_cast<unsigned char*>(t.rot) + jac_rot_head(n));
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = JAC_THREADS / 32;
-    for (int i = tid; i < n; i += JAC_THREADS) rowoff[i] = i * n - i * (i + 1) / 2;
-    __syncthreads();
-    if (sweep == 0) {
-        for (int i = warp; i < n; i += nw)
-            for (int j = i + lane; j < n; j += 32) {
-                const size_t e = (size_t)rowoff[i] + j;
-                if ((int)(e % JC) == rank) Ploc[e / JC] = (T)t.A[(size_t)i * n + j];
-            }
-    } else {
-        for (size_t q = tid; q < nloc; q += JAC_THREADS) {
-            const size_t e = q * JC + rank;
-            if (e < np) Ploc[q] = Pg[e];
-        }
-    }
-    cl.sync();   // every CTA of the cluster is running and has its slice before any remote access
-    auto S = [&](int a, int b) -> T& {
-        const size_t e = a <= b ? (size_t)rowoff[a] + b : (size_t)rowoff[b] + a;
-        return cl.map_shared_rank(Ploc, (int)(e % JC))[e / JC];
-    };
-    // convergence test over the whole matrix (partial sums gathered in rank
-    // 0): |A|_F first (it sets the null level, broadcast to every CTA), then
-    // the off-diagonal norm without null pairs; the diagonal is copied into
-    // the head's spare space so the null test reads it locally
-    __shared__ double nullv;
-    double* dg = reinterpret_cast<double*>(sm + align16((size_t)n * 16) + align16(2 * (size_t)n * sizeof(T)));
-    {
-        double all = 0.0;
-        for (int i = warp; i < n; i += nw)
-            for (int j = i + lane; j < n; j += 32) {
-                const size_t e = (size_t)rowoff[i] + j;
-                if ((int)(e % JC) != rank) continue;
-                const double v = (double)Ploc[e / JC];
-                all += (j == i ? 1.0 : 2.0) * v * v;
-            }
-        for (int o = 16; o > 0; o >>= 1) all += __shfl_xor_sync(0xffffffffu, all, o);
-        if (lane == 0) red[1][warp] = all;
-        __syncthreads();
-        if (tid == 0) {
-            double sd = 0.0;
-            for (int w = 0; w < nw; ++w) sd += red[1][w];
-            cl.map_shared_rank(&part[0][0], 0)[rank] = sd;
-        }
-        for (int i = tid; i < n; i += JAC_THREADS) {
-            const size_t e = (size_t)rowoff[i] + i;
-            dg[i] = (double)cl.map_shared_rank(Ploc, (int)(e % JC))[e / JC];
-        }
-        cl.sync();
-        if (rank == 0 && tid == 0) {
-            double sa = 0.0;
-            for (int r = 0; r < JC; ++r) sa += part[0][r];
-            const double nvv = JacTol<T>::null * sqrt(sa);
-            for (int r = 0; r < JC; ++r) *cl.map_shared_rank(&nullv, r) = nvv;
-        }
-        cl.sync();
-        const double nv = nullv;
-        double off = 0.0;
-        all = 0.0;
-        for (int i = warp; i < n; i += nw)
-            for (int j = i + lane; j < n; j += 32) {
-                const size_t e = (size_t)rowoff[i] + j;
-                if ((int)(e % JC) != rank) continue;
-                const double v = (double)Ploc[e / JC];
-                if (j == i) { all += v * v; continue; }
-                if (fabs(v) < nv && fabs(dg[i]) < nv && fabs(dg[j]) < nv) all += 2.0 * v * v;
-                else off += 2.0 * v * v;
-            }
-        for (int o = 16; o > 0; o >>= 1) {
-            off += __shfl_xor_sync(0xffffffffu, off, o);
-            all += __shfl_xor_sync(0xffffffffu, all, o);
-        }
-        __syncthreads();
-        if (lane == 0) { red[0][warp] = off; red[1][warp] = all; }
-        __syncthreads();
-        if (tid == 0) {
-            double so = 0.0, sd = 0.0;
-            for (int w = 0; w < nw; ++w) { so += red[0][w]; sd += red[1][w]; }
-            double* p0 = cl.map_shared_rank(&part[0][0], 0);
-            p0[rank] = so;
-            p0[JC + rank] = sd;
-        }
-        cl.sync();
-        if (rank == 0 && tid == 0) {
-            double so = 0.0, sd = 0.0;
-            for (int r = 0; r < JC; ++r) { so += part[0][r]; sd += part[1][r]; }
-            const double sa = so + sd;
-            const double prev = sweep == 0 ? 1e300 : *t.prev;
-            const int conv = (so <= JacTol<T>::stop * sa) || sa == 0.0 ||
-                             (so <= JacTol<T>::stall * sa && so > 0.81 * prev) || n < 2;
-            const int s = conv || sweep >= maxs;
-            *t.prev = so;
-            *t.done = s ? (conv ? 1 : 2) : 0;   // 2: stopped by the sweep cap
-            if (s) *t.nsw = sweep;
-            const double th = JacTol<T>::absf * sqrt(sa);
-            for (int r = 0; r < JC; ++r) { *cl.map_shared_rank(&stop, r) = s; *cl.map_shared_rank(&thr, r) = th; }
-        }
-        cl.sync();
-    }
-    if (stop) {
-        if (t.w)
-            for (int i = tid; i < n; i += JAC_THREADS) {
-                const size_t e = (size_t)rowoff[i] + i;
-                if ((int)(e % JC) == rank) t.w[i] = (double)Ploc[e / JC];
-            }
-        return;
-    }
-    Sched sc;
-    sc.init(n);
-    const int nr = sc.rounds();
-    if (rank == 0 && tid == 0) rhead[0] = nr;
-    constexpr T SKIP = (T)JacTol<T>::skip;
-    for (int r = 0; r < nr; ++r) {
-        const int ns = sc.slots(r);
-        if (tid == 0) cnt = 0;
-        __syncthreads();
-        for (int k = tid; k < ns; k += JAC_THREADS) {
-            int p, q;
-            sc.slot(r, k, p, q);
-            T c = T(1), s = T(0);
-            if (q >= 0) {
-                const T apq = S(p, q), app = S(p, p), aqq = S(q, q);
-                const bool null_pair = (double)fabs(apq) < nullv && (double)fabs(app) < nullv &&
-                                       (double)fabs(aqq) < nullv;
-                if (!null_pair && fabs(apq) > SKIP * sqrt(fabs(app * aqq)) && (double)fabs(apq) > thr &&
-                    apq != T(0)) {
-                    const T th = (aqq - app) / (T(2) * apq);
-                    const T tt = (th >= T(0) ? T(1) : T(-1)) / (fabs(th) + sqrt(th * th + T(1)));
-                    c = T(1) / sqrt(tt * tt + T(1));
-                    s = tt * c;
-                }
-            }
-            Pp[k] = p; Qq[k] = q; Cc[k] = c; Ss[k] = s;
-            if (rank == 0 && s != T(0)) {
-                const int slot = atomicAdd(&cnt, 1);
-                rlist[(size_t)r * half + slot] = RotE<T>{c, s, p, q};
-            }
-        }
-        __syncthreads();
-        if (rank == 0 && tid == 0) rhead[1 + r] = cnt;
-        cl.sync();   // every CTA has read the pair entries before any is updated
-        for (int k = rank + JC * warp; k < ns; k += JC * nw) {
-            const int p = Pp[k], q = Qq[k];
-            const T ck = Cc[k], sk = Ss[k];
-            for (int l = k + lane; l < ns; l += 32) {
-                const T cl_ = Cc[l], sl = Ss[l];
-                if (sk == T(0) && sl == T(0)) continue;
-                if (l == k) {
-                    const T app = S(p, p), apq = S(p, q), aqq = S(q, q);
-                    const T r_pp = ck * app - sk * apq, r_pq = ck * apq - sk * aqq;
-                    const T r_qp = sk * app + ck * apq, r_qq = sk * apq + ck * aqq;
-                    S(p, p) = ck * r_pp - sk * r_pq;
-                    S(q, q) = sk * r_qp + ck * r_qq;
-                    S(p, q) = T(0);
-                    continue;
-                }
-                const int u = Pp[l], v = Qq[l];
-                const bool hq = q >= 0, hv = v >= 0;
-                const T a_pu = S(p, u);
-                const T a_pv = hv ? S(p, v) : T(0);
-                const T a_qu = hq ? S(q, u) : T(0);
-                const T a_qv = (hq && hv) ? S(q, v) : T(0);
-                const T r_pu = ck * a_pu - sk * a_qu, r_qu = sk * a_pu + ck * a_qu;
-                const T r_pv = ck * a_pv - sk * a_qv, r_qv = sk * a_pv + ck * a_qv;
-                S(p, u) = cl_ * r_pu - sl * r_pv;
-                if (hv) S(p, v) = sl * r_pu + cl_ * r_pv;
-                if (hq) S(q, u) = cl_ * r_qu - sl * r_qv;
-                if (hq && hv) S(q, v) = sl * r_qu + cl_ * r_qv;
-            }
-        }
-        cl.sync();   // updates visible to every CTA before the next pair phase
-    }
-    for (size_t q = tid; q < nloc; q += JAC_THREADS) {
-        const size_t e = q * JC + rank;
-        if (e < np) Pg[e] = Ploc[q];
+__global__ void k_jac_rot64(const JacTask* __restrict__ tasks) {
+    const JacTask t = tasks[blockIdx.y];
+    const int m = t.n + (t.n & 1);
+    const size_t tot = (size_t)*t.nsw * (m - 1) * (m / 2);
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < tot; i += (size_t)gridDim.x * blockDim.x) {
+        const float tn = t.rot[i].x;
+        double c = 1.0, s = (double)tn;
+        if (fabsf(tn) > 1e-9f) jac_cs64(s, c, s);   // below, c rounds to 1 and s to t
+        t.rot64[i] = make_double2(c, s);
     }
 }
 
+// A warp per row of V.  The lane of slot k of a round rotates the row's
+// entries of that slot's two columns; the next round's list entries are
+// fetched while the present ones are applied.  Float64: four operations per
+// rotation and row on the float64 pipe, spread over n / 4 CTAs (32 rows per
+// warp, as before, left it on n / 32 SMs).
+template <class T> struct Vec2;
+template <> struct Vec2<float> { using type = float2; };
+template <> struct Vec2<double> { using type = double2; };
+
 template <class T>
-__global__ void __launch_bounds__(32) k_jac_apply(const JacTask* __restrict__ tasks, const JacRows* __restrict__ rb,
-                                                 int sweep) {
+__global__ void __launch_bounds__(32 * JAC_APPLY_ROWS) k_jac_apply(const JacTask* __restrict__ tasks,
+                                                                  const JacRows* __restrict__ rb, int ident) {
     extern __shared__ __align__(16) unsigned char sm[];
+    using T2 = typename Vec2<T>::type;
     const JacRows b = rb[blockIdx.x];
     const JacTask t = tasks[b.task];
-    const int done = *(volatile const int*)t.done;
-    if (sweep > 0 && done) return;
-    const int n = t.n, ld = n | 1, lane = threadIdx.x;
-    T* R = reinterpret_cast<T*>(sm);
-    for (int e = lane; e < b.rows * n; e += 32) {
-        const int i = e / n, j = e % n;
-        R[i * ld + j] = (sweep == 0 && !t.vinit) ? T(b.r0 + i == j ? 1 : 0) : (T)t.V[(size_t)(b.r0 + i) * n + j];
-    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nsw = *(volatile const int*)t.nsw;
+    if (warp >= b.rows || (nsw == 0 && !ident)) return;
+    const int n = t.n, m = n + (n & 1), half = m / 2, rounds = m - 1, row = b.r0 + warp;
+    T* R = reinterpret_cast<T*>(sm) + (size_t)warp * m;
+    double* Vr = t.V + (size_t)row * n;
+    for (int j = lane; j < m; j += 32) R[j] = j >= n ? T(0) : ident ? T(j == row ? 1 : 0) : (T)Vr[j];
     __syncwarp();
-    if (!done) {   // the whole warp takes part (shuffles); lanes >= rows only relay rotations
-        const int m = n + (n & 1), half = m / 2;
-        const int* rhead = reinterpret_cast<const int*>(t.rot);
-        const RotE<T>* rlist =
-            reinterpret_cast<const RotE<T>*>(reinterpret_cast<const unsigned char*>(t.rot) + jac_rot_head(n));
-        const int nr = __ldg(rhead);
-        for (int r = 0; r < nr; ++r) {
-            const int c = __ldg(rhead + 1 + r);
-            const RotE<T>* L = rlist + (size_t)r * half;
-            // the rotations of one round act on disjoint columns.  The warp
-            // reads 32 of them at a time, one per lane (coalesced), and hands
-            // them round by shuffles; each lane then runs them on its own row
-            // eight at a time, all loads before all stores.
-            for (int j0 = 0; j0 < c; j0 += 32) {
-                const int cnt = min(32, c - j0);
-                RotE<T> mine{};
-                if (lane < cnt) mine = L[j0 + lane];
-                for (int q0 = 0; q0 < cnt; q0 += 8) {
-                    const int nq = min(8, cnt - q0);
-                    T cs[8], sn[8], x[8], y[8];
-                    int pp[8], qq[8];
+    const T2* list;
+    if constexpr (sizeof(T) == 8) list = t.rot64; else list = t.rot;
+    constexpr int PF = 4;   // list entries per lane fetched ahead
+    T2 nx[PF];
+    const size_t total = (size_t)nsw * rounds;
+    auto fetch = [&](size_t g) {
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        const int src = q0 + (q < nq ? q : 0);
-                        cs[q] = __shfl_sync(0xffffffffu, mine.c, src);
-                        sn[q] = __shfl_sync(0xffffffffu, mine.s, src);
-                        pp[q] = __shfl_sync(0xffffffffu, mine.p, src);
-                        qq[q] = __shfl_sync(0xffffffffu, mine.q, src);
-                    }
-                    if (lane < b.rows) {
-                        T* row = R + lane * ld;
+        for (int q = 0; q < PF; ++q)
+            if (g < total && lane + 32 * q < half) nx[q] = list[g * half + lane + 32 * q];
+    };
+    auto rotate = [&](int k, int r, T2 cs) {
+        if (cs.y == T(0)) return;
+        int pa = k - 1 + r, pb = m - 2 - k + r;
+        pa = k == 0 ? 0 : (pa >= rounds ? pa - rounds : pa) + 1;
+        pb = (pb >= rounds ? pb - rounds : pb) + 1;
+        const T x = R[pa], y = R[pb];
+        R[pa] = cs.x * x - cs.y * y;
+        R[pb] = cs.y * x + cs.x * y;
+    };
+    fetch(0);
+    int r = 0;
+    for (size_t g = 0; g < total; ++g) {
+        T2 cs[PF];
 #pragma unroll
-                        for (int q = 0; q < 8; ++q)
-                            if (q < nq) { x[q] = row[pp[q]]; y[q] = row[qq[q]]; }
+        for (int q = 0; q < PF; ++q) cs[q] = nx[q];
+        fetch(g + 1);
 #pragma unroll
-                        for (int q = 0; q < 8; ++q)
-                            if (q < nq) {
-                                row[pp[q]] = cs[q] * x[q] - sn[q] * y[q];
-                                row[qq[q]] = sn[q] * x[q] + cs[q] * y[q];
-                            }
+        for (int q = 0; q < PF; ++q)
+            if (lane + 32 * q < half) rotate(lane + 32 * q, r, cs[q]);
+        for (int k = lane + 32 * PF; k < half; k += 32) rotate(k, r, list[g * half + k]);
+        __syncwarp();
+        if (++r == rounds) r = 0;
+    }
+    for (int j = lane; j < n; j += 32) Vr[j] = (double)R[j];
+}
+
+// -------------------------------------------------------------- float64
+// All float64 sweeps of one matrix in one launch, on C CTAs (a cluster of 8,
+// or one CTA for small matrices).  The packed upper triangle is spread over
+// the CTAs' shared memories (entry e in CTA e mod C, slot e / C; with a_sm
+// false it is the upper part of t.A, which is then destroyed), the rows of V
+// likewise (row i in CTA i mod C; with v_sm false in t.V).  A round: every CTA
+// computes all rotations from the distributed entries; barrier; it transforms
+// its share of the 2 x 2 blocks of slots and its rows of V; barrier.  Bound by
+// the float64 pipes of the C SMs (4 n^2 operations a round) and, for small n,
+// by the chain rotation - barrier - update - barrier.  A float64 instruction
+// occupies a sub-partition for 64 clocks however few lanes are active, so what
+// counts is their number per warp.  Measured against the one-CTA kernel with
+// divisions and square roots: twelve 13 x 13 350 -> 188 us, seven of 90 and
+// down 25.6 -> 4.1 ms; against the launch-per-sweep cluster form 21 -> 4.2 ms.
+constexpr int JC = 8;
+
+struct EigFit { size_t head, a, v; };   // shared memory of one CTA: head, triangle share, V rows
+__host__ __device__ inline EigFit eig_fit(int n, int C) {
+    EigFit f;
+    const size_t half = (size_t)(n + 1) / 2;
+    // rowoff, slots, (c, s, tan) and the rotated pairs' blocks, the diagonal
+    f.head = align16((size_t)n * 4) + align16(half * 8) + align16(half * 48) + align16((size_t)n * 8);
+    f.a = align16(((size_t)n * (n + 1) / 2 + C - 1) / C * 8);
+    f.v = align16(((size_t)n + C - 1) / C * n * 8);
+    return f;
+}
+__host__ __device__ inline bool eig_a_sm(int n, int C) { const EigFit f = eig_fit(n, C); return f.head + f.a <= (size_t)JAC_SMEM; }
+__host__ __device__ inline bool eig_v_sm(int n, int C) { const EigFit f = eig_fit(n, C); return f.head + f.a + f.v <= (size_t)JAC_SMEM; }
+inline size_t eig_smem(int n, int C) {
+    const EigFit f = eig_fit(n, C);
+    return f.head + (eig_a_sm(n, C) ? f.a : 0) + (eig_v_sm(n, C) ? f.v : 0);
+}
+
+template <int C, int NT, bool A_SM>
+__device__ __forceinline__ void eig_body(const EigTask& t, double nullrel, int maxs, int* flag, int rank) {
+    namespace cg = cooperative_groups;
+    extern __shared__ __align__(16) unsigned char sm[];
+    constexpr int NW = NT / 32, NBC = 4;
+    __shared__ float red[2][NW];
+    __shared__ float part[2][C];
+    const int n = t.n, m = n + (n & 1), half = m / 2, rounds = m - 1;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool v_sm = A_SM && eig_v_sm(n, C);
+    const EigFit fit = eig_fit(n, C);
+    int* rowoff = reinterpret_cast<int*>(sm);
+    int2* slots = reinterpret_cast<int2*>(sm + align16((size_t)n * 4));   // (p, q); q < 0: not rotated
+    double* Cc = reinterpret_cast<double*>(sm + align16((size_t)n * 4) + align16((size_t)half * 8));
+    double *Ss = Cc + half, *Xa = Ss + half, *Xe = Xa + half, *Xb = Xe + half;
+    double* Tt = Xb + half;
+    double* dg = reinterpret_cast<double*>(sm + align16((size_t)n * 4) + align16((size_t)half * 8) +
+                                           align16((size_t)half * 48));
+    double* Ploc = reinterpret_cast<double*>(sm + fit.head);
+    const int nrow = (n - rank + C - 1) / C;          // this CTA's rows of V
+    double* Vl = v_sm ? reinterpret_cast<double*>(sm + fit.head + fit.a) : t.V + (size_t)rank * n;
+    const size_t vld = v_sm ? n : (size_t)C * n;
+    auto sync = [&] {
+        if constexpr (C > 1) cg::this_cluster().sync();
+        else __syncthreads();
+    };
+    auto at = [&](int a, int b) -> double& {   // any order
+        const int e = rowoff[min(a, b)] + max(a, b);
+        if constexpr (!A_SM) return t.A[e];
+        else if constexpr (C > 1) return cg::this_cluster().map_shared_rank(Ploc, e % C)[e / C];
+        else return Ploc[e];
+    };
+    // scaled by a power of two so that the largest entry is in [1/2, 1)
+    unsigned mx = 0;
+    for (int i = warp; i < n; i += NW)
+        for (int j = i + lane; j < n; j += 32) mx = max(mx, (unsigned)dexp(t.A[(size_t)i * n + j]));
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if (lane == 0) red[0][warp] = __uint_as_float(mx);
+    for (int i = tid; i < n; i += NT) rowoff[i] = A_SM ? i * n - i * (i + 1) / 2 : i * n;
+    sync();   // (in place: nobody scales an entry before all have looked)
+    for (int w = 0; w < NW; ++w) mx = max(mx, __float_as_uint(red[0][w]));
+    const int sh = mx == 0 ? 0 : (int)mx - 1022;
+    for (int i = warp; i < n; i += NW)
+        for (int j = i + lane; j < n; j += 32) {
+            const int e = rowoff[i] + j;
+            if (A_SM ? e % C != rank : i % C != rank) continue;
+            const double v = ldexp(t.A[(size_t)i * n + j], -sh);
+            if (A_SM) Ploc[e / C] = v;
+            else t.A[e] = v;
+        }
+    for (int i = warp; i < nrow; i += NW)
+        for (int j = lane; j < n; j += 32) Vl[i * vld + j] = j == rank + i * C ? 1.0 : 0.0;
+    // this thread's first blocks (all of them up to n = 256 on a cluster)
+    const int nblk = half * (half - 1) / 2;
+    int bk[NBC];
+#pragma unroll
+    for (int i = 0; i < NBC; ++i) {
+        const int blk = rank + C * (tid + i * NT);
+        int k = 0, l = 0;
+        if (blk < nblk) block_slots(half, blk, k, l);
+        bk[i] = k | (l << 16);
+    }
+    int ek = 0, el = 0;   // this thread's block when every entry has a thread
+    if (C == 1 && 4 * nblk <= NT && tid < 4 * nblk) block_slots(half, tid >> 2, ek, el);
+    const unsigned hinv = 0xFFFFFFFFu / (unsigned)half + 1u;   // e / half = umulhi(e, hinv) for e < 2^20
+    sync();   // every CTA of the cluster is running and has its share before any remote access
+    double nullv = 0.0;
+    float prev = 3e38f;
+    for (int sweep = 0;; ++sweep) {
+        // off-norm without null pairs, and |A|_F^2, in float32 (they decide
+        // when to stop, to no more than a few digits); the partial sums of all
+        // CTAs are added in rank order by everyone
+        for (int i = tid; i < n; i += NT) dg[i] = at(i, i);
+        __syncthreads();
+        float off = 0.f, all = 0.f;
+        for (int i = warp; i < n; i += NW)
+            for (int j = i + lane; j < n; j += 32) {
+                if (A_SM ? (rowoff[i] + j) % C != rank : i % C != rank) continue;
+                const double v = at(i, j);
+                const float f = d2f_trunc(v);
+                if (j == i) all = fmaf(f, f, all);
+                else if (abs_below(v, nullv) && abs_below(dg[i], nullv) && abs_below(dg[j], nullv))
+                    all = fmaf(2.f * f, f, all);
+                else off = fmaf(2.f * f, f, off);
+            }
+        for (int o = 16; o > 0; o >>= 1) {
+            off += __shfl_xor_sync(0xffffffffu, off, o);
+            all += __shfl_xor_sync(0xffffffffu, all, o);
+        }
+        if (lane == 0) { red[0][warp] = off; red[1][warp] = all; }
+        __syncthreads();
+        if (tid < 2 * C) {
+            const int which = tid & 1, to = tid >> 1;
+            float y = 0.f;
+            for (int w = 0; w < NW; ++w) y += red[which][w];
+            float* p = &part[which][rank];
+            if constexpr (C > 1) p = cg::this_cluster().map_shared_rank(p, to);
+            *p = y;
+        }
+        sync();
+        float so = 0.f, sd = 0.f;
+        for (int r = 0; r < C; ++r) { so += part[0][r]; sd += part[1][r]; }
+        const float sa = so + sd;
+        if (sweep == 0) nullv = nullrel * (double)sqrtf(sa);   // the first test counts every pair
+        const bool conv = so <= (float)Tol::stop * sa || sa == 0.f || (so <= (float)Tol::stall * sa && so > 0.81f * prev) || n < 2;
+        prev = so;
+        if (conv || sweep >= maxs) {
+            if (flag && rank == 0 && tid == 0) *flag = conv ? 1 : 2;
+            break;
+        }
+        for (int r = 0; r < rounds; ++r) {
+            for (int k = tid; k < half; k += NT) {
+                int x = k - 1 + r, y = m - 2 - k + r;
+                x = k == 0 ? 0 : (x >= rounds ? x - rounds : x) + 1;
+                y = (y >= rounds ? y - rounds : y) + 1;
+                const int p = min(x, y), q = max(x, y);
+                bool on = q < n;
+                if (on) {
+                    const double a = at(p, p), e = at(p, q), b = at(q, q);
+                    const float fd = d2f_trunc(b - a), fe = d2f_trunc(e);
+                    on = fe != 0.f && !jac_negligible(e, a, b) &&
+                         !(abs_below(e, nullv) && abs_below(a, nullv) && abs_below(b, nullv));
+                    if (on) {
+                        const double tn = jac_tan64(b - a, e, fd, fe);
+                        double c, s;
+                        jac_cs64(tn, c, s);
+                        Cc[k] = c; Ss[k] = s; Tt[k] = tn;
+                        Xa[k] = a; Xe[k] = e; Xb[k] = b;
                     }
                 }
+                if (!on) { Cc[k] = 1.0; Ss[k] = 0.0; }
+                slots[k] = make_int2(p | (on ? 1 << 16 : 0), q < n ? q : -1);
             }
+            sync();   // every CTA has read the pair entries before any is updated
+            auto block = [&](int k, int l) {
+                const int2 sk_ = slots[k], sl_ = slots[l];
+                if (((sk_.x | sl_.x) >> 16) == 0) return;
+                const double ck = Cc[k], sk = Ss[k], cl = Cc[l], sl = Ss[l];
+                const int p = sk_.x & 0xffff, q = sk_.y, u = sl_.x & 0xffff, v = sl_.y;
+                const bool hq = q >= 0, hv = v >= 0;
+                // a missing partner (odd n) reads the pair's own entry with s = 0
+                double& pu = at(p, u);
+                double& pv = at(p, hv ? v : u);
+                double& qu = at(hq ? q : p, u);
+                double& qv = at(hq ? q : p, hv ? v : u);
+                const double a_pu = pu, a_pv = pv, a_qu = qu, a_qv = qv;
+                const double r_pu = fma(ck, a_pu, -(sk * a_qu)), r_qu = fma(sk, a_pu, ck * a_qu);
+                const double r_pv = fma(ck, a_pv, -(sk * a_qv)), r_qv = fma(sk, a_pv, ck * a_qv);
+                if (hq && hv) qv = fma(sl, r_qu, cl * r_qv);
+                if (hq) qu = fma(cl, r_qu, -(sl * r_qv));
+                if (hv) pv = fma(sl, r_pu, cl * r_pv);
+                pu = fma(cl, r_pu, -(sl * r_pv));
+            };
+            if (C == 1 && 4 * nblk <= NT) {
+                // few blocks: a thread per entry (six operations instead of
+                // sixteen; a float64 instruction takes a warp's sub-partition
+                // 64 clocks however few lanes it has)
+                double out = 0.0;
+                double* dst = nullptr;
+                if (tid < 4 * nblk) {
+                    const int2 sk_ = slots[ek], sl_ = slots[el];
+                    const int p = sk_.x & 0xffff, q = sk_.y, u = sl_.x & 0xffff, v = sl_.y;
+                    const bool lo = tid & 1, ro = tid & 2;
+                    if ((!lo || q >= 0) && (!ro || v >= 0) && ((sk_.x | sl_.x) >> 16)) {
+                        const double ck = Cc[ek], sk = Ss[ek], cl = Cc[el], sl = Ss[el];
+                        const int q_ = q >= 0 ? q : p, v_ = v >= 0 ? v : u;
+                        const double a_pu = at(p, u), a_pv = at(p, v_), a_qu = at(q_, u), a_qv = at(q_, v_);
+                        const double al = lo ? sk : ck, be = lo ? ck : -sk, ga = ro ? sl : cl, de = ro ? cl : -sl;
+                        const double x = fma(al, a_pu, be * a_qu), y = fma(al, a_pv, be * a_qv);
+                        out = fma(ga, x, de * y);
+                        dst = &at(lo ? q : p, ro ? v : u);
+                    }
+                }
+                __syncwarp();   // the four lanes of a block have read it
+                if (dst) *dst = out;
+            } else
+#pragma unroll
+                for (int i = 0; i < NBC; ++i)
+                    if (rank + C * (tid + i * NT) < nblk) block(bk[i] & 0xffff, bk[i] >> 16);
+            for (int blk = rank + C * (tid + NBC * NT); blk < nblk; blk += C * NT) {
+                int k, l;
+                block_slots(half, blk, k, l);
+                block(k, l);
+            }
+            for (int k = NT - 1 - tid; k < half; k += NT)
+                if (k % C == rank && (slots[k].x >> 16)) {   // the rotated pairs' own blocks
+                    const int p = slots[k].x & 0xffff, q = slots[k].y;
+                    double a = Xa[k], e = Xe[k], b = Xb[k];
+                    jac_block64(Tt[k], Cc[k], a, e, b);
+                    at(p, p) = a;
+                    at(p, q) = e;
+                    at(q, q) = b;
+                }
+            for (int e = tid; e < nrow * half; e += NT) {
+                const int i = half > 1 && nrow * half < (1 << 20) ? (int)__umulhi((unsigned)e, hinv) : e / half, k = e - i * half;
+                const int2 sk_ = slots[k];
+                if (!(sk_.x >> 16)) continue;
+                const double c = Cc[k], s = Ss[k];
+                double* v = Vl + i * vld;
+                const double x = v[sk_.x & 0xffff], y = v[sk_.y];
+                v[sk_.x & 0xffff] = fma(c, x, -(s * y));
+                v[sk_.y] = fma(s, x, c * y);
+            }
+            sync();   // updates visible to every CTA before the next pair phase
         }
     }
-    __syncwarp();
-    for (int e = lane; e < b.rows * n; e += 32) {
-        const int i = e / n, j = e % n;
-        t.V[(size_t)(b.r0 + i) * n + j] = (double)R[i * ld + j];
-    }
+    // the diagonal was gathered by the last test
+    for (int i = rank + C * tid; i < n; i += C * NT) t.w[i] = ldexp(dg[i], sh);
+    if (v_sm)
+        for (int i = warp; i < nrow; i += NW)
+            for (int j = lane; j < n; j += 32) t.V[(size_t)(rank + i * C) * n + j] = Vl[(size_t)i * n + j];
+    if constexpr (C > 1) cg::this_cluster().sync();   // no CTA leaves while its shared memory may be read
+}
+
+__global__ void __launch_bounds__(128) k_eig_one(const EigTask* __restrict__ tasks, double nullrel, int maxs, int* flags) {
+    eig_body<1, 128, true>(tasks[blockIdx.x], nullrel, maxs, flags ? flags + blockIdx.x : nullptr, 0);
+}
+__global__ void __cluster_dims__(JC, 1, 1) __launch_bounds__(256)
+    k_eig_cl(const EigTask* __restrict__ tasks, double nullrel, int maxs, int* flags) {
+    const EigTask t = tasks[blockIdx.x / JC];
+    int* flag = flags ? flags + blockIdx.x / JC : nullptr;
+    const int rank = (int)cooperative_groups::this_cluster().block_rank();
+    if (eig_a_sm(t.n, JC)) eig_body<JC, 256, true>(t, nullrel, maxs, flag, rank);
+    else eig_body<JC, 256, false>(t, nullrel, maxs, flag, rank);
 }
 
 }  // namespace
 
-size_t jac_p_bytes(int n) { return (size_t)n * (n + 1) / 2 * sizeof(double); }
-size_t jac_rot_bytes(int n) {
-    const int m = n + (n & 1), half = m / 2;
-    return jac_rot_head(n) + (size_t)jac_max_rounds(n) * half * sizeof(RotE<double>);
+size_t jac_e_bytes(int n) {
+    const size_t m = n + (n & 1);
+    return n <= 236 ? 0 : 4 * m * (m - 1);
 }
-// Rows of V per apply block (one warp, one row per lane).
-int jac_rows_per_block(int n, bool f32) {
-    const size_t row = (size_t)(n | 1) * (f32 ? 4 : 8);
-    const size_t r = (size_t)JAC_SMEM / row;
-    return (int)(r < 32 ? (r < 1 ? 1 : r) : 32);
+size_t jac_rot_entries(int n) {
+    const size_t m = n + (n & 1);
+    return (m - 1) * (m / 2);
 }
 
-static void jac_attributes() {
-    ensure_smem_attr(reinterpret_cast<const void*>(k_jac_sweep<double>), JAC_SMEM);
-    ensure_smem_attr(reinterpret_cast<const void*>(k_jac_sweep<float>), JAC_SMEM);
-    ensure_smem_attr(reinterpret_cast<const void*>(k_jac_apply<double>), JAC_SMEM);
-    ensure_smem_attr(reinterpret_cast<const void*>(k_jac_apply<float>), JAC_SMEM);
-}
-
-void launch_jac_sweep(const JacTask* tasks, int ntask, int sweep, int maxs, bool f32, cudaStream_t st) {
-    if (ntask <= 0) return;
-    jac_attributes();
+template <int NT, int NB>
+static void launch_mixed(const JacTask* tasks, int ntask, size_t smem, bool polish, int maxs, cudaStream_t st) {
     count_launch();
-    if (f32) k_jac_sweep<float><<<ntask, JAC_THREADS, JAC_SMEM, st>>>(tasks, sweep, maxs);
-    else k_jac_sweep<double><<<ntask, JAC_THREADS, JAC_SMEM, st>>>(tasks, sweep, maxs);
+    if (polish) {
+        ensure_smem_attr(reinterpret_cast<const void*>(k_jac_mixed<NT, NB, true>), MIX_SMEM);
+        k_jac_mixed<NT, NB, true><<<ntask, NT, smem, st>>>(tasks, maxs);
+    } else {
+        ensure_smem_attr(reinterpret_cast<const void*>(k_jac_mixed<NT, NB, false>), MIX_SMEM);
+        k_jac_mixed<NT, NB, false><<<ntask, NT, smem, st>>>(tasks, maxs);
+    }
 }
 
-// Shared memory of the cluster sweep for an n x n matrix (0: does not fit).
-int jac_cluster_smem(int n) {
-    const size_t np = (size_t)n * (n + 1) / 2;
-    const size_t b = jac_head_bytes<double>(n) + (np + JC - 1) / JC * sizeof(double);
-    return b <= (size_t)JAC_SMEM ? (int)b : 0;
-}
-
-void launch_jac_sweep_cluster(const JacTask* tasks, int ntask, int sweep, int maxs, int smem, cudaStream_t st) {
+// The number of threads follows the largest matrix (half (half - 1) / 2
+// blocks): enough that a round's update is a few blocks per thread, few
+// enough that its barriers stay cheap (21 clocks at 128 threads, 45 at 512).
+// n up to 46: at most 253 blocks; 92: 1035; 180: 4005; 236 (shared memory): 6903.
+void launch_jac_mixed(const JacTask* tasks, int ntask, int nmax, bool polish, int maxs, cudaStream_t st) {
     if (ntask <= 0) return;
-    ensure_smem_attr(reinterpret_cast<const void*>(k_jac_sweep_cl<double>), JAC_SMEM);
-    count_launch();
-    k_jac_sweep_cl<double><<<ntask * JC, JAC_THREADS, smem, st>>>(tasks, sweep, maxs);
+    if (nmax <= 46) launch_mixed<128, 2>(tasks, ntask, mixed_smem(nmax, mixed_cap(2)), polish, maxs, st);
+    else if (nmax <= 92) launch_mixed<256, 5>(tasks, ntask, mixed_smem(nmax, mixed_cap(5)), polish, maxs, st);
+    else if (nmax <= 180) launch_mixed<512, 8>(tasks, ntask, mixed_smem(nmax, mixed_cap(8)), polish, maxs, st);
+    else if (nmax <= 236) launch_mixed<512, 14>(tasks, ntask, mixed_smem(nmax, mixed_cap(14)), polish, maxs, st);
+    else launch_mixed<1024, 0>(tasks, ntask, mixed_smem(nmax, 0), polish, maxs, st);
 }
 
-void launch_jac_apply(const JacTask* tasks, const JacRows* rows, int nblocks, int smem, int sweep, bool f32,
+void launch_jac_rot64(const JacTask* tasks, int ntask, cudaStream_t st) {
+    for (int i = 0; i < ntask; i += 65535) {
+        count_launch();
+        k_jac_rot64<<<dim3(16, ntask - i < 65535 ? ntask - i : 65535), 256, 0, st>>>(tasks + i);
+    }
+}
+
+// One CTA below n = 28, a cluster of 8 from there (measured, eight matrices:
+// n = 23 and 24 both 0.5 ms, n = 31 and 32 on the cluster 0.8 ms).
+bool eig_on_cluster(int n) { return n >= 28; }
+bool eig_in_place(int n) { return eig_on_cluster(n) && !eig_a_sm(n, JC); }
+
+void order_eig_tasks(EigTask* tasks, int ntask) {
+    std::stable_sort(tasks, tasks + ntask, [](const EigTask& x, const EigTask& y) { return x.n > y.n; });
+}
+
+void launch_eig(const EigTask* tasks, const EigTask* host, int ntask, bool null_rule, int maxs, int* flags,
+                cudaStream_t st) {
+    const double nullrel = null_rule ? Tol::null : 0.0;
+    int ncl = 0;
+    size_t smem = 0, smem1 = 0;
+    for (int i = 0; i < ntask; ++i) {
+        if (eig_on_cluster(host[i].n)) {
+            ncl = i + 1;
+            smem = std::max(smem, eig_smem(host[i].n, JC));
+        } else {
+            smem1 = std::max(smem1, eig_smem(host[i].n, 1));
+        }
+    }
+    if (ncl > 0) {
+        ensure_smem_attr(reinterpret_cast<const void*>(k_eig_cl), JAC_SMEM);
+        count_launch();
+        k_eig_cl<<<ncl * JC, 256, smem, st>>>(tasks, nullrel, maxs, flags);
+    }
+    if (ncl < ntask) {
+        count_launch();
+        k_eig_one<<<ntask - ncl, 128, smem1, st>>>(tasks + ncl, nullrel, maxs, flags ? flags + ncl : nullptr);
+    }
+}
+
+void launch_jac_apply(const JacTask* tasks, const JacRows* rows, int nblocks, int nmax, bool f32, bool ident,
                       cudaStream_t st) {
     if (nblocks <= 0) return;
-    jac_attributes();
+    const size_t smem = (size_t)JAC_APPLY_ROWS * (nmax + (nmax & 1)) * (f32 ? 4 : 8);
     count_launch();
-    if (f32) k_jac_apply<float><<<nblocks, 32, smem, st>>>(tasks, rows, sweep);
-    else k_jac_apply<double><<<nblocks, 32, smem, st>>>(tasks, rows, sweep);
+    if (f32) {
+        ensure_smem_attr(reinterpret_cast<const void*>(k_jac_apply<float>), JAC_SMEM);
+        k_jac_apply<float><<<nblocks, 32 * JAC_APPLY_ROWS, smem, st>>>(tasks, rows, ident ? 1 : 0);
+    } else {
+        ensure_smem_attr(reinterpret_cast<const void*>(k_jac_apply<double>), JAC_SMEM);
+        k_jac_apply<double><<<nblocks, 32 * JAC_APPLY_ROWS, smem, st>>>(tasks, rows, ident ? 1 : 0);
+    }
 }
 
 }  // namespace mpspt

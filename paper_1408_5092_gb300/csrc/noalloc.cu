@@ -83,15 +83,21 @@ extern "C" mpspt_status mpspt_eigh_batched_noalloc(int device, void* stream, int
     double* work = base + kTaskDoubles;
     size_t o = 0, ow = 0;
     for (int i = 0; i < batch; ++i) {
-        tasks[i] = {work + o, V + o, w + ow, n[i], 0};
-        o += (size_t)n[i] * n[i];
+        const size_t nn = (size_t)n[i] * n[i];
+        double* a = const_cast<double*>(A) + o;
+        if (mpspt::eig_in_place(n[i])) {   // a work copy only where the solver cannot hold the matrix on chip
+            if (cudaMemcpyAsync(work + o, a, nn * sizeof(double), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+                return MPSPT_ERR_CUDA;
+            a = work + o;
+        }
+        tasks[i] = {a, V + o, w + ow, n[i], 0};
+        o += nn;
         ow += (size_t)n[i];
     }
-    if (cudaMemcpyAsync(work, A, tot * sizeof(double), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-        return MPSPT_ERR_CUDA;
+    mpspt::order_eig_tasks(tasks, batch);
     if (cudaMemcpyAsync(base, tasks, batch * sizeof(mpspt::EigTask), cudaMemcpyHostToDevice, st) != cudaSuccess)
         return MPSPT_ERR_CUDA;
-    mpspt::launch_eig(reinterpret_cast<const mpspt::EigTask*>(base), batch, st);
+    mpspt::launch_eig(reinterpret_cast<const mpspt::EigTask*>(base), tasks, batch, false, mpspt::kEighSweeps, nullptr, st);
     if (cudaGetLastError() != cudaSuccess) return MPSPT_ERR_CUDA;
     return MPSPT_OK;
 }

@@ -116,18 +116,27 @@ void GemmPlan::units(int tile, std::vector<GemmBlk>& gb, std::vector<unsigned>& 
     *ticks = tk;
 }
 
-namespace {
 // 32 x 32 units when there are enough of them to keep every SM busy for two
 // rounds of its eight (fewer unit starts, half the operand traffic), the
 // narrow 16 x 16 ones below that.  Both give the same bits and nearly the same
 // time near the line (the float64 pipe bounds both); in the M = 256 sweep the
 // tuner takes 32 x 32 for a third of the launches.
-int dgemm_tile(const GemmPlan& g) {
+int GemmPlan::tile_rule() const {
     size_t n = 0;
-    for (const auto& b : g.blocks) n += (size_t)((b.m + 31) / 32) * ((b.n + 31) / 32);
+    for (const auto& b : blocks) n += (size_t)((b.m + 31) / 32) * ((b.n + 31) / 32);
     return n >= 2432 ? 32 : 16;
 }
 
+void GemmPlan::workspace(size_t part_elems, size_t ticks, cudaStream_t st) {
+    if (part_elems) dpart.ensure(part_elems * sizeof(double) + 16, st);
+    if (ticks) {
+        const size_t had = dtick.bytes();
+        dtick.ensure(ticks * sizeof(unsigned), st);
+        if (dtick.bytes() != had) MPSPT_CUDA(cudaMemsetAsync(dtick.get(), 0, dtick.bytes(), st));
+    }
+}
+
+namespace {
 // longest K-list first: the persistent kernels hand out tasks in strides of
 // the grid, so this order balances the CTAs (each output tile has exactly
 // one task, so the order does not change any result)
@@ -171,15 +180,10 @@ void GemmPlan::upload(cudaStream_t st) {
     if (kind == GEMM_F64) {
         size_t tk = 0;
         std::vector<long long> cm;
-        tile64 = tuner && !blocks.empty() ? (tm == 32 ? 32 : 16) : dgemm_tile(*this);
+        tile64 = tuner && !blocks.empty() ? (tm == 32 ? 32 : 16) : tile_rule();
         units(tile64, gblk, unit_blk, &cm, &pe, &tk);
         for (size_t i = 0; i < gblk.size(); ++i) gblk[i].cmap = cm[i] >= 0 ? cbase + cm[i] : nullptr;
-        if (pe) dpart.ensure(pe * sizeof(double) + 16, st);
-        if (tk) {   // the kernel leaves the counters at zero; new ones are set here
-            const size_t had = dtick.bytes();
-            dtick.ensure(tk * sizeof(unsigned), st);
-            if (dtick.bytes() != had) MPSPT_CUDA(cudaMemsetAsync(dtick.get(), 0, dtick.bytes(), st));
-        }
+        workspace(pe, tk, st);
         mpspt::upload(dgblk, gblk, st);
         mpspt::upload(dunit, unit_blk, st);
     } else {

@@ -92,6 +92,9 @@ struct GemmPlan {
     DBuf dgblk, dunit, dtick;
     // block and unit lists for a tile of 16 or 32 (no map pointers yet; cm, if
     // given: each block's map offset); partial-tile elements and split tiles
+    int tile_rule() const;
+    // partial-tile and counter space (the kernel leaves the counters at zero)
+    void workspace(size_t part_elems, size_t ticks, cudaStream_t st);
     void units(int tile, std::vector<GemmBlk>& gb, std::vector<unsigned>& ub, std::vector<long long>* cm,
                size_t* part_elems, size_t* ticks) const;
     void clear() {
