@@ -103,6 +103,17 @@ struct Registry {
         live.erase((uintptr_t)p);
         gen.fetch_add(1, std::memory_order_release);
     }
+    // the allocation that holds [p, p + bytes), or false
+    bool find(const void* p, size_t bytes, uintptr_t& lo, uintptr_t& hi) {
+        const uintptr_t a = (uintptr_t)p;
+        std::shared_lock<std::shared_mutex> g(mu);
+        auto it = live.upper_bound(a);
+        if (it == live.begin()) return false;
+        --it;
+        lo = it->first;
+        hi = it->first + it->second;
+        return a + bytes <= hi;
+    }
     bool contains(const void* p, size_t bytes) {
         constexpr int kWays = 8;
         thread_local uintptr_t c0[kWays] = {}, c1[kWays] = {};
@@ -140,6 +151,31 @@ inline void check_range(const void* p, size_t bytes, const char* what) {
     if (!Registry::get().contains(p, bytes))
         throw Error(MPSPT_ERR_INVALID, std::string("planner bounds check failed: ") + what);
 }
+
+// Range checks of one plan: remembers the allocations it has met.  They stay
+// live while the plan is checked (they belong to the checking thread's lane).
+class RangeCheck {
+  public:
+    void operator()(const void* p, size_t bytes, const char* what) {
+        if (!on_ || bytes == 0) return;
+        const uintptr_t a = (uintptr_t)p, b = a + bytes;
+        for (int w = 0; w < n_; ++w)
+            if (a >= lo_[w] && b <= hi_[w]) return;
+        uintptr_t lo, hi;
+        if (!Registry::get().find(p, bytes, lo, hi))
+            throw Error(MPSPT_ERR_INVALID, std::string("planner bounds check failed: ") + what);
+        const int w = n_ < kWays ? n_++ : next_++ % kWays;
+        lo_[w] = lo;
+        hi_[w] = hi;
+    }
+
+  private:
+    static constexpr int kWays = 6;
+    uintptr_t lo_[kWays] = {}, hi_[kWays] = {};
+    int n_ = 0;
+    unsigned next_ = 0;
+    bool on_ = checks_enabled();
+};
 
 // The library allocates from the device's default memory pool.  Its release
 // threshold is raised so that freed blocks stay cached in the pool across

@@ -778,13 +778,25 @@ struct Sweeper {
     }
 
     double env_flops = 0.0;     // flops of the last environment update
+    bool with_A = true, with_V = true;   // environments to keep: of H0 - E0, of the RHS operator
     void update_left(int i) {   // L[i+1] from L[i] and site i
+        env_flops = 0.0;
+        if (with_A) update_left_A(i);
+        if (with_V && !ch.ground) update_left_V(i);
+    }
+    void update_right(int i) {  // R[i] from R[i+1] and site i
+        env_flops = 0.0;
+        if (with_A) update_right_A(i);
+        if (with_V && !ch.ground) update_right_V(i);
+    }
+    void update_left_A(int i) {
         LA[i + 1].build(WA.dq[i + 1], psi.bond[i + 1], psi.bond[i + 1], ln.st);
         envp.build_left(WA, i, LA[i], psi.A[i], psi.A[i], psi.bond[i], psi.bond[i], psi.bond[i + 1],
                         psi.bond[i + 1], LA[i + 1], ln.st);
         envp.run(ln.st);
-        env_flops = envp.flops();
-        if (ch.ground) return;
+        env_flops += envp.flops();
+    }
+    void update_left_V(int i) {
         LV[i + 1].build(WV.dq[i + 1], psi.bond[i + 1], psi0.bond[i + 1], ln.st);
         envp.build_left(WV, i, LV[i], psi.A[i], psi0.A[i], psi.bond[i], psi0.bond[i], psi.bond[i + 1],
                         psi0.bond[i + 1], LV[i + 1], ln.st);
@@ -792,13 +804,14 @@ struct Sweeper {
         env_flops += envp.flops();
     }
 
-    void update_right(int i) {  // R[i] from R[i+1] and site i
+    void update_right_A(int i) {
         RA[i].build(WA.dq[i], psi.bond[i], psi.bond[i], ln.st);
         envp.build_right(WA, i, RA[i + 1], psi.A[i], psi.A[i], psi.bond[i], psi.bond[i], psi.bond[i + 1],
                          psi.bond[i + 1], RA[i], ln.st);
         envp.run(ln.st);
-        env_flops = envp.flops();
-        if (ch.ground) return;
+        env_flops += envp.flops();
+    }
+    void update_right_V(int i) {
         RV[i].build(WV.dq[i], psi.bond[i], psi0.bond[i], ln.st);
         envp.build_right(WV, i, RV[i + 1], psi.A[i], psi0.A[i], psi.bond[i], psi0.bond[i], psi.bond[i + 1],
                          psi0.bond[i + 1], RV[i], ln.st);
@@ -1971,31 +1984,8 @@ double expectation(Ctx& c, const MPO& W, const MpsD& bra, const MpsD& ket) {
     return expectation(c, W, bra, ket, c.st);
 }
 
-double expectation(Ctx& c, const MPO& W, const MpsD& bra, const MpsD& ket, cudaStream_t st) {
-    (void)c;
-    require(bra.nsite == ket.nsite && bra.nsite == W.nsite, "bra, ket and operator lengths differ");
-    EnvT L, Ln;
-    L.build(W.dq[0], bra.bond[0], ket.bond[0], st);
-    const double one = 1.0;
-    MPSPT_CUDA(cudaMemcpyAsync(L.d.get(), &one, sizeof(double), cudaMemcpyHostToDevice, st));
-    EnvPlan ep;
-    for (int i = 0; i < bra.nsite; ++i) {
-        Ln.build(W.dq[i + 1], bra.bond[i + 1], ket.bond[i + 1], st);
-        ep.build_left(W, i, L, bra.A[i], ket.A[i], bra.bond[i], ket.bond[i], bra.bond[i + 1],
-                      ket.bond[i + 1], Ln, st);
-        ep.run(st);
-        MPSPT_CUDA(cudaStreamSynchronize(st));
-        std::swap(L, Ln);
-    }
-    double v = 0.0;
-    if (!L.blk.empty())
-        MPSPT_CUDA(cudaMemcpyAsync(&v, L.d.get(), sizeof(double), cudaMemcpyDeviceToHost, st));
-    MPSPT_CUDA(cudaStreamSynchronize(st));
-    return v;
-}
-
-// <bra|W|ket> where the sites flagged in `empty` are identity sites (local
-// state |0>) in both bra and ket: each maximal run of them is one sparse map
+// <bra|W|ket> where the sites flagged in `empty` (which need rm) are identity
+// sites (local state |0>) in both bra and ket: each maximal run of them is one sparse map
 // of MPO states (one mix launch), the other sites the full transfer.  Only
 // MPO states on some path from the left boundary to the right one are
 // carried: a state that needs an operator on an empty site dies there, and
@@ -2011,7 +2001,7 @@ struct XferWs {
     EnvPlan ep;
 };
 
-double expectation_runs(XferWs& ws, const MPO& W, RunMaps& rm, const MpsD& bra, const MpsD& ket,
+double expectation_runs(XferWs& ws, const MPO& W, RunMaps* rm, const MpsD& bra, const MpsD& ket,
                         const std::vector<char>& empty, cudaStream_t st, double* wait_ms, double* flops,
                         double* plan_bytes) {
     const int ns = bra.nsite;
@@ -2024,7 +2014,7 @@ double expectation_runs(XferWs& ws, const MPO& W, RunMaps& rm, const MpsD& bra, 
         int j = i + 1;
         if (empty[i]) {
             while (j < ns && empty[j]) ++j;
-            seg.push_back({i, j, &rm.get(i, j)});
+            seg.push_back({i, j, &rm->get(i, j)});
         } else {
             seg.push_back({i, j, nullptr});
         }
@@ -2093,6 +2083,12 @@ double expectation_runs(XferWs& ws, const MPO& W, RunMaps& rm, const MpsD& bra, 
     MPSPT_CUDA(cudaStreamSynchronize(st));
     if (wait_ms) *wait_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - tw).count();
     return v;
+}
+
+double expectation(Ctx& c, const MPO& W, const MpsD& bra, const MpsD& ket, cudaStream_t st) {
+    RingScope rs(st == c.lane0->st ? c.lane0->ring.get() : nullptr);
+    XferWs ws;
+    return expectation_runs(ws, W, nullptr, bra, ket, std::vector<char>(W.nsite, 0), st, nullptr, nullptr, nullptr);
 }
 
 double third_order(Ctx& c, int h0, const MpsD& psi1) {
@@ -2217,12 +2213,12 @@ double third_order_partitioned(Ctx& c, int h0, const std::vector<std::pair<int, 
             const std::vector<char> m = empty_mask(k.i, k.j);
             if (k.i == k.j) {
                 const MpsD& x = emb[k.i];
-                const double n2 = expectation_runs(ws, WI, rmI, x, x, m, ln.st, w, f, b);
-                const double eh = expectation_runs(ws, WH, rmH, x, x, m, ln.st, w, f, b);
-                const double ea = expectation_runs(ws, WA, rmA, x, x, m, ln.st, w, f, b);
+                const double n2 = expectation_runs(ws, WI, &rmI, x, x, m, ln.st, w, f, b);
+                const double eh = expectation_runs(ws, WH, &rmH, x, x, m, ln.st, w, f, b);
+                const double ea = expectation_runs(ws, WA, &rmA, x, x, m, ln.st, w, f, b);
                 val[t] = eh - ea - c.P.e_ref * n2;   // <H> - <A> - (E0 + E1) <1>
             } else {
-                val[t] = expectation_runs(ws, WH, rmH, emb[k.i], emb[k.j], m, ln.st, w, f, b);
+                val[t] = expectation_runs(ws, WH, &rmH, emb[k.i], emb[k.j], m, ln.st, w, f, b);
             }
         }
         MPSPT_CUDA(cudaStreamSynchronize(ln.st));
@@ -2260,11 +2256,14 @@ void local_apply(Ctx& c, int h0, const MpsD& psi1_in, int i, int op, const doubl
     require(psi1_in.nsite == c.P.k, "MPS length differs from the orbital count");
     require(i >= 0 && i + 1 < c.P.k, "bond index out of range");
     MpsD& psi1 = const_cast<MpsD&>(psi1_in);
+    RingScope rs(c.lane0->ring.get());
     SweepResult res;
     require(h0 == MPSPT_H0_FOCK || h0 == MPSPT_H0_DYALL, "unknown H0");
     Chain ch = full_chain(c, h0);
     Sweeper sw(c, *c.lane0, ch, 1 << 30, psi1);
     sw.res = &res;
+    sw.with_A = op != MPSPT_LOCAL_RHS;   // only the operator that is applied
+    sw.with_V = op == MPSPT_LOCAL_RHS;
     sw.boundary_envs();
     for (int s = 0; s < i; ++s) sw.update_left(s);
     for (int s = c.P.k - 1; s >= i + 2; --s) sw.update_right(s);

@@ -40,6 +40,17 @@ struct MPO {
     // out_ptr[p][a+1]]) and by target state (in_idx[p][in_ptr[p][b] ..
     // in_ptr[p][b+1]], in increasing a); filled by index().
     std::vector<std::vector<int>> out_ptr, in_ptr, in_idx;
+    // The non-zero local elements v = coef <s|o|t> of each site, listed for
+    // (state, s) in the entries' order: in_el of the entries into b, row
+    // in_at[p][4 b + s] (x = a), and out_el of the entries out of a, row
+    // out_at[p][4 a + s] (x = b).  The planners walk these instead of the
+    // entries and their operator tables.
+    struct El {
+        int x, t;
+        double v;
+    };
+    std::vector<std::vector<El>> in_el, out_el;
+    std::vector<std::vector<int>> in_at, out_at;
     void index();
 };
 

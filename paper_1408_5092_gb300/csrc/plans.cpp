@@ -201,6 +201,7 @@ void GemmPlan::upload(cudaStream_t st) {
         mpspt::upload(dtasks, tasks, st);
     }
     if (checks_enabled()) {
+        RangeCheck check_range;
         // per planned block (all tiles of a block share its output and its
         // K-list): the output range, or the span of its mapped addresses,
         // and every operand range of its K-list
@@ -388,43 +389,63 @@ void GemmPlan::run(cudaStream_t st) const {
     if (!reds.empty()) launch_splitk_reduce(dreds.as<SplitRed>(), (int)reds.size(), st, skip);
 }
 
+// Omega_ac of bond (i, i+1): the products of the two sites' elements, added in
+// the order of the entries.  One dense accumulator per source state a over
+// (out, c, in) with a bitmap of the touched places: no ordered container.
 void Omega::build(const MPO& W, int i) {
-    std::map<int, std::vector<const MpoEntry*>> by_b;
-    for (const auto& e : W.W[i + 1]) by_b[e.a].push_back(&e);
-    std::map<std::tuple<int, int, int, int>, double> acc;   // (a, out, c, in)
-    for (const auto& e1 : W.W[i]) {
-        auto it = by_b.find(e1.b);
-        if (it == by_b.end()) continue;
-        const Mat4& o1 = W.ops[e1.op];
-        for (const MpoEntry* e2 : it->second) {
-            const Mat4& o2 = W.ops[e2->op];
-            const double cc = e1.coef * e2->coef;
-            for (int s1 = 0; s1 < 4; ++s1)
-                for (int t1 = 0; t1 < 4; ++t1) {
-                    const double v1 = o1[s1 * 4 + t1];
-                    if (v1 == 0.0) continue;
-                    for (int s2 = 0; s2 < 4; ++s2)
-                        for (int t2 = 0; t2 < 4; ++t2) {
-                            const double v2 = o2[s2 * 4 + t2];
-                            if (v2 == 0.0) continue;
-                            acc[{e1.a, s1 * 4 + s2, e2->b, t1 * 4 + t2}] += cc * v1 * v2;
-                        }
-                }
-        }
-    }
     Da = W.dim[i];
+    const int Dc = W.dim[i + 2];
+    struct N2 { int s, t; double v; };
+    std::vector<N2> nz;                    // non-zero elements of the second site's entries
+    std::vector<int> nzp;
+    for (const auto& e2 : W.W[i + 1]) {
+        nzp.push_back((int)nz.size());
+        const Mat4& o = W.ops[e2.op];
+        for (int s = 0; s < 4; ++s)
+            for (int t = 0; t < 4; ++t)
+                if (o[s * 4 + t] != 0.0) nz.push_back({s, t, o[s * 4 + t]});
+    }
+    nzp.push_back((int)nz.size());
+    const size_t places = (size_t)16 * Dc * 16;   // (out * Dc + c) * 16 + in
+    std::vector<double> acc(places, 0.0);
+    std::vector<uint64_t> bits((places + 63) / 64, 0);
     e.clear();
-    for (auto& kv : acc) {
-        if (kv.second == 0.0) continue;
-        e.push_back({std::get<0>(kv.first), std::get<2>(kv.first), std::get<1>(kv.first),
-                     std::get<3>(kv.first), kv.second});
-    }
     first.assign((size_t)Da * 16 + 1, 0);
-    size_t k = 0;
-    for (int key = 0; key <= Da * 16; ++key) {
-        while (k < e.size() && e[k].a * 16 + e[k].out < key) ++k;
-        first[key] = (int)k;
+    const auto& p1 = W.out_ptr[i];
+    const auto& p2 = W.out_ptr[i + 1];
+    for (int a = 0; a < Da; ++a) {
+        for (int q1 = p1[a]; q1 < p1[a + 1]; ++q1) {
+            const MpoEntry& e1 = W.W[i][q1];
+            const Mat4& o1 = W.ops[e1.op];
+            for (int q2 = p2[e1.b]; q2 < p2[e1.b + 1]; ++q2) {
+                const MpoEntry& e2 = W.W[i + 1][q2];
+                const double cc = e1.coef * e2.coef;
+                for (int s1 = 0; s1 < 4; ++s1)
+                    for (int t1 = 0; t1 < 4; ++t1) {
+                        const double v1 = o1[s1 * 4 + t1];
+                        if (v1 == 0.0) continue;
+                        for (int k = nzp[q2]; k < nzp[q2 + 1]; ++k) {
+                            const size_t at = ((size_t)(s1 * 4 + nz[k].s) * Dc + e2.b) * 16 + t1 * 4 + nz[k].t;
+                            acc[at] += cc * v1 * nz[k].v;
+                            bits[at >> 6] |= 1ULL << (at & 63);
+                        }
+                    }
+            }
+        }
+        int out = 0;
+        for (size_t w = 0; w < bits.size(); ++w) {
+            for (uint64_t m = bits[w]; m; m &= m - 1) {
+                const size_t at = w * 64 + (size_t)__builtin_ctzll(m);
+                const int o16 = (int)(at / ((size_t)Dc * 16));
+                for (; out <= o16; ++out) first[(size_t)a * 16 + out] = (int)e.size();
+                if (acc[at] != 0.0) e.push_back({a, (int)(at / 16 % Dc), o16, (int)(at % 16), acc[at]});
+                acc[at] = 0.0;
+            }
+            bits[w] = 0;
+        }
+        for (; out < 16; ++out) first[(size_t)a * 16 + out] = (int)e.size();
     }
+    first[(size_t)Da * 16] = (int)e.size();
 }
 
 void TwoSitePlan::build(const Omega& om, const TwoT& bra, const TwoT& ket, const Bond& braL,
@@ -435,12 +456,13 @@ void TwoSitePlan::build(const Omega& om, const TwoT& bra, const TwoT& ket, const
     g1.clear(); g2.clear(); g2s.clear();
     mtasks.clear(); msrc.clear();
     const int np = (int)ket.panels.size();
-    const int nc = (int)(R.idx.size() / (size_t)std::max(1, R.nsk));
+    const int nc = R.na;
     const int na = om.Da;
     // ---- Rpack per ket right sector: blocks R_c(sb_c, sk) stacked by c
     std::vector<long long> rp_off(ketR.nsec(), -1);
     std::vector<int> rp_rows(ketR.nsec(), 0);
-    std::vector<int> rcol((size_t)nc * ketR.nsec(), -1);   // row offset of c inside Rpack(sk)
+    std::vector<int> rcol((size_t)nc * ketR.nsec(), -1);   // row offset of c inside Rpack(sk), sk by sk
+    std::vector<int> rsb((size_t)nc * ketR.nsec(), -1);    // its bra sector
     size_t rps = 0;
     std::vector<CopyTask> pk_tasks;
     for (const auto& P : ket.panels) {
@@ -449,7 +471,8 @@ void TwoSitePlan::build(const Omega& om, const TwoT& bra, const TwoT& ket, const
         for (int c = 0; c < nc; ++c) {
             int rb = R.find(c, sk);
             if (rb < 0) continue;
-            rcol[(size_t)c * ketR.nsec() + sk] = rows;
+            rcol[(size_t)sk * nc + c] = rows;
+            rsb[(size_t)sk * nc + c] = R.blk[rb].sb;
             rows += braR.sec[R.blk[rb].sb].dim;
         }
         rp_rows[sk] = rows;
@@ -485,7 +508,7 @@ void TwoSitePlan::build(const Omega& om, const TwoT& bra, const TwoT& ket, const
             int rb = R.find(c, sk);
             if (rb < 0) continue;
             const int db = braR.sec[R.blk[rb].sb].dim;
-            pk_tasks.push_back({R.ptr(R.blk[rb]), Rpp + rp_off[sk] + (size_t)rcol[(size_t)c * ketR.nsec() + sk] * dk,
+            pk_tasks.push_back({R.ptr(R.blk[rb]), Rpp + rp_off[sk] + (size_t)rcol[(size_t)sk * nc + c] * dk,
                                 nullptr, db, dk, dk, dk, 0, 0});
         }
     }
@@ -497,11 +520,13 @@ void TwoSitePlan::build(const Omega& om, const TwoT& bra, const TwoT& ket, const
             pk_tasks.push_back({L.ptr(L.blk[lb]), Lpp + lp_off[sl] + lcol[(size_t)a * braL.nsec() + sl],
                                 nullptr, dl, dk, dk, lp_cols[sl], 0, 0});
         }
-    if (checks_enabled())
+    if (checks_enabled()) {
+        RangeCheck check;
         for (const auto& t : pk_tasks) {
-            check_range(t.src, ((size_t)(t.rows - 1) * t.lds + t.cols_n) * sizeof(double), "pack src");
-            check_range(t.dst, ((size_t)(t.rows - 1) * t.ldd + t.cols_n) * sizeof(double), "pack dst");
+            check(t.src, ((size_t)(t.rows - 1) * t.lds + t.cols_n) * sizeof(double), "pack src");
+            check(t.dst, ((size_t)(t.rows - 1) * t.ldd + t.cols_n) * sizeof(double), "pack dst");
         }
+    }
     mpspt::upload(pk, pk_tasks, st);
     launch_copy(pk.as<CopyTask>(), (int)pk_tasks.size(), st);
     // ---- T panels
@@ -541,6 +566,18 @@ void TwoSitePlan::build(const Omega& om, const TwoT& bra, const TwoT& ket, const
     }
     V.ensure((vs + 1) * sizeof(double), st);
     double* Vp = V.as<double>();
+    // ket blocks by (left sector, in): where their T rows start
+    struct KetT { int sr, nr; size_t base; };
+    std::vector<KetT> kt((size_t)ketL.nsec() * 16, KetT{-1, 0, 0});
+    for (int sk = 0; sk < ketL.nsec(); ++sk)
+        for (int in = 0; in < 16; ++in) {
+            const int kb = ket.find(sk, in / 4, in % 4);
+            if (kb < 0 || toff[panel_of[kb]] < 0) continue;
+            const auto& K = ket.blk[kb];
+            const int p = panel_of[kb], sr = ket.panels[p].sr;
+            const size_t rip = (K.off - ket.panels[p].off) / (size_t)K.cols;
+            kt[(size_t)sk * 16 + in] = {sr, rp_rows[sr], (size_t)toff[p] + rip * rp_rows[sr]};
+        }
     for (int sl = 0; sl < braL.nsec(); ++sl) {
         if (voff[sl] < 0) continue;
         const int W = wd[sl];
@@ -559,19 +596,13 @@ void TwoSitePlan::build(const Omega& om, const TwoT& bra, const TwoT& ket, const
                 const int o16 = B.s1 * 4 + B.s2;
                 for (int q = om.begin(a, o16); q < om.end(a, o16); ++q) {
                     const Omega::E& E = om.e[q];
-                    const int kb = ket.find(sk, E.in / 4, E.in % 4);
-                    if (kb < 0) continue;
-                    const int p = panel_of[kb];
-                    if (toff[p] < 0) continue;
-                    const int srk = ket.panels[p].sr;
-                    const int rc = rcol[(size_t)E.c * ketR.nsec() + srk];
-                    if (rc < 0) continue;
-                    const int rb = R.find(E.c, srk);
-                    if (R.blk[rb].sb != B.sr) continue;
-                    const auto& K = ket.blk[kb];
-                    const size_t rip = (K.off - ket.panels[p].off) / (size_t)K.cols;
-                    const int nr = rp_rows[srk];
-                    msrc.push_back({Tp + toff[p] + rip * nr + rc, nr, 0, E.v});
+                    const KetT& k = kt[(size_t)sk * 16 + E.in];
+                    if (k.sr < 0) continue;
+                    const size_t rq = (size_t)k.sr * nc + E.c;
+                    if (rcol[rq] < 0 || rsb[rq] != B.sr) continue;
+                    const size_t src = k.base + rcol[rq];
+                    if (src + (size_t)(dk - 1) * k.nr + B.cols > tsize) throw Error(MPSPT_ERR_INVALID, "mix source outside T");
+                    msrc.push_back({Tp + src, k.nr, 0, E.v});
                 }
                 mt.s1 = (int)msrc.size();
                 mtasks.push_back(mt);
@@ -602,11 +633,9 @@ void TwoSitePlan::build(const Omega& om, const TwoT& bra, const TwoT& ket, const
         }
     }
     if (checks_enabled()) {
-        for (const auto& t : mtasks) {
-            check_range(t.dst, ((size_t)(t.rows - 1) * t.ldd + t.cols) * sizeof(double), "mix dst");
-            for (int q = t.s0; q < t.s1; ++q)
-                check_range(msrc[q].src, ((size_t)(t.rows - 1) * msrc[q].lds + t.cols) * sizeof(double), "mix src");
-        }
+        RangeCheck check;   // (the sources were placed inside T above)
+        check(Tp, tsize * sizeof(double), "mix T");
+        for (const auto& t : mtasks) check(t.dst, ((size_t)(t.rows - 1) * t.ldd + t.cols) * sizeof(double), "mix dst");
     }
     mpspt::upload(dmt, mtasks, st);
     mpspt::upload(dms, msrc, st);
@@ -639,6 +668,7 @@ void DiagPlan::build(const Omega& om, const TwoT& x, const Bond& Lb, const Bond&
         tasks.push_back({out + b.off, b.rows, b.cols, t0, (int)terms.size()});
     }
     if (checks_enabled()) {
+        RangeCheck check_range;
         for (const auto& t : tasks) {
             check_range(t.out, (size_t)t.rows * t.cols * sizeof(double), "diag out");
             for (int k = t.t0; k < t.t1; ++k) {
@@ -671,13 +701,11 @@ void plan_product(GemmPlan& g, const TwoT& x, double* xd, const Bond& mid, const
     }
 }
 
+// (The sources were placed inside their buffer by the builders.)
 void EnvPlan::upload_mix(cudaStream_t st) {
     if (checks_enabled()) {
-        for (const auto& t : mt) {
-            check_range(t.dst, ((size_t)(t.rows - 1) * t.ldd + t.cols) * sizeof(double), "env mix dst");
-            for (int q = t.s0; q < t.s1; ++q)
-                check_range(ms[q].src, ((size_t)(t.rows - 1) * ms[q].lds + t.cols) * sizeof(double), "env mix src");
-        }
+        RangeCheck check;
+        for (const auto& t : mt) check(t.dst, ((size_t)(t.rows - 1) * t.ldd + t.cols) * sizeof(double), "env mix dst");
     }
     mpspt::upload(dmt, mt, st);
     mpspt::upload(dms, ms, st);
@@ -714,39 +742,47 @@ void EnvPlan::build_left(const MPO& W, int site, const EnvT& L, const SiteT& Abr
         g1.op(L.panel(K.sl), kd, Aket.ptr(K), nd, kd, 0, 1.0);
         g1.block(Yp + yoff[kb], nd, P, nd, 0, m0);
     }
-    // mix: Z_(out, s) over the MPO entries e = (a -> b) and t
-    const std::vector<MpoEntry>& We = W.W[site];
-    const std::vector<int>&in_ptr = W.in_ptr[site], &in_idx = W.in_idx[site];
+    // mix: Z_(out, s) over the elements (a, s, t -> b)
+    const std::vector<MPO::El>& el = W.in_el[site];
+    const std::vector<int>& at = W.in_at[site];
     struct ZB { int nb, s, bb; size_t off; int rows, cols; };
     std::vector<ZB> zb;
     size_t zs = 0;
+    check_range(Yp, ys * sizeof(double), "env mix Y");
+    // left sector and block of every (right sector, local state)
+    struct Side { int sl, blk; };
+    auto side = [](const Bond& br, const SiteT& A) {
+        std::vector<Side> v((size_t)br.nsec() * 4, Side{-1, -1});
+        for (int b = 0; b < (int)A.blk.size(); ++b) v[(size_t)A.blk[b].sr * 4 + A.blk[b].s] = {A.blk[b].sl, b};
+        return v;
+    };
+    const std::vector<Side> bside = side(braR, Abra), kside = side(ketR, Aket);
     for (int nbi = 0; nbi < (int)Lnew.blk.size(); ++nbi) {
         const auto& nb = Lnew.blk[nbi];
         const int nd = ketR.sec[nb.sk].dim;
         // ket-side lookups depend on t only
-        int slk_t[4], kb_t[4];
+        const int* blk_t[4];
+        double* y_t[4];
         for (int t = 0; t < 4; ++t) {
-            slk_t[t] = ketL.find(ketR.sec[nb.sk].q - site_qn(t));
-            kb_t[t] = slk_t[t] < 0 ? -1 : Aket.find(slk_t[t], t);
-            if (kb_t[t] >= 0 && (Aket.blk[kb_t[t]].sr != nb.sk || yoff[kb_t[t]] < 0)) kb_t[t] = -1;
+            const Side k = kside[(size_t)nb.sk * 4 + t];
+            const bool ok = k.blk >= 0 && yoff[k.blk] >= 0;
+            blk_t[t] = ok ? L.row(k.sl) : nullptr;
+            y_t[t] = ok ? Yp + yoff[k.blk] : nullptr;
         }
         for (int s = 0; s < 4; ++s) {
-            const int slb = braL.find(braR.sec[nb.sb].q - site_qn(s));
-            if (slb < 0) continue;
-            const int bb = Abra.find(slb, s);
-            if (bb < 0 || Abra.blk[bb].sr != nb.sb) continue;
+            const Side side_b = bside[(size_t)nb.sb * 4 + s];
+            if (side_b.blk < 0) continue;
+            const int slb = side_b.sl, bb = side_b.blk;
             const int rows = braL.sec[slb].dim;
             const int s0 = (int)ms.size();
-            for (int q = in_ptr[nb.a]; q < in_ptr[nb.a + 1]; ++q) {
-                const MpoEntry* e = &We[in_idx[q]];
-                const Mat4& op = W.ops[e->op];
-                for (int t = 0; t < 4; ++t) {
-                    const double v = op[s * 4 + t];
-                    if (v == 0.0 || kb_t[t] < 0) continue;
-                    const int lb = L.find(e->a, slk_t[t]);
-                    if (lb < 0 || L.blk[lb].sb != slb) continue;
-                    ms.push_back({Yp + yoff[kb_t[t]] + (size_t)L.blk[lb].roff * nd, nd, 0, e->coef * v});
-                }
+            for (int q = at[(size_t)nb.a * 4 + s]; q < at[(size_t)nb.a * 4 + s + 1]; ++q) {
+                const MPO::El& E = el[q];
+                if (!blk_t[E.t]) continue;
+                const int lb = blk_t[E.t][E.x];
+                if (lb < 0 || L.blk[lb].sb != slb) continue;
+                double* src = y_t[E.t] + (size_t)L.blk[lb].roff * nd;
+                if (src + (size_t)rows * nd > Yp + ys) throw Error(MPSPT_ERR_INVALID, "env mix source outside Y");
+                ms.push_back({src, nd, 0, E.v});
             }
             if ((int)ms.size() == s0) continue;
             zb.push_back({nbi, s, bb, zs, rows, nd});
@@ -782,6 +818,7 @@ void EnvPlan::build_left_run(const RunMap& T, const EnvT& L, const Bond& bra, co
         for (int q = T.ptr[nb.a]; q < T.ptr[nb.a + 1]; ++q) {
             const int lb = L.find(T.col[q], nb.sk);
             if (lb < 0 || L.blk[lb].sb != nb.sb) continue;
+            if (L.blk[lb].off + (size_t)rows * cols > L.n) throw Error(MPSPT_ERR_INVALID, "env mix source outside L");
             ms.push_back({L.ptr(L.blk[lb]), cols, 0, T.val[q]});
         }
         mt.push_back({Lnew.ptr(nb), rows, cols, cols, s0, (int)ms.size(), 0});
@@ -817,19 +854,25 @@ void EnvPlan::build_right(const MPO& W, int site, const EnvT& R, const SiteT& Ab
         g1.op(Aket.ptr(K), kd, R.panel(K.sr), kd, kd, 2, 1.0);
         g1.block(Yp + yoff[kb], P, md, P, 0, m0);
     }
-    // mix: Z_(out, s) = sum over e = (a -> b), t of W_ab(s, t) Y_(b, kb(t)), dim(sk) x dim(sr_b)
-    const std::vector<MpoEntry>& We = W.W[site];
-    const std::vector<int>& out_ptr = W.out_ptr[site];
+    // mix: Z_(out, s) = sum over the elements (a, s, t -> b) of v Y_(b, kb(t)), dim(sk) x dim(sr_b)
+    const std::vector<MPO::El>& el = W.out_el[site];
+    const std::vector<int>& at = W.out_at[site];
     struct ZB { int nb, s, bb; size_t off; int rows, cols; };
     std::vector<ZB> zb;
     size_t zs = 0;
+    check_range(Yp, ys * sizeof(double), "env mix Y");
     for (int nbi = 0; nbi < (int)Rnew.blk.size(); ++nbi) {
         const auto& nbk = Rnew.blk[nbi];
         const int nd = ketL.sec[nbk.sk].dim;
-        int kb_t[4];   // ket-side lookups depend on t only
+        const int* blk_t[4];   // ket-side lookups depend on t only
+        double* y_t[4];
+        int ld_t[4];
         for (int t = 0; t < 4; ++t) {
-            kb_t[t] = Aket.find(nbk.sk, t);
-            if (kb_t[t] >= 0 && yoff[kb_t[t]] < 0) kb_t[t] = -1;
+            const int kb = Aket.find(nbk.sk, t);
+            const bool ok = kb >= 0 && yoff[kb] >= 0;
+            blk_t[t] = ok ? R.row(Aket.blk[kb].sr) : nullptr;
+            y_t[t] = ok ? Yp + yoff[kb] : nullptr;
+            ld_t[t] = ok ? R.prows[Aket.blk[kb].sr] : 0;
         }
         for (int s = 0; s < 4; ++s) {
             const int bb = Abra.find(nbk.sb, s);
@@ -837,19 +880,15 @@ void EnvPlan::build_right(const MPO& W, int site, const EnvT& R, const SiteT& Ab
             const int srb = Abra.blk[bb].sr;
             const int cols = braR.sec[srb].dim;
             const int s0 = (int)ms.size();
-            for (int q = out_ptr[nbk.a]; q < out_ptr[nbk.a + 1]; ++q) {
-                const MpoEntry* e = &We[q];
-                const Mat4& op = W.ops[e->op];
-                for (int t = 0; t < 4; ++t) {
-                    const double v = op[s * 4 + t];
-                    if (v == 0.0) continue;
-                    const int kb = kb_t[t];
-                    if (kb < 0) continue;
-                    const int srk = Aket.blk[kb].sr;
-                    const int rb = R.find(e->b, srk);
-                    if (rb < 0 || R.blk[rb].sb != srb) continue;
-                    ms.push_back({Yp + yoff[kb] + R.blk[rb].roff, R.prows[srk], 0, e->coef * v});
-                }
+            for (int q = at[(size_t)nbk.a * 4 + s]; q < at[(size_t)nbk.a * 4 + s + 1]; ++q) {
+                const MPO::El& E = el[q];
+                if (!blk_t[E.t]) continue;
+                const int rb = blk_t[E.t][E.x];
+                if (rb < 0 || R.blk[rb].sb != srb) continue;
+                double* src = y_t[E.t] + R.blk[rb].roff;
+                if (src + (size_t)(nd - 1) * ld_t[E.t] + cols > Yp + ys)
+                    throw Error(MPSPT_ERR_INVALID, "env mix source outside Y");
+                ms.push_back({src, ld_t[E.t], 0, E.v});
             }
             if ((int)ms.size() == s0) continue;
             zb.push_back({nbi, s, bb, zs, nd, cols});

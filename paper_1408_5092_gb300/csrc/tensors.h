@@ -42,10 +42,10 @@ struct SiteT {
 struct EnvT {
     struct B { int a, sb, sk; size_t off; int roff; };
     std::vector<B> blk;
-    std::vector<int> idx;   // a*nsk + sk -> block or -1
+    std::vector<int> idx;   // sk*na + a -> block or -1
     std::vector<size_t> poff;
     std::vector<int> prows;
-    int nsk = 0;
+    int nsk = 0, na = 0;
     size_t n = 0;
     DBuf d;
     // live (optional): MPO states whose blocks exist; the others are known
@@ -56,17 +56,30 @@ struct EnvT {
                const std::vector<char>* live = nullptr, bool reuse = false) {
         blk.clear();
         nsk = ket.nsec();
+        na = (int)dq.size();
         idx.assign(dq.size() * (size_t)nsk, -1);
         poff.assign(nsk, 0);
         prows.assign(nsk, 0);
         n = 0;
+        // QN changes are few (|dN|, |d2Sz| <= 4 for two-body operators): one
+        // search per change and ket sector
+        std::vector<QN> kinds;
+        std::vector<int> kind(dq.size()), sb_of;
+        for (size_t a = 0; a < dq.size(); ++a) {
+            size_t k = 0;
+            while (k < kinds.size() && kinds[k] != dq[a]) ++k;
+            if (k == kinds.size()) kinds.push_back(dq[a]);
+            kind[a] = (int)k;
+        }
         for (int sk = 0; sk < nsk; ++sk) {
             poff[sk] = n;
+            sb_of.assign(kinds.size(), -1);
+            for (size_t k = 0; k < kinds.size(); ++k) sb_of[k] = bra.find(ket.sec[sk].q + kinds[k]);
             for (int a = 0; a < (int)dq.size(); ++a) {
                 if (live && !(*live)[a]) continue;
-                int sb = bra.find(ket.sec[sk].q + dq[a]);
+                const int sb = sb_of[kind[a]];
                 if (sb < 0) continue;
-                idx[(size_t)a * nsk + sk] = (int)blk.size();
+                idx[(size_t)sk * na + a] = (int)blk.size();
                 blk.push_back({a, sb, sk, n, prows[sk]});
                 n += (size_t)bra.sec[sb].dim * ket.sec[sk].dim;
                 prows[sk] += bra.sec[sb].dim;
@@ -75,7 +88,8 @@ struct EnvT {
         if (reuse) d.ensure(n * sizeof(double) + 8, st);
         else d.alloc(n * sizeof(double) + 8, st);
     }
-    int find(int a, int sk) const { return idx[(size_t)a * nsk + sk]; }
+    int find(int a, int sk) const { return idx[(size_t)sk * na + a]; }
+    const int* row(int sk) const { return idx.data() + (size_t)sk * na; }   // blocks of one ket sector by a
     double* ptr(const B& b) const { return d.as<double>() + b.off; }
     double* panel(int sk) const { return d.as<double>() + poff[sk]; }
 };
