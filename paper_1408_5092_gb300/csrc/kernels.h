@@ -227,11 +227,22 @@ struct BlockRef {      // one QN block of a two-site vector
     int pad;
 };
 constexpr int MLP_NF = 16;   // features per block
-void mlp_gemm(int M, int N, int K, const float* A, int lda, bool ta, const float* B, int ldb, bool tb,
-              float* C, int ldc, const float* bias, const float* mask, int epi, cudaStream_t st);
 void mlp_gemm_bf16w(int M, int N, int K, const float* A, int lda, bool ta, const void* B, int ldb, bool tb,
                     float* C, int ldc, const float* bias, const float* mask, int epi, cudaStream_t st);
-void mlp_colsum(int M, int N, const float* A, float* out, cudaStream_t st);
+// Weight gradient gW (M x N) = dY^T X over K samples and bias gradient gb (M) =
+// column sums of dY.  With mlp_wgrad_pieces(K) > 1 the pieces go to part
+// (pieces * (M N + M) floats) and mlp_wgrad_sum adds them.
+int mlp_wgrad_pieces(int K);
+void mlp_wgrad(int M, int N, int K, const float* dY, const float* X, float* gW, float* gb, float* part, cudaStream_t st);
+struct MlpSums {
+    struct L {
+        const float* part;
+        float *gW, *gb;
+        int wn, bn, pieces;
+    } l[3];
+    int count;
+};
+void mlp_wgrad_sum(const MlpSums& s, cudaStream_t st);
 void mlp_mse(int B, int N, const float* Y, const float* T, float* dY, float* rowloss, cudaStream_t st);
 void mlp_adam(int n, float* w, const float* g, float* m, float* v, void* wb, float lr, int step, cudaStream_t st);
 void mlp_to_bf16(int n, const float* w, void* wb, cudaStream_t st);

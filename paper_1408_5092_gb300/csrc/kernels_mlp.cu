@@ -4,7 +4,18 @@
 //
 // One tiled GEMM kernel covers every product of training and inference:
 //   C[m][n] = sum_k opA(m, k) * opB(k, n)  (+ bias[n]) (relu / relu-mask)
-// with A, B float32 or bfloat16 and optional transposes.
+// with A, B float32 or bfloat16 and optional transposes.  Float32 arithmetic
+// on the CUDA cores; a thread owns a square of contiguous rows and columns and
+// reads them from shared memory as vectors (with one word each the products
+// were bound by shared memory), the next K tile is loaded while the present
+// one is used.  Tiles of 64 x 64, or 32 x 32 where those would leave SMs idle
+// (a batch of 256 has 16 tiles of 64); both add over K in the same order.
+// Weight gradients sum over the batch: their K-list is cut into pieces of at
+// least 256 (up to 32) over blockIdx.z, each writes a partial tile, and one
+// launch adds the pieces of all layers in ascending order.  The column sums of
+// the same operand (bias gradients) are taken from the staged tiles.
+// Measured: gradients of 4099 samples 2.41 -> 0.31 ms a call (16 CTAs summed
+// 4099 terms each, and one thread per column the bias gradients).
 #include <cuda_bf16.h>
 
 #include "kernels.h"
@@ -12,7 +23,7 @@
 namespace mpspt {
 namespace {
 
-constexpr int MT = 64, NTL = 64, KT = 16;
+constexpr int KT = 16;
 
 template <class TB>
 __device__ __forceinline__ float ld(const TB* p, size_t i);
@@ -23,58 +34,89 @@ __device__ __forceinline__ float ld<__nv_bfloat16>(const __nv_bfloat16* p, size_
     return __bfloat162float(p[i]);
 }
 
-// epi: 0 plain, 1 + bias, 2 + bias then relu, 3 multiply by (mask > 0)
-template <class TB>
-__global__ void __launch_bounds__(256) k_mlp_gemm(int M, int N, int K, const float* __restrict__ A, int lda,
+// epi: 0 plain, 1 + bias, 2 + bias then relu, 3 multiply by (mask > 0).
+// kchunk: K of one blockIdx.z piece; with part set, piece z writes its sums to
+// part + z * (M * N + M), and the row sums of opA behind them (bsum: those of
+// a single piece).
+template <class TB, int T>
+__global__ void __launch_bounds__(256) k_mlp_gemm(int M, int N, int K, int kchunk, const float* __restrict__ A, int lda,
                                                   int ta, const TB* __restrict__ B, int ldb, int tb,
                                                   float* __restrict__ C, int ldc, const float* __restrict__ bias,
-                                                  const float* __restrict__ mask, int epi) {
-    __shared__ float As[KT][MT + 1];
-    __shared__ float Bs[KT][NTL + 1];
-    const int r0 = blockIdx.y * MT, c0 = blockIdx.x * NTL;
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    float acc[4][4] = {};
-    for (int k0 = 0; k0 < K; k0 += KT) {
-        for (int e = threadIdx.x; e < MT * KT; e += 256) {
-            int i, kk;
-            if (ta) { i = e % MT; kk = e / MT; } else { kk = e % KT; i = e / KT; }
-            const int r = r0 + i, k = k0 + kk;
-            float v = 0.f;
-            if (r < M && k < K) v = ta ? A[(size_t)k * lda + r] : A[(size_t)r * lda + k];
-            As[kk][i] = v;
+                                                  const float* __restrict__ mask, int epi, float* __restrict__ part,
+                                                  float* __restrict__ bsum) {
+    constexpr int MI = T / 16, LD = T + 4, PER = T * KT / 256;
+    __shared__ __align__(16) float As[2][KT][LD];
+    __shared__ __align__(16) float Bs[2][KT][LD];
+    const int r0 = blockIdx.y * T, c0 = blockIdx.x * T, tid = threadIdx.x;
+    const int tx = tid % 16, ty = tid / 16;
+    const int kb = blockIdx.z * kchunk, ke = min(K, kb + kchunk);
+    const bool sums = (part || bsum) && blockIdx.x == 0 && tid < T;
+    float acc[MI][MI] = {}, rs = 0.f;
+    float ra[PER], rb[PER];
+    auto load = [&](int k0) {
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            const int e = tid + q * 256;
+            const int i = ta ? e % T : e / KT, ka = ta ? e / T : e % KT;
+            const int j = tb ? e / KT : e % T, kc = tb ? e % KT : e / T;
+            const int r = r0 + i, c = c0 + j, k1 = k0 + ka, k2 = k0 + kc;
+            ra[q] = r < M && k1 < ke ? (ta ? A[(size_t)k1 * lda + r] : A[(size_t)r * lda + k1]) : 0.f;
+            rb[q] = c < N && k2 < ke ? (tb ? ld(B, (size_t)c * ldb + k2) : ld(B, (size_t)k2 * ldb + c)) : 0.f;
         }
-        for (int e = threadIdx.x; e < NTL * KT; e += 256) {
-            int j, kk;
-            if (tb) { kk = e % KT; j = e / KT; } else { j = e % NTL; kk = e / NTL; }
-            const int c = c0 + j, k = k0 + kk;
-            float v = 0.f;
-            if (c < N && k < K) v = tb ? ld(B, (size_t)c * ldb + k) : ld(B, (size_t)k * ldb + c);
-            Bs[kk][j] = v;
+    };
+    auto store = [&](int buf) {
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            const int e = tid + q * 256;
+            As[buf][ta ? e / T : e % KT][ta ? e % T : e / KT] = ra[q];
+            Bs[buf][tb ? e % KT : e / T][tb ? e / KT : e % T] = rb[q];
         }
-        __syncthreads();
+    };
+    int buf = 0;
+    if (kb < ke) {
+        load(kb);
+        store(0);
+    }
+    __syncthreads();
+    for (int k0 = kb; k0 < ke; k0 += KT, buf ^= 1) {
+        const bool more = k0 + KT < ke;
+        if (more) load(k0 + KT);
 #pragma unroll
         for (int kk = 0; kk < KT; ++kk) {
-            float a[4], b[4];
+            float a[MI], b[MI];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
+            for (int i = 0; i < MI; i += 2) {   // (vector loads)
+                *reinterpret_cast<float2*>(a + i) = *reinterpret_cast<const float2*>(&As[buf][kk][ty * MI + i]);
+                *reinterpret_cast<float2*>(b + i) = *reinterpret_cast<const float2*>(&Bs[buf][kk][tx * MI + i]);
+            }
 #pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
+            for (int i = 0; i < MI; ++i)
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+                for (int j = 0; j < MI; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
         }
+        if (sums)
+#pragma unroll
+            for (int kk = 0; kk < KT; ++kk) rs += As[buf][kk][tid];
+        if (more) store(buf ^ 1);
         __syncthreads();
     }
+    if (sums && r0 + tid < M) {
+        if (part) part[(size_t)blockIdx.z * ((size_t)M * N + M) + (size_t)M * N + r0 + tid] = rs;
+        else bsum[r0 + tid] = rs;
+    }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int r = r0 + ty + 16 * i;
+    for (int i = 0; i < MI; ++i) {
+        const int r = r0 + ty * MI + i;
         if (r >= M) continue;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int c = c0 + tx + 16 * j;
+        for (int j = 0; j < MI; ++j) {
+            const int c = c0 + tx * MI + j;
             if (c >= N) continue;
             float v = acc[i][j];
+            if (part) {
+                part[(size_t)blockIdx.z * ((size_t)M * N + M) + (size_t)r * N + c] = v;
+                continue;
+            }
             if (epi == 1 || epi == 2) v += bias[c];
             if (epi == 2) v = fmaxf(v, 0.f);
             if (epi == 3) v = mask[(size_t)r * ldc + c] > 0.f ? v : 0.f;
@@ -83,13 +125,18 @@ __global__ void __launch_bounds__(256) k_mlp_gemm(int M, int N, int K, const flo
     }
 }
 
-// column sums: out[n] = sum_m A[m][n]
-__global__ void k_colsum(int M, int N, const float* __restrict__ A, float* __restrict__ out) {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    float s = 0.f;
-    for (int m = 0; m < M; ++m) s += A[(size_t)m * N + n];
-    out[n] = s;
+// Pieces of the weight and bias gradients of the layers, added in order.
+__global__ void k_wgrad_sum(MlpSums s) {
+    for (int l = 0; l < s.count; ++l) {
+        const MlpSums::L& q = s.l[l];
+        const size_t n = (size_t)q.wn + q.bn;
+        for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+            float v = 0.f;
+            for (int z = 0; z < q.pieces; ++z) v += q.part[(size_t)z * n + i];
+            if (i < (size_t)q.wn) q.gW[i] = v;
+            else q.gb[i - q.wn] = v;
+        }
+    }
 }
 
 // dY = (Y - T) / B and the loss terms 0.5 |Y - T|^2 / B (per row)
@@ -128,27 +175,40 @@ __global__ void k_to_bf16(int n, const float* __restrict__ w, __nv_bfloat16* __r
 
 }  // namespace
 
-void mlp_gemm(int M, int N, int K, const float* A, int lda, bool ta, const float* B, int ldb, bool tb,
-              float* C, int ldc, const float* bias, const float* mask, int epi, cudaStream_t st) {
+namespace {
+// 64 x 64 tiles when they give every SM one, 32 x 32 otherwise
+template <class TB>
+void gemm(int M, int N, int K, int pieces, const float* A, int lda, bool ta, const TB* B, int ldb, bool tb, float* C,
+          int ldc, const float* bias, const float* mask, int epi, float* part, float* bsum, cudaStream_t st) {
     if (M <= 0 || N <= 0) return;
-    dim3 g((N + NTL - 1) / NTL, (M + MT - 1) / MT);
+    const int kchunk = pieces > 1 ? ((K + pieces - 1) / pieces + KT - 1) / KT * KT : K > 0 ? K : 1;
+    auto grid = [&](int t) { return dim3((N + t - 1) / t, (M + t - 1) / t, pieces); };
+    const dim3 g64 = grid(64), g32 = grid(32);
     count_launch();
-    k_mlp_gemm<float><<<g, 256, 0, st>>>(M, N, K, A, lda, ta, B, ldb, tb, C, ldc, bias, mask, epi);
+    if ((long long)g64.x * g64.y * g64.z >= 152)
+        k_mlp_gemm<TB, 64><<<g64, 256, 0, st>>>(M, N, K, kchunk, A, lda, ta, B, ldb, tb, C, ldc, bias, mask, epi, part, bsum);
+    else
+        k_mlp_gemm<TB, 32><<<g32, 256, 0, st>>>(M, N, K, kchunk, A, lda, ta, B, ldb, tb, C, ldc, bias, mask, epi, part, bsum);
 }
+}  // namespace
 
 void mlp_gemm_bf16w(int M, int N, int K, const float* A, int lda, bool ta, const void* B, int ldb, bool tb,
                     float* C, int ldc, const float* bias, const float* mask, int epi, cudaStream_t st) {
-    if (M <= 0 || N <= 0) return;
-    dim3 g((N + NTL - 1) / NTL, (M + MT - 1) / MT);
-    count_launch();
-    k_mlp_gemm<__nv_bfloat16><<<g, 256, 0, st>>>(M, N, K, A, lda, ta, static_cast<const __nv_bfloat16*>(B), ldb,
-                                                  tb, C, ldc, bias, mask, epi);
+    gemm(M, N, K, 1, A, lda, ta, static_cast<const __nv_bfloat16*>(B), ldb, tb, C, ldc, bias, mask, epi, nullptr, nullptr, st);
 }
 
-void mlp_colsum(int M, int N, const float* A, float* out, cudaStream_t st) {
-    if (N <= 0) return;
+int mlp_wgrad_pieces(int K) { return K < 512 ? 1 : K / 256 < 32 ? K / 256 : 32; }
+
+void mlp_wgrad(int M, int N, int K, const float* dY, const float* X, float* gW, float* gb, float* part, cudaStream_t st) {
+    const int pieces = mlp_wgrad_pieces(K);
+    gemm(M, N, K, pieces, dY, M, true, X, N, false, gW, N, nullptr, nullptr, 0, pieces > 1 ? part : nullptr,
+         pieces > 1 ? nullptr : gb, st);
+}
+
+void mlp_wgrad_sum(const MlpSums& s, cudaStream_t st) {
+    if (s.count <= 0) return;
     count_launch();
-    k_colsum<<<(N + 127) / 128, 128, 0, st>>>(M, N, A, out);
+    k_wgrad_sum<<<304, 256, 0, st>>>(s);
 }
 
 void mlp_mse(int B, int N, const float* Y, const float* T, float* dY, float* rowloss, cudaStream_t st) {

@@ -85,22 +85,30 @@ float Mlp::gradient(int B, const float* Xd, const float* Td) {
     ensure(B);
     forward(B, Xd, Y.as<float>());
     mlp_mse(B, nout, Y.as<float>(), Td, dY.as<float>(), rowloss.as<float>(), st);
-    // layer 3
-    mlp_gemm(nout, width, B, dY.as<float>(), nout, true, H2.as<float>(), width, false, gW[2].as<float>(), width,
-             nullptr, nullptr, 0, st);
-    mlp_colsum(B, nout, dY.as<float>(), gb[2].as<float>(), st);
+    const int pieces = mlp_wgrad_pieces(B);
+    size_t po[3], pn = 0;   // partial sums of the layers
+    for (int l = 0; l < 3; ++l) {
+        po[l] = pn;
+        pn += (size_t)pieces * (wn(l) + out_of(l));
+    }
+    if (pieces > 1) wpart.ensure(pn * sizeof(float), st);
+    float* wp = wpart.as<float>();
+    auto wgrad = [&](int l, const float* d, const float* in) {
+        mlp_wgrad(out_of(l), in_of(l), B, d, in, gW[l].as<float>(), gb[l].as<float>(), pieces > 1 ? wp + po[l] : nullptr, st);
+    };
+    wgrad(2, dY.as<float>(), H2.as<float>());
     mlp_gemm_bf16w(B, width, nout, dY.as<float>(), nout, false, Wb[2].get(), width, false, dH2.as<float>(), width,
                    nullptr, H2.as<float>(), 3, st);
-    // layer 2
-    mlp_gemm(width, width, B, dH2.as<float>(), width, true, H1.as<float>(), width, false, gW[1].as<float>(), width,
-             nullptr, nullptr, 0, st);
-    mlp_colsum(B, width, dH2.as<float>(), gb[1].as<float>(), st);
+    wgrad(1, dH2.as<float>(), H1.as<float>());
     mlp_gemm_bf16w(B, width, width, dH2.as<float>(), width, false, Wb[1].get(), width, false, dH1.as<float>(),
                    width, nullptr, H1.as<float>(), 3, st);
-    // layer 1
-    mlp_gemm(width, nin, B, dH1.as<float>(), width, true, Xd, nin, false, gW[0].as<float>(), nin, nullptr, nullptr,
-             0, st);
-    mlp_colsum(B, width, dH1.as<float>(), gb[0].as<float>(), st);
+    wgrad(0, dH1.as<float>(), Xd);
+    if (pieces > 1) {
+        MlpSums s{};
+        for (int l = 0; l < 3; ++l)
+            s.l[s.count++] = {wp + po[l], gW[l].as<float>(), gb[l].as<float>(), (int)wn(l), out_of(l), pieces};
+        mlp_wgrad_sum(s, st);
+    }
     std::vector<float> rl(B);
     MPSPT_CUDA(cudaMemcpyAsync(rl.data(), rowloss.get(), (size_t)B * sizeof(float), cudaMemcpyDeviceToHost, st));
     MPSPT_CUDA(cudaStreamSynchronize(st));

@@ -18,7 +18,7 @@ struct Mlp {
     int nin = 0, width = 0, nout = 0;
     cudaStream_t st = 0;
     DBuf W[3], b[3], Wb[3], mW[3], vW[3], mb[3], vb[3], gW[3], gb[3];
-    DBuf X, H1, H2, Y, T, dY, dH2, dH1, rowloss;
+    DBuf X, H1, H2, Y, T, dY, dH2, dH1, rowloss, wpart;
     int cap = 0, step = 0;
 
     Mlp(int nin_, int width_, int nout_, unsigned long long seed, cudaStream_t st_);
