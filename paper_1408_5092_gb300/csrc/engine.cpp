@@ -1410,6 +1410,7 @@ struct Sweeper {
     // the host.  Returns the Ritz value; x holds the unit Ritz vector.
     double davidson(size_t n) {
         constexpr int kmax = 16;
+        static_assert(kmax <= 16, "the passes take at most 16 vectors");
         const int maxit = std::max(8, c.opt.cg_max_iter);
         dvec.ensure((size_t)kmax * n * sizeof(double) + 16, ln.st);
         davec.ensure((size_t)kmax * n * sizeof(double) + 16, ln.st);
@@ -1420,36 +1421,34 @@ struct Sweeper {
         double* x = w.x.as<double>();
         auto V = [&](int j) { return Vb + (size_t)j * n; };
         auto AV = [&](int j) { return AVb + (size_t)j * n; };
-        auto dots = [&](int cnt, const double* const* a, const double* const* b) {
-            for (int q = 0; q < cnt; ++q)
-                vec_dot(a[q], b[q], n, dsc.as<double>() + q, ln.red.as<double>(), ln.cnt.as<unsigned>(), ln.st);
-            MPSPT_CUDA(cudaMemcpyAsync(dsc_host, dsc.get(), cnt * sizeof(double), cudaMemcpyDeviceToHost, ln.st));
+        double* red = ln.red.as<double>();
+        unsigned* cnt = ln.cnt.as<unsigned>();
+        // device scalars: [0, 16) column of H, 16 the squared norm before
+        // normalisation, 17 the squared residual, [18, 34) and [34, 50) overlaps
+        double* sc = dsc.as<double>();
+        auto fetch = [&](int first, int count) {
+            MPSPT_CUDA(cudaMemcpyAsync(dsc_host, sc + first, count * sizeof(double), cudaMemcpyDeviceToHost, ln.st));
             wait();
         };
-        {   // v0 = x / |x|
-            const double* a[1] = {x};
-            dots(1, a, a);
-            const double nx = std::sqrt(dsc_host[0]);
-            require(nx > 0.0 && std::isfinite(nx), "Davidson: zero start vector");
-            vec_scale_mask(V(0), x, 1.0 / nx, n, ln.st);
-        }
+        // v0 = x / |x|
+        MPSPT_CUDA(cudaMemcpyAsync(V(0), x, n * sizeof(double), cudaMemcpyDeviceToDevice, ln.st));
+        vec_dot(x, x, n, sc + 16, red, cnt, ln.st);
         std::vector<double> H((size_t)kmax * kmax, 0.0);
         int m = 1;
-        bool need_av = true;
         double theta = 0.0;
         const double tol = c.opt.cg_tol;
         for (int it = 0; it < maxit; ++it) {
-            if (need_av) {   // AV[m-1] = A V[m-1] and the new column of H
-                MPSPT_CUDA(cudaMemcpyAsync(w.p.get(), V(m - 1), n * sizeof(double), cudaMemcpyDeviceToDevice, ln.st));
-                sigma64();
-                MPSPT_CUDA(cudaMemcpyAsync(AV(m - 1), w.Ap.get(), n * sizeof(double), cudaMemcpyDeviceToDevice, ln.st));
-                std::vector<const double*> a(m), b(m, AV(m - 1));
-                for (int j = 0; j < m; ++j) a[j] = V(j);
-                dots(m, a.data(), b.data());
-                for (int j = 0; j < m; ++j) H[(size_t)j * kmax + m - 1] = H[(size_t)(m - 1) * kmax + j] = dsc_host[j];
-            }
+            // AV[m-1] = A V[m-1] (normalised here) and the new column of H
+            dav_unit(V(m - 1), w.p.as<double>(), sc + 16, n, ln.st);
+            sigma64();
+            dav_column(AV(m - 1), w.Ap.as<double>(), Vb, m, n, sc, red, cnt, ln.st);
+            fetch(0, 17);
+            const double vn = std::sqrt(dsc_host[16]);
+            if (it == 0) require(vn > 0.0 && std::isfinite(vn), "Davidson: zero start vector");
+            else require(vn > 1e-300, "Davidson: correction vanished before convergence", MPSPT_ERR_NOT_CONVERGED);
+            for (int j = 0; j < m; ++j) H[(size_t)j * kmax + m - 1] = H[(size_t)(m - 1) * kmax + j] = dsc_host[j];
             // Rayleigh-Ritz on span V
-            std::vector<double> Hm((size_t)m * m), ev, U;
+            std::vector<double> Hm((size_t)m * m), ev, U, y(m);
             for (int i2 = 0; i2 < m; ++i2)
                 for (int j = 0; j < m; ++j) Hm[(size_t)i2 * m + j] = H[(size_t)i2 * kmax + j];
             jacobi_eigh(m, Hm, ev, U);
@@ -1457,19 +1456,9 @@ struct Sweeper {
             for (int j = 1; j < m; ++j) if (ev[j] < ev[lo]) lo = j;
             theta = ev[lo];
             // u = V y -> x, A u = AV y -> w.r, residual r = A u - theta u -> w.z
-            vec_zero(x, n, ln.st);
-            vec_zero(w.r.as<double>(), n, ln.st);
-            for (int j = 0; j < m; ++j) {
-                const double y = U[(size_t)j * m + lo];
-                vec_axpy(x, V(j), y, n, ln.st);
-                vec_axpy(w.r.as<double>(), AV(j), y, n, ln.st);
-            }
-            MPSPT_CUDA(cudaMemcpyAsync(w.z.get(), w.r.get(), n * sizeof(double), cudaMemcpyDeviceToDevice, ln.st));
-            vec_axpy(w.z.as<double>(), x, -theta, n, ln.st);
-            {
-                const double* a[1] = {w.z.as<double>()};
-                dots(1, a, a);
-            }
+            for (int j = 0; j < m; ++j) y[j] = U[(size_t)j * m + lo];
+            dav_ritz(x, w.r.as<double>(), w.z.as<double>(), Vb, AVb, m, n, y.data(), theta, sc + 17, red, cnt, ln.st);
+            fetch(17, 1);
             const double rn = std::sqrt(dsc_host[0]);
             if (rn <= tol * std::max(1.0, std::fabs(theta))) return theta;
             if (m == kmax) {   // restart from the Ritz vector
@@ -1480,24 +1469,12 @@ struct Sweeper {
                 m = 1;
             }
             // correction t = r / (theta - diag) on the masked entries, then
-            // orthogonalised against V twice and normalised
+            // orthogonalised against V twice (and normalised by the next pass)
             double* t = V(m);
-            davidson_correction(t, w.z.as<double>(), w.dg.as<double>(), theta, n, ln.st);
-            for (int pass = 0; pass < 2; ++pass) {
-                std::vector<const double*> a(m), b(m, t);
-                for (int j = 0; j < m; ++j) a[j] = V(j);
-                dots(m, a.data(), b.data());
-                for (int j = 0; j < m; ++j) vec_axpy(t, V(j), -dsc_host[j], n, ln.st);
-            }
-            {
-                const double* a[1] = {t};
-                dots(1, a, a);
-            }
-            const double tn = std::sqrt(dsc_host[0]);
-            require(tn > 1e-300, "Davidson: correction vanished before convergence", MPSPT_ERR_NOT_CONVERGED);
-            vec_scale_mask(t, t, 1.0 / tn, n, ln.st);
+            dav_correct(t, w.z.as<double>(), w.dg.as<double>(), theta, Vb, m, n, sc + 18, red, cnt, ln.st);
+            dav_project(t, Vb, m, n, sc + 18, sc + 34, false, red, cnt, ln.st);
+            dav_project(t, Vb, m, n, sc + 34, sc + 16, true, red, cnt, ln.st);
             ++m;
-            need_av = true;
         }
         throw Error(MPSPT_ERR_NOT_CONVERGED, "Davidson reached its iteration cap (cg_max_iter)");
     }

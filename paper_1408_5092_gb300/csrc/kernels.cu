@@ -197,76 +197,79 @@ __global__ void k_copy(const CopyTask* __restrict__ tasks) {
 }
 
 // ----------------------------------------------------------------- vectors
+// Sums over a vector: a float64 addition occupies a warp's sub-partition for
+// 64 clocks however few lanes it has, so a block adds its 256 partial values
+// with 8 + 5 additions of one warp per sum (a shuffle tree in every warp took
+// 5 per warp and sum, and one thread adding the blocks one by one 64 clocks
+// and a cache miss each).  Fixed order: deterministic.
 constexpr int RB = 256;        // threads per reduction block
-constexpr int RG_MAX = 1024;   // max reduction blocks
+constexpr int RG_MAX = 456;    // max reduction blocks (three a SM)
 
 inline int red_grid(size_t n) {
-    size_t g = (n + (size_t)RB * 4 - 1) / ((size_t)RB * 4);
+    size_t g = (n + (size_t)RB * 2 - 1) / ((size_t)RB * 2);
     if (g < 1) g = 1;
     if (g > RG_MAX) g = RG_MAX;
     return (int)g;
 }
 
-template <int NV>
-__device__ void block_sum(double (&v)[NV], double (*sh)[RB / 32]) {
-#pragma unroll
-    for (int q = 0; q < NV; ++q)
-        for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
-    if ((threadIdx.x & 31) == 0)
-#pragma unroll
-        for (int q = 0; q < NV; ++q) sh[q][threadIdx.x >> 5] = v[q];
-    __syncthreads();
-    if (threadIdx.x == 0)
-#pragma unroll
-        for (int q = 0; q < NV; ++q) {
-            double s = 0.0;
-            for (int w = 0; w < RB / 32; ++w) s += sh[q][w];
-            v[q] = s;
-        }
+// sum of sh[0 .. n) over the calling warp, in all its lanes
+__device__ __forceinline__ double warp_total(const double* x, int n) {
+    double v = 0.0;
+    for (int i = threadIdx.x & 31; i < n; i += 32) v += __ldcg(x + i);
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
 }
 
-// Last-block-done pattern: every block stores its partial sums, the last one
-// to finish adds them in block order (deterministic) and runs `fin`.
+// Every block adds its threads' v[q], q < nv, stores the sums, and the last
+// block to finish adds them over the blocks, in block order, into tot (shared
+// memory, nv values); returns true in all its threads.  sh: nv x RB doubles
+// of shared memory.
 template <int NV>
-__device__ bool last_block(double (&v)[NV], double* scratch, unsigned* counter, double (&tot)[NV]) {
+__device__ bool grid_sum(const double (&v)[NV], int nv, double (*sh)[RB], double* tot, double* scratch,
+                         unsigned* counter) {
     __shared__ bool is_last;
-    if (threadIdx.x == 0) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
-        for (int q = 0; q < NV; ++q) scratch[q * RG_MAX + blockIdx.x] = v[q];
-        __threadfence();
-        unsigned prev = atomicAdd(counter, 1u);
-        is_last = (prev == gridDim.x - 1);
+    for (int q = 0; q < NV; ++q)
+        if (q < nv) sh[q][threadIdx.x] = v[q];
+    __syncthreads();
+    for (int q = warp; q < nv; q += RB / 32) {
+        double x = 0.0;
+#pragma unroll
+        for (int i = 0; i < RB / 32; ++i) x += sh[q][lane + 32 * i];
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (lane == 0) scratch[(size_t)q * gridDim.x + blockIdx.x] = x;
     }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) is_last = atomicAdd(counter, 1u) == gridDim.x - 1;
     __syncthreads();
     if (!is_last) return false;
-    if (threadIdx.x == 0) {
-        __threadfence();
-#pragma unroll
-        for (int q = 0; q < NV; ++q) {
-            double s = 0.0;
-            for (unsigned b = 0; b < gridDim.x; ++b) s += ((volatile double*)scratch)[q * RG_MAX + b];
-            tot[q] = s;
-        }
-        *counter = 0;
+    __threadfence();
+    for (int q = warp; q < nv; q += RB / 32) {
+        const double x = warp_total(scratch + (size_t)q * gridDim.x, gridDim.x);
+        if (lane == 0) tot[q] = x;
     }
-    return threadIdx.x == 0;
+    if (threadIdx.x == 0) *counter = 0;
+    __syncthreads();
+    return true;
 }
 
 __global__ void k_dot(const double* __restrict__ x, const double* __restrict__ y, size_t n,
                       double* out, double* scratch, unsigned* counter) {
-    __shared__ double sh[1][RB / 32];
+    __shared__ double sh[1][RB];
+    __shared__ double tot[1];
     double v[1] = {0.0};
     for (size_t i = blockIdx.x * (size_t)RB + threadIdx.x; i < n; i += (size_t)gridDim.x * RB)
         v[0] += x[i] * y[i];
-    block_sum<1>(v, sh);
-    double tot[1];
-    if (last_block<1>(v, scratch, counter, tot)) *out = tot[0];
+    if (grid_sum<1>(v, 1, sh, tot, scratch, counter) && threadIdx.x == 0) *out = tot[0];
 }
 
 __global__ void k_cg_init(double* r, double* z, double* p, const double* __restrict__ b,
                           const double* __restrict__ Ax, const double* __restrict__ minv, size_t n,
                           CgState* S, double tol, double* scratch, unsigned* counter) {
-    __shared__ double sh[3][RB / 32];
+    __shared__ double sh[3][RB];
+    __shared__ double tot[3];
     double v[3] = {0.0, 0.0, 0.0};
     for (size_t i = blockIdx.x * (size_t)RB + threadIdx.x; i < n; i += (size_t)gridDim.x * RB) {
         const double ri = b[i] - Ax[i];
@@ -278,9 +281,7 @@ __global__ void k_cg_init(double* r, double* z, double* p, const double* __restr
         v[1] += ri * ri;
         v[2] += b[i] * b[i];
     }
-    block_sum<3>(v, sh);
-    double tot[3];
-    if (last_block<3>(v, scratch, counter, tot)) {
+    if (grid_sum<3>(v, 3, sh, tot, scratch, counter) && threadIdx.x == 0) {
         S->rz = tot[0];
         S->rr = tot[1];
         S->bb = tot[2];
@@ -294,13 +295,12 @@ __global__ void k_cg_init(double* r, double* z, double* p, const double* __restr
 __global__ void k_cg_pap(const double* __restrict__ p, const double* __restrict__ Ap, size_t n,
                          CgState* S, double* scratch, unsigned* counter) {
     if (S->done) return;
-    __shared__ double sh[1][RB / 32];
+    __shared__ double sh[1][RB];
+    __shared__ double tot[1];
     double v[1] = {0.0};
     for (size_t i = blockIdx.x * (size_t)RB + threadIdx.x; i < n; i += (size_t)gridDim.x * RB)
         v[0] += p[i] * Ap[i];
-    block_sum<1>(v, sh);
-    double tot[1];
-    if (last_block<1>(v, scratch, counter, tot)) {
+    if (grid_sum<1>(v, 1, sh, tot, scratch, counter) && threadIdx.x == 0) {
         S->pAp = tot[0];
         if (!(tot[0] > 0.0)) { S->not_spd = 1; S->done = 1; }
         else S->alpha = S->rz / tot[0];
@@ -311,7 +311,8 @@ __global__ void k_cg_update(double* x, double* r, double* z, const double* __res
                             const double* __restrict__ Ap, const double* __restrict__ minv,
                             size_t n, CgState* S, double* scratch, unsigned* counter) {
     if (S->done) return;
-    __shared__ double sh[2][RB / 32];
+    __shared__ double sh[2][RB];
+    __shared__ double tot[2];
     const double a = S->alpha;
     double v[2] = {0.0, 0.0};
     for (size_t i = blockIdx.x * (size_t)RB + threadIdx.x; i < n; i += (size_t)gridDim.x * RB) {
@@ -323,9 +324,7 @@ __global__ void k_cg_update(double* x, double* r, double* z, const double* __res
         v[0] += ri * zi;
         v[1] += ri * ri;
     }
-    block_sum<2>(v, sh);
-    double tot[2];
-    if (last_block<2>(v, scratch, counter, tot)) {
+    if (grid_sum<2>(v, 2, sh, tot, scratch, counter) && threadIdx.x == 0) {
         S->rz_new = tot[0];
         S->rr = tot[1];
         S->beta = tot[0] / S->rz;
@@ -358,16 +357,93 @@ __global__ void k_minv(double* y, const double* __restrict__ d, size_t n) {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
         y[i] = d[i] > 0.0 ? 1.0 / d[i] : 0.0;
 }
-// Davidson correction t = r / (theta - d), the denominator kept at least
-// 1e-8 max(1, |theta|) away from zero (its sign kept)
-__global__ void k_dav_corr(double* t, const double* __restrict__ r, const double* __restrict__ d, double theta,
-                           size_t n) {
+// ---- Davidson (ground-state DMRG).  Bases V, AV: vectors of n, leading
+// dimension n.  One pass over the vectors per step instead of one launch per
+// inner product and per update.
+constexpr int DAV_MAX = 16;   // basis vectors at most
+struct DavY { double y[DAV_MAX]; };
+
+// q < m: out[q] = V_q . t
+// MODE 0: t = r / (theta - d), the denominator kept at least 1e-8 max(1,
+//         |theta|) away from zero (its sign kept)
+// MODE 1: t -= sum_q coef[q] V_q
+// MODE 2: the same, and out[0] = t . t instead
+// MODE 3: t = src
+template <int MODE>
+__global__ void __launch_bounds__(RB) k_dav_pass(double* t, const double* __restrict__ V, int m, size_t n,
+                                                 const double* __restrict__ src, const double* __restrict__ d,
+                                                 double theta, const double* coef, double* out, double* scratch,
+                                                 unsigned* counter) {
+    constexpr int NV = MODE == 2 ? 1 : DAV_MAX;
+    __shared__ double sh[NV][RB];
+    __shared__ double tot[NV];
     const double eps = 1e-8 * fmax(1.0, fabs(theta));
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        double den = theta - d[i];
-        if (fabs(den) < eps) den = den < 0.0 ? -eps : eps;
-        t[i] = r[i] / den;
+    double c[DAV_MAX], v[NV];
+#pragma unroll
+    for (int q = 0; q < NV; ++q) v[q] = 0.0;
+    if (MODE == 1 || MODE == 2)
+#pragma unroll
+        for (int q = 0; q < DAV_MAX; ++q) c[q] = q < m ? coef[q] : 0.0;
+    for (size_t i = blockIdx.x * (size_t)RB + threadIdx.x; i < n; i += (size_t)gridDim.x * RB) {
+        double x;
+        if (MODE == 0) {
+            double den = theta - d[i];
+            if (fabs(den) < eps) den = den < 0.0 ? -eps : eps;
+            x = src[i] / den;
+        } else {
+            x = MODE == 3 ? src[i] : t[i];
+        }
+        double b[DAV_MAX];
+#pragma unroll
+        for (int q = 0; q < DAV_MAX; ++q) b[q] = q < m && MODE != 2 ? V[(size_t)q * n + i] : 0.0;
+        if (MODE == 1 || MODE == 2)
+#pragma unroll
+            for (int q = 0; q < DAV_MAX; ++q)
+                if (q < m) x = fma(-c[q], MODE == 2 ? V[(size_t)q * n + i] : b[q], x);
+        t[i] = x;
+        if (MODE == 2) v[0] = fma(x, x, v[0]);
+        else
+#pragma unroll
+            for (int q = 0; q < NV; ++q)
+                if (q < m) v[q] = fma(b[q], x, v[q]);
     }
+    const int nv = MODE == 2 ? 1 : m;
+    __syncthreads();
+    if (grid_sum<NV>(v, nv, sh, tot, scratch, counter) && threadIdx.x < nv) out[threadIdx.x] = tot[threadIdx.x];
+}
+
+// p = t = t / sqrt(*norm2)
+__global__ void k_dav_unit(double* t, double* p, const double* __restrict__ norm2, size_t n) {
+    const double a = 1.0 / sqrt(*norm2);
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        const double v = a * t[i];
+        t[i] = v;
+        p[i] = v;
+    }
+}
+
+// Ritz vector x = sum y_q V_q, ax = sum y_q AV_q, z = ax - theta x; *out = z . z
+__global__ void __launch_bounds__(RB) k_dav_ritz(double* x, double* ax, double* z, const double* __restrict__ V,
+                                                 const double* __restrict__ AV, int m, size_t n, DavY y, double theta,
+                                                 double* out, double* scratch, unsigned* counter) {
+    __shared__ double sh[1][RB];
+    __shared__ double tot[1];
+    double v[1] = {0.0};
+    for (size_t i = blockIdx.x * (size_t)RB + threadIdx.x; i < n; i += (size_t)gridDim.x * RB) {
+        double s = 0.0, w = 0.0;
+#pragma unroll
+        for (int q = 0; q < DAV_MAX; ++q)
+            if (q < m) {
+                s = fma(y.y[q], V[(size_t)q * n + i], s);
+                w = fma(y.y[q], AV[(size_t)q * n + i], w);
+            }
+        const double r = fma(-theta, s, w);
+        x[i] = s;
+        ax[i] = w;
+        z[i] = r;
+        v[0] = fma(r, r, v[0]);
+    }
+    if (grid_sum<1>(v, 1, sh, tot, scratch, counter) && threadIdx.x == 0) *out = tot[0];
 }
 __global__ void k_d2f(float* y, const double* __restrict__ x, size_t n) {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
@@ -494,8 +570,33 @@ void f64_to_f32(float* y, const double* x, size_t n, cudaStream_t st) {
 void f32_to_f64(double* y, const float* x, size_t n, cudaStream_t st) {
     if (n) { counted(); k_f2d<<<ew_grid(n), 256, 0, st>>>(y, x, n); }
 }
-void davidson_correction(double* t, const double* r, const double* diag, double theta, size_t n, cudaStream_t st) {
-    if (n) { counted(); k_dav_corr<<<ew_grid(n), 256, 0, st>>>(t, r, diag, theta, n); }
+namespace {
+inline int dav_grid(size_t n) {   // scratch: DAV_MAX sums of at most 228 blocks
+    return std::min(red_grid(n), 228);
+}
+}  // namespace
+void dav_correct(double* t, const double* r, const double* diag, double theta, const double* V, int m, size_t n,
+                 double* coef, double* scratch, unsigned* counter, cudaStream_t st) {
+    counted(); k_dav_pass<0><<<dav_grid(n), RB, 0, st>>>(t, V, m, n, r, diag, theta, nullptr, coef, scratch, counter);
+}
+void dav_project(double* t, const double* V, int m, size_t n, const double* coef, double* next, bool last,
+                 double* scratch, unsigned* counter, cudaStream_t st) {
+    counted();
+    if (last) k_dav_pass<2><<<dav_grid(n), RB, 0, st>>>(t, V, m, n, nullptr, nullptr, 0.0, coef, next, scratch, counter);
+    else k_dav_pass<1><<<dav_grid(n), RB, 0, st>>>(t, V, m, n, nullptr, nullptr, 0.0, coef, next, scratch, counter);
+}
+void dav_unit(double* t, double* p, const double* norm2, size_t n, cudaStream_t st) {
+    counted(); k_dav_unit<<<ew_grid(n), 256, 0, st>>>(t, p, norm2, n);
+}
+void dav_column(double* av, const double* ap, const double* V, int m, size_t n, double* h, double* scratch,
+                unsigned* counter, cudaStream_t st) {
+    counted(); k_dav_pass<3><<<dav_grid(n), RB, 0, st>>>(av, V, m, n, ap, nullptr, 0.0, nullptr, h, scratch, counter);
+}
+void dav_ritz(double* x, double* ax, double* z, const double* V, const double* AV, int m, size_t n, const double* y,
+              double theta, double* out, double* scratch, unsigned* counter, cudaStream_t st) {
+    DavY yy{};
+    for (int q = 0; q < m; ++q) yy.y[q] = y[q];
+    counted(); k_dav_ritz<<<red_grid(n), RB, 0, st>>>(x, ax, z, V, AV, m, n, yy, theta, out, scratch, counter);
 }
 void make_minv(double* minv, const double* diag, size_t n, cudaStream_t st) {
     if (n) { counted(); k_minv<<<ew_grid(n), 256, 0, st>>>(minv, diag, n); }

@@ -201,7 +201,7 @@ void launch_copy(const CopyTask* tasks, int ntask, cudaStream_t st);
 void vec_zero(double* x, size_t n, cudaStream_t st);
 void vec_scale_mask(double* y, const double* x, double a, size_t n, cudaStream_t st);  // y = a*x
 void vec_axpy(double* y, const double* x, double a, size_t n, cudaStream_t st);       // y += a*x
-// out[slot] = x.y  (partial sums in scratch, which needs >= 1024 doubles)
+// out[slot] = x.y  (partial sums in scratch: 4096 doubles, for all of these)
 void vec_dot(const double* x, const double* y, size_t n, double* out, double* scratch,
              unsigned* counter, cudaStream_t st);
 void f64_to_f32(float* y, const double* x, size_t n, cudaStream_t st);
@@ -217,8 +217,21 @@ void cg_init(double* r, double* z, double* p, const double* b, const double* Ax,
 void cg_step(double* x, double* r, double* z, double* p, const double* Ap, const double* minv,
              size_t n, CgState* S, double* scratch, unsigned* counter, cudaStream_t st);
 void make_minv(double* minv, const double* diag, size_t n, cudaStream_t st);
-// t = r / (theta - diag), denominators kept away from zero (Davidson correction)
-void davidson_correction(double* t, const double* r, const double* diag, double theta, size_t n, cudaStream_t st);
+// Davidson passes over a basis V (and AV) of m <= 16 vectors of n:
+//  dav_correct: t = r / (theta - diag), denominators kept away from zero, and coef[q] = V_q . t
+//  dav_project: t -= sum coef[q] V_q, and next[q] = V_q . t (last: next[0] = t . t)
+//  dav_unit:    p = t = t / sqrt(*norm2)
+//  dav_column:  av = ap and h[q] = V_q . av
+//  dav_ritz:    x = sum y_q V_q, ax = sum y_q AV_q, z = ax - theta x, *out = z . z
+void dav_correct(double* t, const double* r, const double* diag, double theta, const double* V, int m, size_t n,
+                 double* coef, double* scratch, unsigned* counter, cudaStream_t st);
+void dav_project(double* t, const double* V, int m, size_t n, const double* coef, double* next, bool last,
+                 double* scratch, unsigned* counter, cudaStream_t st);
+void dav_unit(double* t, double* p, const double* norm2, size_t n, cudaStream_t st);
+void dav_column(double* av, const double* ap, const double* V, int m, size_t n, double* h, double* scratch,
+                unsigned* counter, cudaStream_t st);
+void dav_ritz(double* x, double* ax, double* z, const double* V, const double* AV, int m, size_t n, const double* y,
+              double theta, double* out, double* scratch, unsigned* counter, cudaStream_t st);
 
 // ---- learned preconditioner (kernels_mlp.cu)
 struct BlockRef {      // one QN block of a two-site vector
