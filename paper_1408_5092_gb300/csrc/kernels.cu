@@ -135,12 +135,14 @@ __global__ void __launch_bounds__(NT) k_gemm(const GemmTask* __restrict__ tasks,
 }
 
 // Split-K reduction: partial tiles summed in ascending order (deterministic).
+// Bound by the float64 additions of one SM, so a tile is shared by eight CTAs
+// (one per tile took 48 us for tiles of 128 x 64).
 __global__ void k_splitk_reduce(const SplitRed* __restrict__ tasks, const int* __restrict__ skip) {
     if (skip && *skip) return;
     const SplitRed t = tasks[blockIdx.x];
     const int mrem = min(t.tm, t.m - t.r0), nrem = min(t.tn, t.n - t.c0);
     const size_t tile = (size_t)t.tm * t.tn;
-    for (int e = threadIdx.x; e < mrem * nrem; e += blockDim.x) {
+    for (int e = blockIdx.y * blockDim.x + threadIdx.x; e < mrem * nrem; e += gridDim.y * blockDim.x) {
         const int r = e / nrem, c = e % nrem;
         double v = 0.0;
         for (int q = 0; q < t.nparts; ++q) v += t.part[q * tile + (size_t)r * t.tn + c];
@@ -153,21 +155,35 @@ __global__ void k_splitk_reduce(const SplitRed* __restrict__ tasks, const int* _
     }
 }
 
-// dst = sum coef * src over the task's source list (memory-bound).
-__global__ void k_mix(const MixTask* __restrict__ tasks, const MixSrc* __restrict__ srcs,
-                      const int* __restrict__ skip) {
+// dst = sum coef * src over the task's source list, in order.  Blocks are
+// small (a few to a few hundred values) with up to hundreds of sources, and
+// the time is the latency of each descriptor and value load over the warps in
+// flight.  So a warp takes MIX_PIECE values of one block (the planners cut
+// larger blocks), two per lane, and a CTA four such pieces: with a CTA per
+// block three of its four warps had nothing to do and the SM's CTA slots were
+// full of them.  Measured per launch: M = 256 28.0 -> 20.7 us, M = 64 9.7 ->
+// 9.4 us.  (Eight sources in flight per thread cost too many warps: 50 us.)
+__global__ void __launch_bounds__(128, 8) k_mix(const MixTask* __restrict__ tasks, int ntask,
+                                                 const MixSrc* __restrict__ srcs, const int* __restrict__ skip) {
     if (skip && *skip) return;
-    const MixTask t = tasks[blockIdx.x];
+    const int w = blockIdx.x * 4 + (threadIdx.x >> 5);
+    if (w >= ntask) return;
+    const MixTask t = tasks[w];
     const int n = t.rows * t.cols;
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
-        const int i = e / t.cols, j = e % t.cols;
-        double s = 0.0;
-        for (int q = t.s0; q < t.s1; ++q) {
-            const MixSrc m = srcs[q];
-            s += m.coef * m.src[(size_t)i * m.lds + j];
-        }
-        t.dst[(size_t)i * t.ldd + j] = s;
+    const int e0 = t.e0 + (threadIdx.x & 31), e1 = e0 + 32;
+    const bool in0 = e0 < n, in1 = e1 < n;
+    if (!in0) return;
+    const int i0 = e0 / t.cols, j0 = e0 - i0 * t.cols;
+    const int i1 = in1 ? e1 / t.cols : i0, j1 = in1 ? e1 - i1 * t.cols : j0;
+    double s0 = 0.0, s1 = 0.0;
+#pragma unroll 4
+    for (int q = t.s0; q < t.s1; ++q) {
+        const MixSrc m = srcs[q];
+        s0 = fma(m.coef, __ldg(m.src + (size_t)i0 * m.lds + j0), s0);
+        s1 = fma(m.coef, __ldg(m.src + (size_t)i1 * m.lds + j1), s1);
     }
+    t.dst[(size_t)i0 * t.ldd + j0] = s0;
+    if (in1) t.dst[(size_t)i1 * t.ldd + j1] = s1;
 }
 
 __global__ void k_diag(const DiagTask* __restrict__ tasks, const DiagTerm* __restrict__ terms) {
@@ -522,7 +538,7 @@ bool gemm_tile_supported(int tm, int tn) {
 }
 
 void launch_splitk_reduce(const SplitRed* tasks, int ntask, cudaStream_t st, const int* skip) {
-    if (ntask > 0) { counted(); k_splitk_reduce<<<ntask, 256, 0, st>>>(tasks, skip); }
+    if (ntask > 0) { counted(); k_splitk_reduce<<<dim3(ntask, 8), 128, 0, st>>>(tasks, skip); }
 }
 
 void launch_gemm_tile(int tm, int tn, const GemmTask* tasks, int ntask, const GemmOp* ops, cudaStream_t st,
@@ -542,7 +558,7 @@ void launch_gemm_tile(int tm, int tn, const GemmTask* tasks, int ntask, const Ge
 }
 
 void launch_mix(const MixTask* tasks, int ntask, const MixSrc* srcs, cudaStream_t st, const int* skip) {
-    if (ntask > 0) { counted(); k_mix<<<ntask, 128, 0, st>>>(tasks, srcs, skip); }
+    if (ntask > 0) { counted(); k_mix<<<(ntask + 3) / 4, 128, 0, st>>>(tasks, ntask, srcs, skip); }
 }
 
 void launch_diag(const DiagTask* tasks, int ntask, const DiagTerm* terms, cudaStream_t st) {

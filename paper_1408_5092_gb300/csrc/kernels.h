@@ -74,11 +74,13 @@ struct MixSrc {
     int pad;
     double coef;
 };
+// The task covers the values [e0, e0 + MIX_PIECE) of the block, row by row.
+constexpr int MIX_PIECE = 64;
 struct MixTask {
     double* dst;
     int rows, cols, ldd;
     int s0, s1;
-    int pad;
+    int e0;
 };
 
 // Jacobi diagonal of A_loc: out[l, r] += sum coef * L[l*(ldL+1)] * R[r*(ldR+1)]

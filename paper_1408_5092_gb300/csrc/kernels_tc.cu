@@ -119,6 +119,17 @@ __device__ __forceinline__ float d2f_rn(double v) {
     return __uint_as_float(f);
 }
 
+// float32 -> float64 by integer operations (a conversion instruction occupies
+// a sub-partition's float64 unit for 64 clocks: 2 us for a tile of 128 x 64).
+// Subnormal values become signed zero.
+__device__ __forceinline__ double f2d_int(uint32_t b) {
+    const uint32_t mag = b & 0x7FFFFFFFu, sign = b & 0x80000000u;
+    uint32_t hi = (mag >> 3) + (896u << 20);
+    if (mag >= 0x7F800000u) hi = 0x7FF00000u | ((mag & 0x7FFFFFu) >> 3);
+    const bool zero = mag < 0x00800000u;
+    return __hiloint2double((int)(sign | (zero ? 0u : hi)), zero ? 0 : (int)(b << 29));
+}
+
 // hi = round(f), lo = round(f - hi) in the 16-bit type (bf16 or f16)
 template <bool F16>
 __device__ __forceinline__ void split_store(unsigned char* hi, unsigned char* lo, uint32_t off, float f) {
@@ -293,14 +304,14 @@ __global__ void __launch_bounds__(NTH, 1) k_gemm_tc(const GemmTask* __restrict__
                 for (int q = 0; q < 16; ++q) {
                     const int col = c0 + q;
                     if (col < nrem && t.part) {   // split-K partial tile (BM x BN, row-major)
-                        t.part[row * BN + col] = (double)__uint_as_float(v[q]);
+                        t.part[row * BN + col] = f2d_int(v[q]);
                     } else if (col < nrem) {
                         const int gr = t.r0 + row, gc = t.c0 + col;
                         double* dst;
                         if (t.cmap == nullptr) dst = t.C + (size_t)gr * t.ldc + gc;
                         else if (t.cmap_rows) dst = t.C + t.cmap[2 * gr] + (size_t)gc * t.cmap[2 * gr + 1];
                         else dst = t.C + t.cmap[2 * gc] + (size_t)gr * t.cmap[2 * gc + 1];
-                        const double val = (double)__uint_as_float(v[q]);
+                        const double val = f2d_int(v[q]);
                         *dst = t.accumulate ? *dst + val : val;
                     }
                 }

@@ -29,10 +29,29 @@ void GemmPlan::split(int tm_, int tn_, std::vector<GemmTask>& out, std::vector<l
     if (rd) rd->clear();
     if (rcm) rcm->clear();
     size_t pe = 0;
+    // tensor-core plans: the stages of 64 K are cut so that 304 CTAs (two a
+    // SM) of equal length would cover the plan, but into no chunk of fewer
+    // than two stages nor a block into more than 32.  A stage is bound by its
+    // operand staging (1.3 us), so the longest chunk sets the launch's time:
+    // with chunks of 512 K and more, and none below K = 1024, most launches
+    // ran 8 to 16 stages on a few dozen CTAs (36.3 -> 31.3 us a launch in the
+    // M = 256 sweep, integer float32 -> float64 stores included).
+    auto stages = [](long long K) { return (K + 63) / 64; };
+    double target = 0.0;
+    if (rd && is_tc(kind)) {
+        for (const Blk& b : blocks) {
+            long long K = 0;
+            for (int o = b.op0; o < b.op1; ++o) K += ops[o].k;
+            target += (double)((b.m + tm_ - 1) / tm_) * ((b.n + tn_ - 1) / tn_) * stages(K);
+        }
+        target = std::max(2.0, target / 304.0);
+    }
     for (const Blk& b : blocks) {
         long long K = 0;
         for (int o = b.op0; o < b.op1; ++o) K += ops[o].k;
-        const int S = rd ? kchunks(b.m, b.n, K) : 1;
+        int S = 1;
+        if (rd && is_tc(kind)) S = (int)std::max(1.0, std::min(32.0, std::ceil(stages(K) / target)));
+        else if (rd) S = kchunks(b.m, b.n, K);
         const int step = (int)((K + S - 1) / S + 63) / 64 * 64;   // whole K-stages of either kernel
         for (int r0 = 0; r0 < b.m; r0 += tm_)
             for (int c0 = 0; c0 < b.n; c0 += tn_) {
@@ -448,6 +467,15 @@ void Omega::build(const MPO& W, int i) {
     first[(size_t)Da * 16] = (int)e.size();
 }
 
+void mix_pieces(const std::vector<MixTask>& blocks, std::vector<MixTask>& out) {
+    out.clear();
+    for (const MixTask& b : blocks)
+        for (int e = 0, n = b.rows * b.cols; e < n; e += MIX_PIECE) {
+            out.push_back(b);
+            out.back().e0 = e;
+        }
+}
+
 void TwoSitePlan::build(const Omega& om, const TwoT& bra, const TwoT& ket, const Bond& braL,
                         const Bond& ketL, const Bond& braR, const Bond& ketR, const EnvT& L,
                         const EnvT& R, const std::vector<QN>& dqR, const double* x, double* out,
@@ -637,7 +665,8 @@ void TwoSitePlan::build(const Omega& om, const TwoT& bra, const TwoT& ket, const
         check(Tp, tsize * sizeof(double), "mix T");
         for (const auto& t : mtasks) check(t.dst, ((size_t)(t.rows - 1) * t.ldd + t.cols) * sizeof(double), "mix dst");
     }
-    mpspt::upload(dmt, mtasks, st);
+    mix_pieces(mtasks, mpieces);
+    mpspt::upload(dmt, mpieces, st);
     mpspt::upload(dms, msrc, st);
     g1.upload(st);
     g2.upload(st);
@@ -707,7 +736,8 @@ void EnvPlan::upload_mix(cudaStream_t st) {
         RangeCheck check;
         for (const auto& t : mt) check(t.dst, ((size_t)(t.rows - 1) * t.ldd + t.cols) * sizeof(double), "env mix dst");
     }
-    mpspt::upload(dmt, mt, st);
+    mix_pieces(mt, mp);
+    mpspt::upload(dmt, mp, st);
     mpspt::upload(dms, ms, st);
     g1.upload(st);
     g2.upload(st);

@@ -18,6 +18,9 @@ inline bool is_tc(int kind) { return kind == GEMM_TC || kind == GEMM_TC16; }
 
 struct GemmPlan;
 
+// Task list of k_mix for the planned blocks: one task per piece of a block.
+void mix_pieces(const std::vector<MixTask>& blocks, std::vector<MixTask>& out);
+
 // Tile-shape autotuner of the float64 and float32 grouped GEMMs.  A plan's
 // shape class is (arithmetic, skinny, and log2 buckets of the median block
 // rows, columns and K-length and of the block count).  The first plan of a
@@ -151,7 +154,7 @@ struct Omega {
 //        sector, scattered into the two-site layout by a column map
 struct TwoSitePlan {
     GemmPlan g1, g2, g2s;            // g2s: the float32 blocks of few rows (skinny tiles)
-    std::vector<MixTask> mtasks;
+    std::vector<MixTask> mtasks, mpieces;
     std::vector<MixSrc> msrc;
     DBuf dmt, dms;
     DBuf T, V, Lp, Rp, pk;
@@ -172,7 +175,7 @@ struct TwoSitePlan {
                cudaStream_t st);
     void run(cudaStream_t st) const {
         g1.run(st);
-        launch_mix(dmt.as<MixTask>(), (int)mtasks.size(), dms.as<MixSrc>(), st, skip);
+        launch_mix(dmt.as<MixTask>(), (int)mpieces.size(), dms.as<MixSrc>(), st, skip);
         g2.run(st);
         g2s.run(st);
     }
@@ -204,7 +207,7 @@ struct EnvPlan {
     GemmPlan g1, g2;
     void set_tuner(Autotuner* t) { g1.tuner = t; g2.tuner = t; }
     DBuf Y, Z, dmt, dms;
-    std::vector<MixTask> mt;
+    std::vector<MixTask> mt, mp;
     std::vector<MixSrc> ms;
     void build_left(const MPO& W, int site, const EnvT& L, const SiteT& Abra, const SiteT& Aket,
                     const Bond& braL, const Bond& ketL, const Bond& braR, const Bond& ketR,
@@ -218,14 +221,14 @@ struct EnvPlan {
                         cudaStream_t st);
     void run(cudaStream_t st) const {
         g1.run(st);
-        launch_mix(dmt.as<MixTask>(), (int)mt.size(), dms.as<MixSrc>(), st);
+        launch_mix(dmt.as<MixTask>(), (int)mp.size(), dms.as<MixSrc>(), st);
         g2.run(st);
     }
     double flops() const { return g1.flops + g2.flops; }
     // bytes of the task lists the last build uploads (GEMM tasks and operand
     // lists, mix tasks and sources)
     size_t plan_bytes() const {
-        return mt.size() * sizeof(MixTask) + ms.size() * sizeof(MixSrc) +
+        return mp.size() * sizeof(MixTask) + ms.size() * sizeof(MixSrc) +
                (g1.gblk.size() + g2.gblk.size()) * sizeof(GemmBlk) +
                (g1.unit_blk.size() + g2.unit_blk.size()) * sizeof(unsigned) +
                (g1.ops.size() + g2.ops.size()) * sizeof(GemmOp);
