@@ -2,6 +2,7 @@
 // float32 arithmetic driven by task lists, Jacobi diagonal, block copies, and
 // the CG vector kernels with deterministic (fixed-order) reductions.
 #include "kernels.h"
+#include "mix_piece.h"
 
 #include <atomic>
 #include <algorithm>
@@ -158,32 +159,32 @@ __global__ void k_splitk_reduce(const SplitRed* __restrict__ tasks, const int* _
 // dst = sum coef * src over the task's source list, in order.  Blocks are
 // small (a few to a few hundred values) with up to hundreds of sources, and
 // the time is the latency of each descriptor and value load over the warps in
-// flight.  So a warp takes MIX_PIECE values of one block (the planners cut
-// larger blocks), two per lane, and a CTA four such pieces: with a CTA per
-// block three of its four warps had nothing to do and the SM's CTA slots were
-// full of them.  Measured per launch: M = 256 28.0 -> 20.7 us, M = 64 9.7 ->
-// 9.4 us.  (Eight sources in flight per thread cost too many warps: 50 us.)
-__global__ void __launch_bounds__(128, 8) k_mix(const MixTask* __restrict__ tasks, int ntask,
-                                                 const MixSrc* __restrict__ srcs, const int* __restrict__ skip) {
+// flight.  k_mix takes a CTA per block, k_mix_pieces a warp per MIX_PIECE
+// values of a block, two per lane: the warps that a CTA per block leaves idle
+// (three of four in a block of up to 32 values) hold SM slots.
+__global__ void k_mix(const MixTask* __restrict__ tasks, const MixSrc* __restrict__ srcs,
+                      const int* __restrict__ skip) {
+    if (skip && *skip) return;
+    const MixTask t = tasks[blockIdx.x];
+    const int n = t.rows * t.cols;
+    for (int e = threadIdx.x; e < n; e += blockDim.x) {
+        const int i = e / t.cols, j = e % t.cols;
+        double s = 0.0;
+        for (int q = t.s0; q < t.s1; ++q) {
+            const MixSrc m = srcs[q];
+            s += m.coef * m.src[(size_t)i * m.lds + j];
+        }
+        t.dst[(size_t)i * t.ldd + j] = s;
+    }
+}
+__global__ void __launch_bounds__(128, 8) k_mix_pieces(const MixTask* __restrict__ tasks,
+                                                        const unsigned* __restrict__ piece_task, int npiece,
+                                                        const MixSrc* __restrict__ srcs, const int* __restrict__ skip) {
     if (skip && *skip) return;
     const int w = blockIdx.x * 4 + (threadIdx.x >> 5);
-    if (w >= ntask) return;
-    const MixTask t = tasks[w];
-    const int n = t.rows * t.cols;
-    const int e0 = t.e0 + (threadIdx.x & 31), e1 = e0 + 32;
-    const bool in0 = e0 < n, in1 = e1 < n;
-    if (!in0) return;
-    const int i0 = e0 / t.cols, j0 = e0 - i0 * t.cols;
-    const int i1 = in1 ? e1 / t.cols : i0, j1 = in1 ? e1 - i1 * t.cols : j0;
-    double s0 = 0.0, s1 = 0.0;
-#pragma unroll 4
-    for (int q = t.s0; q < t.s1; ++q) {
-        const MixSrc m = srcs[q];
-        s0 = fma(m.coef, __ldg(m.src + (size_t)i0 * m.lds + j0), s0);
-        s1 = fma(m.coef, __ldg(m.src + (size_t)i1 * m.lds + j1), s1);
-    }
-    t.dst[(size_t)i0 * t.ldd + j0] = s0;
-    if (in1) t.dst[(size_t)i1 * t.ldd + j1] = s1;
+    if (w >= npiece) return;
+    const MixTask& t = tasks[piece_task[w]];
+    mix_piece<false>(t, (w - t.p0) * MIX_PIECE, srcs, threadIdx.x & 31);
 }
 
 __global__ void k_diag(const DiagTask* __restrict__ tasks, const DiagTerm* __restrict__ terms) {
@@ -558,7 +559,12 @@ void launch_gemm_tile(int tm, int tn, const GemmTask* tasks, int ntask, const Ge
 }
 
 void launch_mix(const MixTask* tasks, int ntask, const MixSrc* srcs, cudaStream_t st, const int* skip) {
-    if (ntask > 0) { counted(); k_mix<<<(ntask + 3) / 4, 128, 0, st>>>(tasks, ntask, srcs, skip); }
+    if (ntask > 0) { counted(); k_mix<<<ntask, 128, 0, st>>>(tasks, srcs, skip); }
+}
+
+void launch_mix_pieces(const MixTask* tasks, const unsigned* piece_task, int npiece, const MixSrc* srcs,
+                       cudaStream_t st, const int* skip) {
+    if (npiece > 0) { counted(); k_mix_pieces<<<(npiece + 3) / 4, 128, 0, st>>>(tasks, piece_task, npiece, srcs, skip); }
 }
 
 void launch_diag(const DiagTask* tasks, int ntask, const DiagTerm* terms, cudaStream_t st) {

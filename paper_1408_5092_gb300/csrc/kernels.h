@@ -74,13 +74,14 @@ struct MixSrc {
     int pad;
     double coef;
 };
-// The task covers the values [e0, e0 + MIX_PIECE) of the block, row by row.
+// For k_mix_pieces a block's values are cut, row by row, in pieces of MIX_PIECE;
+// p0 is the number of its first piece in the launch, piece_task[p] the task of p.
 constexpr int MIX_PIECE = 64;
 struct MixTask {
     double* dst;
     int rows, cols, ldd;
     int s0, s1;
-    int e0;
+    int p0;
 };
 
 // Jacobi diagonal of A_loc: out[l, r] += sum coef * L[l*(ldL+1)] * R[r*(ldR+1)]
@@ -166,6 +167,30 @@ void launch_gemm_tc(const GemmTask* tasks, int ntask, const GemmOp* ops, int* er
 // partial tiles and tick one zeroed counter per split tile (left at zero).
 void launch_dgemm(int tile, const GemmBlk* blks, const unsigned* unit_blk, int nunit, const GemmOp* ops, double* part,
                   unsigned* tick, cudaStream_t st, const int* skip = nullptr);
+// A grouped GEMM's device lists, 16 x 16 units (see launch_dgemm).
+struct GemmRun {
+    const GemmBlk* blk;
+    const unsigned* unit;
+    const GemmOp* ops;
+    double* part;
+    unsigned* tick;
+    int nunit;
+};
+// One CG solve (state after cg_init in *S): the operator as g1, operator sums,
+// g2 from p to Ap, the vectors of n, at most maxit iterations.
+struct CgArgs {
+    GemmRun g1, g2;
+    const MixTask* mt;
+    const MixSrc* ms;
+    int nmix, maxit;
+    double *x, *r, *z, *p;
+    const double *Ap, *minv;
+    size_t n;
+    CgState* S;
+};
+// The whole solve in one launch on one cluster; false: not available here.
+bool launch_cg_cluster(const CgArgs& a, cudaStream_t st);
+bool cg_cluster_available();
 // Float32 arithmetic on float64 data: grouped GEMM with output tile tm x tn
 // (64x64, 32x64, 64x32, 16x128, 32x32).  Persistent: at most the resident
 // CTAs are launched and each walks a stride of the task list.
@@ -173,8 +198,9 @@ bool gemm_tile_supported(int tm, int tn);
 void launch_splitk_reduce(const SplitRed* tasks, int ntask, cudaStream_t st, const int* skip = nullptr);
 void launch_gemm_tile(int tm, int tn, const GemmTask* tasks, int ntask, const GemmOp* ops, cudaStream_t st,
                       const int* skip = nullptr);
-void launch_mix(const MixTask* tasks, int ntask, const MixSrc* srcs, cudaStream_t st,
-                const int* skip = nullptr);
+void launch_mix(const MixTask* tasks, int ntask, const MixSrc* srcs, cudaStream_t st, const int* skip = nullptr);
+void launch_mix_pieces(const MixTask* tasks, const unsigned* piece_task, int npiece, const MixSrc* srcs,
+                       cudaStream_t st, const int* skip = nullptr);
 void launch_diag(const DiagTask* tasks, int ntask, const DiagTerm* terms, cudaStream_t st);
 // Float64 Jacobi of every matrix, at most maxs sweeps.  host: the same task
 // list on the host, in the order of order_eig_tasks (largest first, so that

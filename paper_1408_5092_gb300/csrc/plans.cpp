@@ -199,7 +199,15 @@ void GemmPlan::upload(cudaStream_t st) {
     if (kind == GEMM_F64) {
         size_t tk = 0;
         std::vector<long long> cm;
-        tile64 = tuner && !blocks.empty() ? (tm == 32 ? 32 : 16) : tile_rule();
+        steps = 0.0;
+        for (const Blk& b : blocks) {
+            long long q = 0;
+            for (int o = b.op0; o < b.op1; ++o) q += (ops[o].k + 3) / 4;
+            steps += (double)((b.m + 7) / 8) * ((b.n + 7) / 8) * q;
+        }
+        // (plans of few steps take the narrow units whatever the tuner found:
+        // the two differ by the launch alone there)
+        tile64 = steps <= kClusterSteps ? 16 : tuner && !blocks.empty() ? (tm == 32 ? 32 : 16) : tile_rule();
         units(tile64, gblk, unit_blk, &cm, &pe, &tk);
         for (size_t i = 0; i < gblk.size(); ++i) gblk[i].cmap = cm[i] >= 0 ? cbase + cm[i] : nullptr;
         workspace(pe, tk, st);
@@ -467,13 +475,16 @@ void Omega::build(const MPO& W, int i) {
     first[(size_t)Da * 16] = (int)e.size();
 }
 
-void mix_pieces(const std::vector<MixTask>& blocks, std::vector<MixTask>& out) {
-    out.clear();
-    for (const MixTask& b : blocks)
-        for (int e = 0, n = b.rows * b.cols; e < n; e += MIX_PIECE) {
-            out.push_back(b);
-            out.back().e0 = e;
-        }
+void mix_pieces(std::vector<MixTask>& tasks, std::vector<unsigned>& piece_task) {
+    int np = 0;
+    for (MixTask& t : tasks) {
+        t.p0 = np;
+        np += (t.rows * t.cols + MIX_PIECE - 1) / MIX_PIECE;
+    }
+    piece_task.resize(np);
+    for (size_t i = 0; i < tasks.size(); ++i)
+        std::fill(piece_task.begin() + tasks[i].p0,
+                  i + 1 < tasks.size() ? piece_task.begin() + tasks[i + 1].p0 : piece_task.end(), (unsigned)i);
 }
 
 void TwoSitePlan::build(const Omega& om, const TwoT& bra, const TwoT& ket, const Bond& braL,
@@ -665,8 +676,14 @@ void TwoSitePlan::build(const Omega& om, const TwoT& bra, const TwoT& ket, const
         check(Tp, tsize * sizeof(double), "mix T");
         for (const auto& t : mtasks) check(t.dst, ((size_t)(t.rows - 1) * t.ldd + t.cols) * sizeof(double), "mix dst");
     }
-    mix_pieces(mtasks, mpieces);
-    mpspt::upload(dmt, mpieces, st);
+    // Pieces cost the host their list and its copy, so they are made for the
+    // low-precision operator alone, which runs tens of times per list and has
+    // the large bonds: M = 256 35.3 -> 26.0 ms a sweep.  A float64 sweep at
+    // M = 64 gained 0.2 ms on the device and lost 4.5 ms on the host.
+    mpieces.clear();
+    if (is_tc(kind)) mix_pieces(mtasks, mpieces);
+    mpspt::upload(dmt, mtasks, st);
+    if (!mpieces.empty()) mpspt::upload(dmp, mpieces, st);
     mpspt::upload(dms, msrc, st);
     g1.upload(st);
     g2.upload(st);
@@ -736,8 +753,7 @@ void EnvPlan::upload_mix(cudaStream_t st) {
         RangeCheck check;
         for (const auto& t : mt) check(t.dst, ((size_t)(t.rows - 1) * t.ldd + t.cols) * sizeof(double), "env mix dst");
     }
-    mix_pieces(mt, mp);
-    mpspt::upload(dmt, mp, st);
+    mpspt::upload(dmt, mt, st);
     mpspt::upload(dms, ms, st);
     g1.upload(st);
     g2.upload(st);

@@ -19,7 +19,7 @@ inline bool is_tc(int kind) { return kind == GEMM_TC || kind == GEMM_TC16; }
 struct GemmPlan;
 
 // Task list of k_mix for the planned blocks: one task per piece of a block.
-void mix_pieces(const std::vector<MixTask>& blocks, std::vector<MixTask>& out);
+void mix_pieces(std::vector<MixTask>& tasks, std::vector<unsigned>& piece_task);
 
 // Tile-shape autotuner of the float64 and float32 grouped GEMMs.  A plan's
 // shape class is (arithmetic, skinny, and log2 buckets of the median block
@@ -55,6 +55,11 @@ struct Autotuner {
     void load(const std::string& path);
     void save(const std::string& path);
 };
+
+// DMMA steps (8 x 8 x 4) up to which one local operator is applied inside the
+// cluster solve (see launch_cg_cluster): 16 SMs against all of them, but no
+// launches.
+constexpr double kClusterSteps = 1200.0;
 
 struct GemmPlan {
     int tm = GEMM_TM, tn = GEMM_TN;   // output tile (TC kernel: 128 x 64; skinny: 16 x 128)
@@ -131,6 +136,13 @@ struct GemmPlan {
                int cmap_rows = 0);
     void upload(cudaStream_t st);
     void run(cudaStream_t st) const;
+    // float64: DMMA steps of one run, and its lists for a kernel that runs
+    // them itself (16 x 16 units only)
+    double steps = 0.0;
+    GemmRun lists() const {
+        return {dgblk.as<GemmBlk>(), dunit.as<unsigned>(), dops.as<GemmOp>(), dpart.as<double>(), dtick.as<unsigned>(),
+                (int)unit_blk.size()};
+    }
 };
 
 // Two-site operator sum_{a,c} L_a (Omega_ac) R_c with Omega_ac = sum_b W1_ab (x) W2_bc.
@@ -154,9 +166,10 @@ struct Omega {
 //        sector, scattered into the two-site layout by a column map
 struct TwoSitePlan {
     GemmPlan g1, g2, g2s;            // g2s: the float32 blocks of few rows (skinny tiles)
-    std::vector<MixTask> mtasks, mpieces;
+    std::vector<MixTask> mtasks;
+    std::vector<unsigned> mpieces;
     std::vector<MixSrc> msrc;
-    DBuf dmt, dms;
+    DBuf dmt, dmp, dms;
     DBuf T, V, Lp, Rp, pk;
     size_t tsize = 0;
     int kind = GEMM_F64;
@@ -175,11 +188,16 @@ struct TwoSitePlan {
                cudaStream_t st);
     void run(cudaStream_t st) const {
         g1.run(st);
-        launch_mix(dmt.as<MixTask>(), (int)mpieces.size(), dms.as<MixSrc>(), st, skip);
+        if (mpieces.empty()) launch_mix(dmt.as<MixTask>(), (int)mtasks.size(), dms.as<MixSrc>(), st, skip);
+        else launch_mix_pieces(dmt.as<MixTask>(), dmp.as<unsigned>(), (int)mpieces.size(), dms.as<MixSrc>(), st, skip);
         g2.run(st);
         g2s.run(st);
     }
     double flops() const { return g1.flops + g2.flops + g2s.flops; }
+    // The operator small enough for the cluster solve
+    bool for_cluster() const {
+        return kind == GEMM_F64 && g1.tile64 == 16 && g2.tile64 == 16 && g1.steps + g2.steps <= kClusterSteps;
+    }
 };
 
 // Jacobi diagonal of sum L_a Omega_ac R_c on the bra layout.
@@ -207,7 +225,7 @@ struct EnvPlan {
     GemmPlan g1, g2;
     void set_tuner(Autotuner* t) { g1.tuner = t; g2.tuner = t; }
     DBuf Y, Z, dmt, dms;
-    std::vector<MixTask> mt, mp;
+    std::vector<MixTask> mt;
     std::vector<MixSrc> ms;
     void build_left(const MPO& W, int site, const EnvT& L, const SiteT& Abra, const SiteT& Aket,
                     const Bond& braL, const Bond& ketL, const Bond& braR, const Bond& ketR,
@@ -221,14 +239,14 @@ struct EnvPlan {
                         cudaStream_t st);
     void run(cudaStream_t st) const {
         g1.run(st);
-        launch_mix(dmt.as<MixTask>(), (int)mp.size(), dms.as<MixSrc>(), st);
+        launch_mix(dmt.as<MixTask>(), (int)mt.size(), dms.as<MixSrc>(), st);
         g2.run(st);
     }
     double flops() const { return g1.flops + g2.flops; }
     // bytes of the task lists the last build uploads (GEMM tasks and operand
     // lists, mix tasks and sources)
     size_t plan_bytes() const {
-        return mp.size() * sizeof(MixTask) + ms.size() * sizeof(MixSrc) +
+        return mt.size() * sizeof(MixTask) + ms.size() * sizeof(MixSrc) +
                (g1.gblk.size() + g2.gblk.size()) * sizeof(GemmBlk) +
                (g1.unit_blk.size() + g2.unit_blk.size()) * sizeof(unsigned) +
                (g1.ops.size() + g2.ops.size()) * sizeof(GemmOp);
