@@ -1191,38 +1191,71 @@ struct Sweeper {
     double solve_plain(size_t n) {
         double* x = w.x.as<double>();
         CgState* S = ln.cg.as<CgState>();
-        MPSPT_CUDA(cudaMemcpyAsync(w.p.get(), x, n * sizeof(double), cudaMemcpyDeviceToDevice, ln.st));
-        sigma64();
-        cg_init(w.r.as<double>(), w.z.as<double>(), w.p.as<double>(), w.b.as<double>(), w.Ap.as<double>(),
-                w.minv.as<double>(), n, S, c.opt.cg_tol, ln.red.as<double>(), ln.cnt.as<unsigned>(), ln.st);
-        sync_state();
         int launched = 0;
-        sig.set_skip(&S->done);
-        if (c.opt.cuda_graphs && ln.st != nullptr && !ln.cg_host->done) {
-            capture(gexec, [&] {
-                for (int q = 0; q < kChunk; ++q) {
-                    sig.run(ln.st);
+        // (partition lanes hide the launches behind one another, and 16 whole
+        // SMs of one cluster are rarely free beside them: 12 partitions on 8
+        // lanes took 164 -> 168 ms with clusters)
+        if (&ln == c.lane0.get() && sig.for_cluster() && cg_cluster_available()) {
+            // start, all iterations and the state in one go; with graphs as
+            // one graph launch (whose iterations come in chunks)
+            const bool graph = c.opt.cuda_graphs && ln.st != nullptr;
+            const int maxit = graph ? (c.opt.cg_max_iter + kChunk - 1) / kChunk * kChunk : c.opt.cg_max_iter;
+            const CgArgs args{sig.g1.lists(), sig.g2.lists(), sig.dmt.as<MixTask>(), sig.dms.as<MixSrc>(),
+                              (int)sig.mtasks.size(), maxit, x, w.r.as<double>(), w.z.as<double>(),
+                              w.p.as<double>(), w.Ap.as<double>(), w.minv.as<double>(), n, S};
+            auto body = [&] {
+                MPSPT_CUDA(cudaMemcpyAsync(w.p.get(), x, n * sizeof(double), cudaMemcpyDeviceToDevice, ln.st));
+                sig.run(ln.st);
+                cg_init(w.r.as<double>(), w.z.as<double>(), w.p.as<double>(), w.b.as<double>(), w.Ap.as<double>(),
+                        w.minv.as<double>(), n, S, c.opt.cg_tol, ln.red.as<double>(), ln.cnt.as<unsigned>(), ln.st);
+                if (!launch_cg_cluster(args, ln.st)) throw Error(MPSPT_ERR_CUDA, "cluster solve: launch failed");
+            };
+            ev_begin();
+            if (graph) {
+                capture(gexec, body);
+                MPSPT_CUDA(cudaGraphLaunch(gexec, ln.st));
+                count_launch();
+            } else {
+                body();
+            }
+            ev_end(true);
+            sync_state();
+            launched = ln.cg_host->iters;
+            res->sigma64_calls += 1 + launched;
+            res->sigma64_flops += (1 + launched) * sig.flops();
+        } else {
+            MPSPT_CUDA(cudaMemcpyAsync(w.p.get(), x, n * sizeof(double), cudaMemcpyDeviceToDevice, ln.st));
+            sigma64();
+            cg_init(w.r.as<double>(), w.z.as<double>(), w.p.as<double>(), w.b.as<double>(), w.Ap.as<double>(),
+                    w.minv.as<double>(), n, S, c.opt.cg_tol, ln.red.as<double>(), ln.cnt.as<unsigned>(), ln.st);
+            sync_state();
+            sig.set_skip(&S->done);
+            if (c.opt.cuda_graphs && ln.st != nullptr && !ln.cg_host->done) {
+                capture(gexec, [&] {
+                    for (int q = 0; q < kChunk; ++q) {
+                        sig.run(ln.st);
+                        cg_step(x, w.r.as<double>(), w.z.as<double>(), w.p.as<double>(), w.Ap.as<double>(),
+                                w.minv.as<double>(), n, S, ln.red.as<double>(), ln.cnt.as<unsigned>(), ln.st);
+                    }
+                });
+                while (!ln.cg_host->done && launched < c.opt.cg_max_iter) {
+                    launch_graph(gexec, true, sig.flops());
+                    launched += kChunk;
+                    sync_state();
+                }
+            }
+            while (!ln.cg_host->done && launched < c.opt.cg_max_iter) {
+                const int chunk = std::min(c.opt.cg_max_iter - launched, launched < 8 ? 4 : 8);
+                for (int q = 0; q < chunk; ++q) {
+                    sigma64();
                     cg_step(x, w.r.as<double>(), w.z.as<double>(), w.p.as<double>(), w.Ap.as<double>(),
                             w.minv.as<double>(), n, S, ln.red.as<double>(), ln.cnt.as<unsigned>(), ln.st);
                 }
-            });
-            while (!ln.cg_host->done && launched < c.opt.cg_max_iter) {
-                launch_graph(gexec, true, sig.flops());
-                launched += kChunk;
+                launched += chunk;
                 sync_state();
             }
+            sig.set_skip(nullptr);
         }
-        while (!ln.cg_host->done && launched < c.opt.cg_max_iter) {
-            const int chunk = std::min(c.opt.cg_max_iter - launched, launched < 8 ? 4 : 8);
-            for (int q = 0; q < chunk; ++q) {
-                sigma64();
-                cg_step(x, w.r.as<double>(), w.z.as<double>(), w.p.as<double>(), w.Ap.as<double>(),
-                        w.minv.as<double>(), n, S, ln.red.as<double>(), ln.cnt.as<unsigned>(), ln.st);
-            }
-            launched += chunk;
-            sync_state();
-        }
-        sig.set_skip(nullptr);
         require(!ln.cg_host->not_spd, "CG: p^T A p <= 0 (H0 - E0 not positive on the local space)",
                 MPSPT_ERR_NOT_SPD);
         require(ln.cg_host->done != 0, "local CG reached cg_max_iter before the residual test",
