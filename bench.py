@@ -205,7 +205,7 @@ def _fp64_roofline(reps, peaks, src):
     return {"bound": "fp64_alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
             "frac": ach / peak if peak else None, "traffic": None,
             "peak_source": f"{src} bf16 burst x nominal fp64/bf16 ratio",
-            "kernel": "k_gemm<64, 64, double> (float64 refinement sigma)"}
+            "kernel": "k_dgemm (float64 refinement sigma)"}
 
 
 def run_reference(args):
@@ -404,7 +404,7 @@ def run_gpu(args):
         "roofline": {"bound": "fp64_alu" if args.prec == "fp64" else "tensor", "achieved": achieved,
                      "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak if peak else None,
                      "traffic": traffic, "peak_source": peak_note,
-                     "kernel": "k_gemm (sigma grouped block GEMM)"},
+                     "kernel": "grouped block GEMM of sigma"},
         "roofline_fp64_sigma": _fp64_roofline(reps, peaks, src),
         "e2e": {"value": e2e, "unit": "s", "runs": args.e2e_steps,
                 "what": "wall clock mpspt_create -> set_integrals -> set_reference_ci -> minimize_hylleraas "

@@ -395,7 +395,7 @@ mpspt_status mpspt_eigh_batched_ex(int device, void* stream, int batch, const in
  * around their accounting, and latency-bound callers that cannot afford the
  * synchronisation a fresh allocation may cost).  Same arguments, results and
  * stream ordering as mpspt_eigh_batched, but the task table and the work
- * copy of A live in one fixed device array of 2^21 doubles (16 MiB) that
+ * copies of large matrices live in one fixed device array of 2^21 doubles (16 MiB) that
  * every GPU loading the library holds until the process exits; the call
  * allocates and frees nothing.  Limits: batch <= 1024 and
  * sum_i n[i]^2 <= 2^21 - 4096 (else MPSPT_ERR_INVALID, nothing launched).

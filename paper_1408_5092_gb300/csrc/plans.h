@@ -18,7 +18,7 @@ inline bool is_tc(int kind) { return kind == GEMM_TC || kind == GEMM_TC16; }
 
 struct GemmPlan;
 
-// Task list of k_mix for the planned blocks: one task per piece of a block.
+// Piece list of k_mix_pieces for the planned blocks (sets their p0).
 void mix_pieces(std::vector<MixTask>& tasks, std::vector<unsigned>& piece_task);
 
 // Tile-shape autotuner of the float64 and float32 grouped GEMMs.  A plan's
