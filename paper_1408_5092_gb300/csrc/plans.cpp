@@ -678,8 +678,9 @@ void TwoSitePlan::build(const Omega& om, const TwoT& bra, const TwoT& ket, const
     }
     // Pieces cost the host their list and its copy, so they are made for the
     // low-precision operator alone, which runs tens of times per list and has
-    // the large bonds: M = 256 35.3 -> 26.0 ms a sweep.  A float64 sweep at
-    // M = 64 gained 0.2 ms on the device and lost 4.5 ms on the host.
+    // the large bonds: M = 256 35.3 -> 29.3 ms of block sums a sweep (26.0
+    // with every plan in pieces).  A float64 sweep at M = 64 gained 0.2 ms on
+    // the device and lost 4.4 ms a pass.
     mpieces.clear();
     if (is_tc(kind)) mix_pieces(mtasks, mpieces);
     mpspt::upload(dmt, mtasks, st);
