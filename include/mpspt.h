@@ -371,7 +371,8 @@ mpspt_status mpspt_train_preconditioner(mpspt_ctx* ctx, mpspt_h0 h0, int M, int 
  * the column order of V, unsorted).  Work is ordered on `stream`
  * (cudaStream_t, 0 = default); the call allocates its task list (and a work
  * copy of matrices too large for the on-chip solver, n above about 590) with
- * cudaMallocAsync on that stream and returns without synchronising. */
+ * cudaMallocAsync on that stream and returns without synchronising.  A
+ * matrix with an infinity or a NaN gives NaN in all of its w and V. */
 mpspt_status mpspt_eigh_batched(int device, void* stream, int batch, const int* n, const double* A,
                                 double* V, double* w);
 
@@ -384,7 +385,9 @@ mpspt_status mpspt_eigh_batched(int device, void* stream, int batch, const int* 
  * V <- V R with float64 rotations, until float32 leaves nothing above
  * float64 rounding.  A is left unchanged.  Allocates device scratch
  * (about 25 n^2 doubles per matrix, rotation lists included) and returns
- * after the stream has finished the work. */
+ * after the stream has finished the work.  A matrix that does not pass the
+ * convergence test (one with an infinity or a NaN among them) gives
+ * MPSPT_ERR_NOT_CONVERGED. */
 mpspt_status mpspt_eigh_batched_ex(int device, void* stream, int batch, const int* n, const double* A,
                                    double* V, double* w, int f32_start);
 

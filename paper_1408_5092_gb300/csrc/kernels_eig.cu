@@ -65,6 +65,12 @@ struct Tol {
     static constexpr double gain = 1e-11, last = 1e-18;
 };
 
+// Scale of a matrix with an infinity or a NaN (largest exponent 2047).  Such a
+// matrix has no eigenvalues, and float32 norms of scaled entries cannot show it
+// (an entry 2^-1025 of its value is zero), so it is told by the exponent: flag
+// 2 and w (from the float64 solver V too) filled with NaN.
+constexpr int kNonFinite = 0x7FF - 1022;
+
 __host__ __device__ inline size_t align16(size_t b) { return (b + 15) & ~(size_t)15; }
 
 // ---------------------------------------------------------------- mixed
@@ -123,6 +129,16 @@ __global__ void __launch_bounds__(NT) k_jac_mixed(const JacTask* __restrict__ ta
         __syncthreads();
     }
     const int sh = shift;
+    if (sh == kNonFinite) {   // no rotation in the start, so that B is not finite either and the polish says so
+        if (tid == 0) {
+            *t.nsw = 0;
+            *t.total = 0;
+            *t.done = POLISH ? 2 : 0;
+        }
+        if (t.w)
+            for (int i = tid; i < n; i += NT) t.w[i] = nan("");
+        return;
+    }
     for (int e = tid; e < np; e += NT) E[e] = 0.f;
     for (int e = tid; e < m; e += NT) D[e] = DT(0);
     __syncthreads();
@@ -213,7 +229,7 @@ __global__ void __launch_bounds__(NT) k_jac_mixed(const JacTask* __restrict__ ta
             if (tid == 0) {
                 double b = 0.0;
                 for (int w = 0; w < NW; ++w) b += red[1][w];
-                so = fmax(0.0, so - 2.0 * b);
+                so = so - 2.0 * b < 0.0 ? 0.0 : so - 2.0 * b;
             }
         }
         if (tid == 0) {
@@ -455,6 +471,12 @@ __device__ __forceinline__ void eig_body(const EigTask& t, double nullrel, int m
     sync();   // (in place: nobody scales an entry before all have looked)
     for (int w = 0; w < NW; ++w) mx = max(mx, __float_as_uint(red[0][w]));
     const int sh = mx == 0 ? 0 : (int)mx - 1022;
+    if (sh == kNonFinite) {   // the same in every CTA
+        for (int i = rank * NT + tid; i < n; i += C * NT) t.w[i] = nan("");
+        for (size_t e = (size_t)rank * NT + tid; e < (size_t)n * n; e += (size_t)C * NT) t.V[e] = nan("");
+        if (flag && rank == 0 && tid == 0) *flag = 2;
+        return;
+    }
     for (int i = warp; i < n; i += NW)
         for (int j = i + lane; j < n; j += 32) {
             const int e = rowoff[i] + j;
