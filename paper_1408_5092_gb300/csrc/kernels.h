@@ -204,7 +204,7 @@ void launch_mix_pieces(const MixTask* tasks, const unsigned* piece_task, int npi
 void launch_diag(const DiagTask* tasks, int ntask, const DiagTerm* terms, cudaStream_t st);
 // Float64 Jacobi of every matrix, at most maxs sweeps.  host: the same task
 // list on the host, in the order of order_eig_tasks (largest first, so that
-// each of the two kernels gets one launch).  null_rule: pairs below
+// each kernel gets one launch; which kernel: eig_route.h).  null_rule: pairs below
 // 1e-14 |A|_F are left alone; flags (nullable): 1 converged, 2 stopped by the
 // cap.
 void order_eig_tasks(EigTask* tasks, int ntask);

@@ -32,6 +32,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "eig_route.h"
 #include "jac_rot.h"
 #include "jacobi_schedule.h"
 #include "kernels.h"
@@ -71,7 +72,7 @@ struct Tol {
 // 2 and w (from the float64 solver V too) filled with NaN.
 constexpr int kNonFinite = 0x7FF - 1022;
 
-__host__ __device__ inline size_t align16(size_t b) { return (b + 15) & ~(size_t)15; }
+__host__ __device__ constexpr size_t align16(size_t b) { return (b + 15) & ~(size_t)15; }
 
 // ---------------------------------------------------------------- mixed
 constexpr int MIX_SMEM = 230000;
@@ -413,8 +414,8 @@ __global__ void __launch_bounds__(32 * JAC_APPLY_ROWS) k_jac_apply(const JacTask
 constexpr int JC = 8;
 
 struct EigFit { size_t head, a, v; };   // shared memory of one CTA: head, triangle share, V rows
-__host__ __device__ inline EigFit eig_fit(int n, int C) {
-    EigFit f;
+__host__ __device__ constexpr EigFit eig_fit(int n, int C) {
+    EigFit f{};
     const size_t half = (size_t)(n + 1) / 2;
     // rowoff, slots, (c, s, tan) and the rotated pairs' blocks, the diagonal
     f.head = align16((size_t)n * 4) + align16(half * 8) + align16(half * 48) + align16((size_t)n * 8);
@@ -422,8 +423,9 @@ __host__ __device__ inline EigFit eig_fit(int n, int C) {
     f.v = align16(((size_t)n + C - 1) / C * n * 8);
     return f;
 }
-__host__ __device__ inline bool eig_a_sm(int n, int C) { const EigFit f = eig_fit(n, C); return f.head + f.a <= (size_t)JAC_SMEM; }
-__host__ __device__ inline bool eig_v_sm(int n, int C) { const EigFit f = eig_fit(n, C); return f.head + f.a + f.v <= (size_t)JAC_SMEM; }
+__host__ __device__ constexpr bool eig_a_sm(int n, int C) { const EigFit f = eig_fit(n, C); return f.head + f.a <= (size_t)JAC_SMEM; }
+__host__ __device__ constexpr bool eig_v_sm(int n, int C) { const EigFit f = eig_fit(n, C); return f.head + f.a + f.v <= (size_t)JAC_SMEM; }
+static_assert(eig_a_sm(kEigOneMaxN, 1) && !eig_a_sm(kEigOneMaxN + 5, 1), "largest matrix of one CTA");
 inline size_t eig_smem(int n, int C) {
     const EigFit f = eig_fit(n, C);
     return f.head + (eig_a_sm(n, C) ? f.a : 0) + (eig_v_sm(n, C) ? f.v : 0);
@@ -649,8 +651,9 @@ __device__ __forceinline__ void eig_body(const EigTask& t, double nullrel, int m
     if constexpr (C > 1) cg::this_cluster().sync();   // no CTA leaves while its shared memory may be read
 }
 
-__global__ void __launch_bounds__(128) k_eig_one(const EigTask* __restrict__ tasks, double nullrel, int maxs, int* flags) {
-    eig_body<1, 128, true>(tasks[blockIdx.x], nullrel, maxs, flags ? flags + blockIdx.x : nullptr, 0);
+template <int NT>
+__global__ void __launch_bounds__(NT) k_eig_one(const EigTask* __restrict__ tasks, double nullrel, int maxs, int* flags) {
+    eig_body<1, NT, true>(tasks[blockIdx.x], nullrel, maxs, flags ? flags + blockIdx.x : nullptr, 0);
 }
 __global__ void __cluster_dims__(JC, 1, 1) __launch_bounds__(256)
     k_eig_cl(const EigTask* __restrict__ tasks, double nullrel, int maxs, int* flags) {
@@ -704,36 +707,40 @@ void launch_jac_rot64(const JacTask* tasks, int ntask, cudaStream_t st) {
     }
 }
 
-// One CTA below n = 28, a cluster of 8 from there (measured, eight matrices:
-// n = 23 and 24 both 0.5 ms, n = 31 and 32 on the cluster 0.8 ms).
-bool eig_on_cluster(int n) { return n >= 28; }
-bool eig_in_place(int n) { return eig_on_cluster(n) && !eig_a_sm(n, JC); }
+bool eig_in_place(int n) { return !eig_a_sm(n, JC); }
 
 void order_eig_tasks(EigTask* tasks, int ntask) {
     std::stable_sort(tasks, tasks + ntask, [](const EigTask& x, const EigTask& y) { return x.n > y.n; });
 }
 
+template <int NT>
+static void launch_eig_one(const EigTask* tasks, int ntask, size_t smem, double nullrel, int maxs, int* flags,
+                           cudaStream_t st) {
+    ensure_smem_attr(reinterpret_cast<const void*>(k_eig_one<NT>), JAC_SMEM);
+    k_eig_one<NT><<<ntask, NT, smem, st>>>(tasks, nullrel, maxs, flags);
+}
+
 void launch_eig(const EigTask* tasks, const EigTask* host, int ntask, bool null_rule, int maxs, int* flags,
                 cudaStream_t st) {
     const double nullrel = null_rule ? Tol::null : 0.0;
-    int ncl = 0;
-    size_t smem = 0, smem1 = 0;
-    for (int i = 0; i < ntask; ++i) {
-        if (eig_on_cluster(host[i].n)) {
-            ncl = i + 1;
-            smem = std::max(smem, eig_smem(host[i].n, JC));
+    const int mid = eig_mid_threads_of(ntask, [host](int i) { return host[i].n; });
+    for (int i = 0, j; i < ntask; i = j) {   // matrices i to j - 1 take the same kernel
+        const int nt = eig_threads(host[i].n, mid);
+        const int C = nt == 0 ? JC : 1;
+        size_t smem = 0;
+        for (j = i; j < ntask && eig_threads(host[j].n, mid) == nt; ++j) smem = std::max(smem, eig_smem(host[j].n, C));
+        int* fl = flags ? flags + i : nullptr;
+        count_launch();
+        if (nt == 0) {
+            ensure_smem_attr(reinterpret_cast<const void*>(k_eig_cl), JAC_SMEM);
+            k_eig_cl<<<(j - i) * JC, 256, smem, st>>>(tasks + i, nullrel, maxs, fl);
+        } else if (nt == 512) {
+            launch_eig_one<512>(tasks + i, j - i, smem, nullrel, maxs, fl, st);
+        } else if (nt == 256) {
+            launch_eig_one<256>(tasks + i, j - i, smem, nullrel, maxs, fl, st);
         } else {
-            smem1 = std::max(smem1, eig_smem(host[i].n, 1));
+            launch_eig_one<128>(tasks + i, j - i, smem, nullrel, maxs, fl, st);
         }
-    }
-    if (ncl > 0) {
-        ensure_smem_attr(reinterpret_cast<const void*>(k_eig_cl), JAC_SMEM);
-        count_launch();
-        k_eig_cl<<<ncl * JC, 256, smem, st>>>(tasks, nullrel, maxs, flags);
-    }
-    if (ncl < ntask) {
-        count_launch();
-        k_eig_one<<<ntask - ncl, 128, smem1, st>>>(tasks + ncl, nullrel, maxs, flags ? flags + ncl : nullptr);
     }
 }
 
