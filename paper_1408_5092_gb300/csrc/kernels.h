@@ -115,7 +115,7 @@ struct JacTask {
     double* w;         // n eigenvalues (unsorted), or null
     void* P;           // scratch for n beyond shared memory: the two float32 triangles
     float2* rot;       // mixed sweeps: (c, s), or (tan, 0) in the polish
-    double2* rot64;    // float64 (c, s)
+    double2* rot64;    // float64 (tangent of the half angle, s)
     int* done;         // 1: converged
     int* nsw;          // sweeps in the lists of the last launch
     int* total;        // sweeps performed so far

@@ -15,7 +15,7 @@
 // addresses are computed once per launch and kept in registers.  The update
 // moves 32 bytes of shared memory per block, 940 clocks a round at n = 173;
 // the pair phase and two barriers are the rest.
-// k_jac_rot64: the float64 (c, s) of the recorded float32 tangents.
+// k_jac_rot64: the float64 rotations (jac_rot.h) of the recorded float32 tangents.
 // k_jac_apply (a warp per row of V): V <- V R over the recorded lists; a row
 // is touched independently of the others, the rotations of a round act on
 // disjoint columns and take one lane each.
@@ -331,9 +331,12 @@ __global__ void k_jac_rot64(const JacTask* __restrict__ tasks) {
     const size_t tot = (size_t)*t.nsw * (m - 1) * (m / 2);
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < tot; i += (size_t)gridDim.x * blockDim.x) {
         const float tn = t.rot[i].x;
-        double c = 1.0, s = (double)tn;
-        if (fabsf(tn) > 1e-9f) jac_cs64(s, c, s);   // below, c rounds to 1 and s to t
-        t.rot64[i] = make_double2(c, s);
+        double s = (double)tn, h = 0.5 * s;
+        if (fabsf(tn) > 1e-9f) {   // below, they round to these
+            h = jac_half64(tn, 0.f);
+            s = jac_sine64(h);
+        }
+        t.rot64[i] = make_double2(h, s);
     }
 }
 
@@ -377,8 +380,13 @@ __global__ void __launch_bounds__(32 * JAC_APPLY_ROWS) k_jac_apply(const JacTask
         pa = k == 0 ? 0 : (pa >= rounds ? pa - rounds : pa) + 1;
         pb = (pb >= rounds ? pb - rounds : pb) + 1;
         const T x = R[pa], y = R[pb];
-        R[pa] = cs.x * x - cs.y * y;
-        R[pb] = cs.y * x + cs.x * y;
+        if constexpr (sizeof(T) == 8) {
+            R[pa] = rot_first(cs.y, cs.x, x, y);
+            R[pb] = rot_second(cs.y, cs.x, x, y);
+        } else {
+            R[pa] = cs.x * x - cs.y * y;
+            R[pb] = cs.y * x + cs.x * y;
+        }
     };
     fetch(0);
     int r = 0;
@@ -417,8 +425,8 @@ struct EigFit { size_t head, a, v; };   // shared memory of one CTA: head, trian
 __host__ __device__ constexpr EigFit eig_fit(int n, int C) {
     EigFit f{};
     const size_t half = (size_t)(n + 1) / 2;
-    // rowoff, slots, (c, s, tan) and the rotated pairs' blocks, the diagonal
-    f.head = align16((size_t)n * 4) + align16(half * 8) + align16(half * 48) + align16((size_t)n * 8);
+    // rowoff, slots, (s, h) and the rotated pairs' blocks, the diagonal
+    f.head = align16((size_t)n * 4) + align16(half * 8) + align16(half * 40) + align16((size_t)n * 8);
     f.a = align16(((size_t)n * (n + 1) / 2 + C - 1) / C * 8);
     f.v = align16(((size_t)n + C - 1) / C * n * 8);
     return f;
@@ -444,11 +452,10 @@ __device__ __forceinline__ void eig_body(const EigTask& t, double nullrel, int m
     const EigFit fit = eig_fit(n, C);
     int* rowoff = reinterpret_cast<int*>(sm);
     int2* slots = reinterpret_cast<int2*>(sm + align16((size_t)n * 4));   // (p, q); q < 0: not rotated
-    double* Cc = reinterpret_cast<double*>(sm + align16((size_t)n * 4) + align16((size_t)half * 8));
-    double *Ss = Cc + half, *Xa = Ss + half, *Xe = Xa + half, *Xb = Xe + half;
-    double* Tt = Xb + half;
+    double* Ss = reinterpret_cast<double*>(sm + align16((size_t)n * 4) + align16((size_t)half * 8));
+    double *Hh = Ss + half, *Xa = Hh + half, *Xe = Xa + half, *Xb = Xe + half;
     double* dg = reinterpret_cast<double*>(sm + align16((size_t)n * 4) + align16((size_t)half * 8) +
-                                           align16((size_t)half * 48));
+                                           align16((size_t)half * 40));
     double* Ploc = reinterpret_cast<double*>(sm + fit.head);
     const int nrow = (n - rank + C - 1) / C;          // this CTA's rows of V
     double* Vl = v_sm ? reinterpret_cast<double*>(sm + fit.head + fit.a) : t.V + (size_t)rank * n;
@@ -560,21 +567,21 @@ __device__ __forceinline__ void eig_body(const EigTask& t, double nullrel, int m
                     on = fe != 0.f && !jac_negligible(e, a, b) &&
                          !(abs_below(e, nullv) && abs_below(a, nullv) && abs_below(b, nullv));
                     if (on) {
-                        const double tn = jac_tan64(b - a, e, fd, fe);
-                        double c, s;
-                        jac_cs64(tn, c, s);
-                        Cc[k] = c; Ss[k] = s; Tt[k] = tn;
+                        const float tn = jac_tan(fd, fe);
+                        const double h = jac_half64(tn, jac_newton(b - a, e, fd, fe, tn));
+                        Hh[k] = h;
+                        Ss[k] = jac_sine64(h);
                         Xa[k] = a; Xe[k] = e; Xb[k] = b;
                     }
                 }
-                if (!on) { Cc[k] = 1.0; Ss[k] = 0.0; }
+                if (!on) { Ss[k] = 0.0; Hh[k] = 0.0; }
                 slots[k] = make_int2(p | (on ? 1 << 16 : 0), q < n ? q : -1);
             }
             sync();   // every CTA has read the pair entries before any is updated
             auto block = [&](int k, int l) {
                 const int2 sk_ = slots[k], sl_ = slots[l];
                 if (((sk_.x | sl_.x) >> 16) == 0) return;
-                const double ck = Cc[k], sk = Ss[k], cl = Cc[l], sl = Ss[l];
+                const double sk = Ss[k], hk = Hh[k], sl = Ss[l], hl = Hh[l];
                 const int p = sk_.x & 0xffff, q = sk_.y, u = sl_.x & 0xffff, v = sl_.y;
                 const bool hq = q >= 0, hv = v >= 0;
                 // a missing partner (odd n) reads the pair's own entry with s = 0
@@ -583,12 +590,12 @@ __device__ __forceinline__ void eig_body(const EigTask& t, double nullrel, int m
                 double& qu = at(hq ? q : p, u);
                 double& qv = at(hq ? q : p, hv ? v : u);
                 const double a_pu = pu, a_pv = pv, a_qu = qu, a_qv = qv;
-                const double r_pu = fma(ck, a_pu, -(sk * a_qu)), r_qu = fma(sk, a_pu, ck * a_qu);
-                const double r_pv = fma(ck, a_pv, -(sk * a_qv)), r_qv = fma(sk, a_pv, ck * a_qv);
-                if (hq && hv) qv = fma(sl, r_qu, cl * r_qv);
-                if (hq) qu = fma(cl, r_qu, -(sl * r_qv));
-                if (hv) pv = fma(sl, r_pu, cl * r_pv);
-                pu = fma(cl, r_pu, -(sl * r_pv));
+                const double r_pu = rot_first(sk, hk, a_pu, a_qu), r_qu = rot_second(sk, hk, a_pu, a_qu);
+                const double r_pv = rot_first(sk, hk, a_pv, a_qv), r_qv = rot_second(sk, hk, a_pv, a_qv);
+                if (hq && hv) qv = rot_second(sl, hl, r_qu, r_qv);
+                if (hq) qu = rot_first(sl, hl, r_qu, r_qv);
+                if (hv) pv = rot_second(sl, hl, r_pu, r_pv);
+                pu = rot_first(sl, hl, r_pu, r_pv);
             };
             if (C == 1 && 4 * nblk <= NT) {
                 // few blocks: a thread per entry (six operations instead of
@@ -601,12 +608,14 @@ __device__ __forceinline__ void eig_body(const EigTask& t, double nullrel, int m
                     const int p = sk_.x & 0xffff, q = sk_.y, u = sl_.x & 0xffff, v = sl_.y;
                     const bool lo = tid & 1, ro = tid & 2;
                     if ((!lo || q >= 0) && (!ro || v >= 0) && ((sk_.x | sl_.x) >> 16)) {
-                        const double ck = Cc[ek], sk = Ss[ek], cl = Cc[el], sl = Ss[el];
+                        const double sk = lo ? Ss[ek] : -Ss[ek], hk = lo ? -Hh[ek] : Hh[ek];
+                        const double sl = ro ? Ss[el] : -Ss[el], hl = ro ? -Hh[el] : Hh[el];
                         const int q_ = q >= 0 ? q : p, v_ = v >= 0 ? v : u;
-                        const double a_pu = at(p, u), a_pv = at(p, v_), a_qu = at(q_, u), a_qv = at(q_, v_);
-                        const double al = lo ? sk : ck, be = lo ? ck : -sk, ga = ro ? sl : cl, de = ro ? cl : -sl;
-                        const double x = fma(al, a_pu, be * a_qu), y = fma(al, a_pv, be * a_qv);
-                        out = fma(ga, x, de * y);
+                        const int p1 = lo ? q_ : p, p2 = lo ? p : q_;   // the entry's own row and the other
+                        const double xu = at(p1, u), xv = at(p1, v_), yu = at(p2, u), yv = at(p2, v_);
+                        const double ru = fma(sk, fma(hk, xu, yu), xu), rv = fma(sk, fma(hk, xv, yv), xv);
+                        const double own = ro ? rv : ru, other = ro ? ru : rv;
+                        out = fma(sl, fma(hl, own, other), own);
                         dst = &at(lo ? q : p, ro ? v : u);
                     }
                 }
@@ -625,7 +634,7 @@ __device__ __forceinline__ void eig_body(const EigTask& t, double nullrel, int m
                 if (k % C == rank && (slots[k].x >> 16)) {   // the rotated pairs' own blocks
                     const int p = slots[k].x & 0xffff, q = slots[k].y;
                     double a = Xa[k], e = Xe[k], b = Xb[k];
-                    jac_block64(Tt[k], Cc[k], a, e, b);
+                    jac_block64(Ss[k], Hh[k], a, e, b);
                     at(p, p) = a;
                     at(p, q) = e;
                     at(q, q) = b;
@@ -634,11 +643,11 @@ __device__ __forceinline__ void eig_body(const EigTask& t, double nullrel, int m
                 const int i = half > 1 && nrow * half < (1 << 20) ? (int)__umulhi((unsigned)e, hinv) : e / half, k = e - i * half;
                 const int2 sk_ = slots[k];
                 if (!(sk_.x >> 16)) continue;
-                const double c = Cc[k], s = Ss[k];
+                const double s = Ss[k], h = Hh[k];
                 double* v = Vl + i * vld;
                 const double x = v[sk_.x & 0xffff], y = v[sk_.y];
-                v[sk_.x & 0xffff] = fma(c, x, -(s * y));
-                v[sk_.y] = fma(s, x, c * y);
+                v[sk_.x & 0xffff] = rot_first(s, h, x, y);
+                v[sk_.y] = rot_second(s, h, x, y);
             }
             sync();   // updates visible to every CTA before the next pair phase
         }
