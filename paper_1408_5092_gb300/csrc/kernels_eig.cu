@@ -34,6 +34,7 @@
 
 #include "eig_route.h"
 #include "jac_rot.h"
+#include "jac_tol.h"
 #include "jacobi_schedule.h"
 #include "kernels.h"
 
@@ -41,30 +42,6 @@ namespace mpspt {
 namespace {
 
 constexpr int JAC_SMEM = 200704;     // dynamic shared memory of the float64 solver and of the apply kernel
-
-// stop: off(A)^2 <= stop |A|_F^2; a solve that reached off(A)^2 <= stall
-// |A|_F^2 also ends when a sweep shrinks off(A)^2 by less than 19%.
-// Null pairs: a pair (p, q) whose 2x2 block has every entry below
-// null * |A|_F is neither rotated nor counted in the off-diagonal norm.  Its
-// eigenvalues are below 2 null |A|_F, so inside such a cluster the vectors
-// are set by rounding anyway; every coupling of a null index to a larger
-// entry is still rotated away.  For the density matrices of the truncation
-// (positive semidefinite) these are the exactly rank-deficient directions,
-// far below the keep threshold; skipping them saves the sweeps the polish
-// spent circulating rounding noise inside the null cluster.  The float32
-// start sweeps every pair.
-struct Tol {
-    static constexpr double stop = 1e-30, stall = 1e-8, null = 1e-14;
-    // start of the mixed solver: off^2 <= 1e-9 |A|_F^2.  Against 1e-11 it
-    // saves one or two float32 sweeps of eight to ten and costs the polish
-    // none (graded, rank-deficient and degenerate spectra)
-    static constexpr double start = 1e-9;
-    // a polish round ends at off^2 <= 1e-11 of its start (float32 resolves no
-    // more than 1e-7 of the start's off-norm), and is the last one if it
-    // started from off^2 <= 1e-18 |A|_F^2: what float32 rounding leaves is
-    // then below 1e-16 |A|_F
-    static constexpr double gain = 1e-11, last = 1e-18;
-};
 
 // Scale of a matrix with an infinity or a NaN (largest exponent 2047).  Such a
 // matrix has no eigenvalues, and float32 norms of scaled entries cannot show it
@@ -235,16 +212,13 @@ __global__ void __launch_bounds__(NT) k_jac_mixed(const JacTask* __restrict__ ta
         }
         if (tid == 0) {
             if (s == 0) off0 = so;
-            int conv;
-            if (POLISH) conv = so <= Tol::stop * sa || so <= Tol::gain * off0;
-            else conv = so <= Tol::start * sa;
-            conv = conv || sa == 0.0 || (so <= Tol::stall * sa && so > 0.81 * prev) || n < 2;
+            const JacStop q = POLISH ? polish_stop(s, so, sa, off0, prev) : start_stop(so, sa, prev);
             prev = so;
-            stop = conv || s >= maxs;
+            stop = q.stop || n < 2 || s >= maxs;
             if (stop) {
                 *t.nsw = s;
                 *t.total = (POLISH ? *t.total : 0) + s;
-                *t.done = POLISH && conv && (off0 <= Tol::last * sa || sa == 0.0 || n < 2) ? 1 : 0;
+                *t.done = POLISH && (q.done || n < 2) ? 1 : 0;
             }
         }
         __syncthreads();
