@@ -371,8 +371,9 @@ mpspt_status mpspt_train_preconditioner(mpspt_ctx* ctx, mpspt_h0 h0, int M, int 
  * the column order of V, unsorted).  Work is ordered on `stream`
  * (cudaStream_t, 0 = default); the call allocates its task list (and a work
  * copy of matrices too large for the on-chip solver, n above about 590) with
- * cudaMallocAsync on that stream and returns without synchronising.  A
- * matrix with an infinity or a NaN gives NaN in all of its w and V. */
+ * cudaMallocAsync on that stream and returns without synchronising.  V and w
+ * may overlap A (V = A solves in place); A is then copied first.  A matrix with
+ * an infinity or a NaN gives NaN in all of its w and V. */
 mpspt_status mpspt_eigh_batched(int device, void* stream, int batch, const int* n, const double* A,
                                 double* V, double* w);
 

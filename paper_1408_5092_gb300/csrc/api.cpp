@@ -430,18 +430,25 @@ mpspt_status mpspt_eigh_batched(int device, void* stream, int batch, const int* 
     return guard(nullptr, [&] {
         MPSPT_CUDA(cudaSetDevice(device));
         cudaStream_t st = static_cast<cudaStream_t>(stream);
-        for (int i = 0; i < batch; ++i) mpspt::require(n[i] >= 1 && n[i] <= 2048, "matrix size must be in [1, 2048]");
-        // a work copy only for matrices that the solver cannot hold on chip
+        size_t tot = 0, totw = 0;
+        for (int i = 0; i < batch; ++i) {
+            mpspt::require(n[i] >= 1 && n[i] <= 2048, "matrix size must be in [1, 2048]");
+            tot += (size_t)n[i] * n[i];
+            totw += (size_t)n[i];
+        }
+        // a work copy only of matrices that the solver cannot hold on chip, or
+        // where V or w overlaps A
+        const bool overlap = mpspt::eig_overlap(A, V, w, tot, totw);
         size_t wtot = 0;
         for (int i = 0; i < batch; ++i)
-            if (mpspt::eig_in_place(n[i])) wtot += (size_t)n[i] * n[i];
+            if (overlap || mpspt::eig_in_place(n[i])) wtot += (size_t)n[i] * n[i];
         mpspt::DBuf work(wtot * sizeof(double), st), dt;
         std::vector<mpspt::EigTask> tasks(batch);
         size_t o = 0, ow = 0, wo = 0;
         for (int i = 0; i < batch; ++i) {
             const size_t nn = (size_t)n[i] * n[i];
             double* a = const_cast<double*>(A) + o;
-            if (mpspt::eig_in_place(n[i])) {
+            if (overlap || mpspt::eig_in_place(n[i])) {
                 MPSPT_CUDA(cudaMemcpyAsync(work.as<double>() + wo, a, nn * sizeof(double), cudaMemcpyDeviceToDevice, st));
                 a = work.as<double>() + wo;
                 wo += nn;

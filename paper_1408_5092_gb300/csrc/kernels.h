@@ -211,6 +211,11 @@ void order_eig_tasks(EigTask* tasks, int ntask);
 void launch_eig(const EigTask* tasks, const EigTask* host, int ntask, bool null_rule, int maxs, int* flags,
                 cudaStream_t st);
 bool eig_in_place(int n);
+// The solver reads A while it writes V and w: a call whose outputs overlap its
+// input (V = A) needs a work copy of it.  tot: sum of n^2, totw: sum of n.
+inline bool eig_overlap(const double* A, const double* V, const double* w, size_t tot, size_t totw) {
+    return (V < A + tot && A < V + tot) || (w < A + tot && A < w + totw);
+}
 constexpr int kEighSweeps = 40;   // sweep cap of the calls that report no flags
 size_t jac_e_bytes(int n);                 // global float32 triangles of the mixed sweeps (0: shared memory)
 size_t jac_rot_entries(int n);             // list entries of one sweep

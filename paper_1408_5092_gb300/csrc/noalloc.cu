@@ -67,10 +67,11 @@ struct DeviceGuard {
 extern "C" mpspt_status mpspt_eigh_batched_noalloc(int device, void* stream, int batch, const int* n,
                                                    const double* A, double* V, double* w) {
     if (batch < 1 || batch > kMaxBatch || !n || !A || !V || !w) return MPSPT_ERR_INVALID;
-    size_t tot = 0;
+    size_t tot = 0, totw = 0;
     for (int i = 0; i < batch; ++i) {
         if (n[i] < 1 || n[i] > 2048) return MPSPT_ERR_INVALID;
         tot += (size_t)n[i] * n[i];
+        totw += (size_t)n[i];
     }
     if (tot > kScratchDoubles - kTaskDoubles) return MPSPT_ERR_INVALID;   // beyond the fixed scratch
     DeviceGuard dg(device);
@@ -81,11 +82,12 @@ extern "C" mpspt_status mpspt_eigh_batched_noalloc(int device, void* stream, int
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     mpspt::EigTask tasks[kMaxBatch];
     double* work = base + kTaskDoubles;
+    const bool overlap = mpspt::eig_overlap(A, V, w, tot, totw);
     size_t o = 0, ow = 0;
     for (int i = 0; i < batch; ++i) {
         const size_t nn = (size_t)n[i] * n[i];
         double* a = const_cast<double*>(A) + o;
-        if (mpspt::eig_in_place(n[i])) {   // a work copy only where the solver cannot hold the matrix on chip
+        if (overlap || mpspt::eig_in_place(n[i])) {   // a work copy only where needed
             if (cudaMemcpyAsync(work + o, a, nn * sizeof(double), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
                 return MPSPT_ERR_CUDA;
             a = work + o;
