@@ -1,4 +1,5 @@
 #include "eig.h"
+#include "jac_lists.h"
 
 #include <algorithm>
 #include <cstring>
@@ -8,10 +9,7 @@ namespace mpspt {
 
 namespace {
 constexpr int kMaxSweepsF64 = 60;    // float64 Jacobi from the identity
-constexpr int kMaxSweepsF32 = 12;    // float32 start (a cap is not an error: the polish follows)
-constexpr int kPolishSweeps = 8;     // sweeps of one polish round
 constexpr int kMaxRounds = 60;       // polish rounds
-constexpr size_t kListBytes = (size_t)32 << 20;   // rotation lists of one launch, per matrix
 size_t a16(size_t b) { return (b + 15) & ~(size_t)15; }
 
 // Host image of several device arrays, sent with one copy.
@@ -94,11 +92,8 @@ void EigSolver::run(const std::vector<EigTask>& et_in, bool fp64_only, cudaStrea
         eoff[i] = elems;
         elems += (size_t)n * n;
     }
-    // sweeps per launch: what the lists of the largest matrix allow (twelve up to n = 590)
-    sweeps = (int)std::max<size_t>(1, std::min<size_t>(kMaxSweepsF32, kListBytes / (jac_rot_entries(nmax) * sizeof(double2))));
-    const int psweeps = std::min(sweeps, kPolishSweeps);
-    auto rot_b = [&](int n) { return a16(jac_rot_entries(n) * sweeps * sizeof(float2)); };
-    auto rot64_b = [&](int n) { return a16(jac_rot_entries(n) * psweeps * sizeof(double2)); };
+    auto rot_b = [](int n) { return a16(jac_rot_entries(n) * jac_sweep_cap(n) * sizeof(float2)); };
+    auto rot64_b = [](int n) { return a16(jac_rot_entries(n) * std::min(jac_sweep_cap(n), kPolishSweeps) * sizeof(double2)); };
     for (int i = 0; i < ntask; ++i) {
         off[i] = tot;
         tot += rot_b(et[i].n) + rot64_b(et[i].n) + a16(jac_e_bytes(et[i].n)) + 16;
@@ -119,7 +114,7 @@ void EigSolver::run(const std::vector<EigTask>& et_in, bool fp64_only, cudaStrea
         unsigned char* S = P + a16(jac_e_bytes(n));
         check_range(R, (size_t)(S + 16 - R), "jacobi scratch");
         JacTask t{et[i].A, et[i].V, nullptr, P, reinterpret_cast<float2*>(R), reinterpret_cast<double2*>(R64),
-                  flags.as<int>() + i, reinterpret_cast<int*>(S), reinterpret_cast<int*>(S + 4), n, 0};
+                  flags.as<int>() + i, reinterpret_cast<int*>(S), reinterpret_cast<int*>(S + 4), n, jac_sweep_cap(n)};
         start.push_back(t);
         t.A = gp + eoff[i];
         t.w = et[i].w;
@@ -191,8 +186,8 @@ void EigSolver::run(const std::vector<EigTask>& et_in, bool fp64_only, cudaStrea
     dunit = reinterpret_cast<const unsigned*>(d + ou);
     dops = reinterpret_cast<const GemmOp*>(d + oo);
     const JacTask* ds = reinterpret_cast<const JacTask*>(d + os);
-    launch_jac_mixed(ds, nsmall, nmax_small, false, sweeps, st);
-    launch_jac_mixed(ds + nsmall, ntask - nsmall, nmax, false, sweeps, st);
+    launch_jac_mixed(ds, nsmall, nmax_small, false, st);
+    launch_jac_mixed(ds + nsmall, ntask - nsmall, nmax, false, st);
     launch_jac_apply(ds, drows, nrows, nmax, true, true, st);
     count(sweeps32, start, st);
     for (int j = 0; j < 4; ++j) product(j, st);
@@ -204,12 +199,11 @@ void EigSolver::product(int j, cudaStream_t st) {
 }
 
 void EigSolver::rounds(int n, cudaStream_t st) {
-    const int psweeps = std::min(sweeps, kPolishSweeps);
     for (int r = 0; r < n; ++r, ++nround) {
         product(4, st);
         product(5, st);
-        launch_jac_mixed(dtask, nsmall, nmax_small, true, psweeps, st);
-        launch_jac_mixed(dtask + nsmall, ntask - nsmall, nmax, true, psweeps, st);
+        launch_jac_mixed(dtask, nsmall, nmax_small, true, st);
+        launch_jac_mixed(dtask + nsmall, ntask - nsmall, nmax, true, st);
         launch_jac_rot64(dtask, ntask, st);
         launch_jac_apply(dtask, drows, nrows, nmax, false, false, st);
     }

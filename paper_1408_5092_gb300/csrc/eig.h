@@ -47,7 +47,7 @@ struct EigSolver {
     DBuf scratch, vt, g, blob;
     GemmPlan ge;                // shape of the batched square products
     // the enqueued batch: device lists in blob, sizes
-    int ntask = 0, nsmall = 0, nmax_small = 0, nmax = 0, nrows = 0, nunit = 0, nround = 0, sweeps = 0;
+    int ntask = 0, nsmall = 0, nmax_small = 0, nmax = 0, nrows = 0, nunit = 0, nround = 0;
     const JacTask* dtask = nullptr;     // polish tasks (input B); small matrices first
     const JacRows* drows = nullptr;
     const GemmBlk* dblk = nullptr;      // ntask blocks per product

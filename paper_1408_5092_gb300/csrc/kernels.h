@@ -119,7 +119,8 @@ struct JacTask {
     int* done;         // 1: converged
     int* nsw;          // sweeps in the lists of the last launch
     int* total;        // sweeps performed so far
-    int n, pad;
+    int n;
+    int cap;           // sweeps the lists have room for
 };
 struct JacRows {       // rows [r0, r0 + rows) of task's V for one apply block
     int task, r0, rows, pad;
@@ -217,11 +218,9 @@ inline bool eig_overlap(const double* A, const double* V, const double* w, size_
     return (V < A + tot && A < V + tot) || (w < A + tot && A < w + totw);
 }
 constexpr int kEighSweeps = 40;   // sweep cap of the calls that report no flags
-size_t jac_e_bytes(int n);                 // global float32 triangles of the mixed sweeps (0: shared memory)
-size_t jac_rot_entries(int n);             // list entries of one sweep
 // Mixed sweeps (float32 off-diagonal, float64 diagonal) of every matrix, up
-// to maxs in the launch; polish: see k_jac_mixed.  nmax: the largest n.
-void launch_jac_mixed(const JacTask* tasks, int ntask, int nmax, bool polish, int maxs, cudaStream_t st);
+// to its cap in the launch; polish: see k_jac_mixed.  nmax: the largest n.
+void launch_jac_mixed(const JacTask* tasks, int ntask, int nmax, bool polish, cudaStream_t st);
 // rot64 <- the float64 rotations of the tangents in rot
 void launch_jac_rot64(const JacTask* tasks, int ntask, cudaStream_t st);
 // V <- V R over the lists (ident: V starts as the identity)

@@ -33,6 +33,7 @@
 #include <type_traits>
 
 #include "eig_route.h"
+#include "jac_lists.h"
 #include "jac_rot.h"
 #include "jac_tol.h"
 #include "jacobi_schedule.h"
@@ -69,7 +70,7 @@ inline size_t mixed_smem(int n, int cap) {
 // 1000, a float64 operation being 64.  In the polish the float64 diagonal is
 // updated beside the blocks, by the last warps.
 template <int NT, int NB, bool POLISH>
-__global__ void __launch_bounds__(NT) k_jac_mixed(const JacTask* __restrict__ tasks, int maxs) {
+__global__ void __launch_bounds__(NT) k_jac_mixed(const JacTask* __restrict__ tasks) {
     extern __shared__ __align__(16) unsigned char sm[];
     constexpr int NW = NT / 32, NC = NB > 0 ? NB : 1;
     __shared__ double red[2][NW];
@@ -219,7 +220,7 @@ __global__ void __launch_bounds__(NT) k_jac_mixed(const JacTask* __restrict__ ta
             if (s == 0) off0 = so;
             const JacStop q = POLISH ? polish_stop(s, so, sa, off0, prev) : start_stop(so, sa, prev);
             prev = so;
-            stop = q.stop || n < 2 || s >= maxs;
+            stop = q.stop || n < 2 || s >= (POLISH ? min(t.cap, kPolishSweeps) : t.cap);
             if (stop) {
                 *t.nsw = s;
                 *t.total = (POLISH ? *t.total : 0) + s;
@@ -654,24 +655,15 @@ __global__ void __cluster_dims__(JC, 1, 1) __launch_bounds__(256)
 
 }  // namespace
 
-size_t jac_e_bytes(int n) {
-    const size_t m = n + (n & 1);
-    return n <= 236 ? 0 : 4 * m * (m - 1);
-}
-size_t jac_rot_entries(int n) {
-    const size_t m = n + (n & 1);
-    return (m - 1) * (m / 2);
-}
-
 template <int NT, int NB>
-static void launch_mixed(const JacTask* tasks, int ntask, size_t smem, bool polish, int maxs, cudaStream_t st) {
+static void launch_mixed(const JacTask* tasks, int ntask, size_t smem, bool polish, cudaStream_t st) {
     count_launch();
     if (polish) {
         ensure_smem_attr(reinterpret_cast<const void*>(k_jac_mixed<NT, NB, true>), MIX_SMEM);
-        k_jac_mixed<NT, NB, true><<<ntask, NT, smem, st>>>(tasks, maxs);
+        k_jac_mixed<NT, NB, true><<<ntask, NT, smem, st>>>(tasks);
     } else {
         ensure_smem_attr(reinterpret_cast<const void*>(k_jac_mixed<NT, NB, false>), MIX_SMEM);
-        k_jac_mixed<NT, NB, false><<<ntask, NT, smem, st>>>(tasks, maxs);
+        k_jac_mixed<NT, NB, false><<<ntask, NT, smem, st>>>(tasks);
     }
 }
 
@@ -679,13 +671,13 @@ static void launch_mixed(const JacTask* tasks, int ntask, size_t smem, bool poli
 // blocks): enough that a round's update is a few blocks per thread, few
 // enough that its barriers stay cheap (21 clocks at 128 threads, 45 at 512).
 // n up to 46: at most 253 blocks; 92: 1035; 180: 4005; 236 (shared memory): 6903.
-void launch_jac_mixed(const JacTask* tasks, int ntask, int nmax, bool polish, int maxs, cudaStream_t st) {
+void launch_jac_mixed(const JacTask* tasks, int ntask, int nmax, bool polish, cudaStream_t st) {
     if (ntask <= 0) return;
-    if (nmax <= 46) launch_mixed<128, 2>(tasks, ntask, mixed_smem(nmax, mixed_cap(2)), polish, maxs, st);
-    else if (nmax <= 92) launch_mixed<256, 5>(tasks, ntask, mixed_smem(nmax, mixed_cap(5)), polish, maxs, st);
-    else if (nmax <= 180) launch_mixed<512, 8>(tasks, ntask, mixed_smem(nmax, mixed_cap(8)), polish, maxs, st);
-    else if (nmax <= 236) launch_mixed<512, 14>(tasks, ntask, mixed_smem(nmax, mixed_cap(14)), polish, maxs, st);
-    else launch_mixed<1024, 0>(tasks, ntask, mixed_smem(nmax, 0), polish, maxs, st);
+    if (nmax <= 46) launch_mixed<128, 2>(tasks, ntask, mixed_smem(nmax, mixed_cap(2)), polish, st);
+    else if (nmax <= 92) launch_mixed<256, 5>(tasks, ntask, mixed_smem(nmax, mixed_cap(5)), polish, st);
+    else if (nmax <= 180) launch_mixed<512, 8>(tasks, ntask, mixed_smem(nmax, mixed_cap(8)), polish, st);
+    else if (nmax <= 236) launch_mixed<512, 14>(tasks, ntask, mixed_smem(nmax, mixed_cap(14)), polish, st);
+    else launch_mixed<1024, 0>(tasks, ntask, mixed_smem(nmax, 0), polish, st);
 }
 
 void launch_jac_rot64(const JacTask* tasks, int ntask, cudaStream_t st) {
