@@ -118,6 +118,7 @@ void EigSolver::run(const std::vector<EigTask>& et_in, bool fp64_only, cudaStrea
         start.push_back(t);
         t.A = gp + eoff[i];
         t.w = et[i].w;
+        t.total += 1;
         polish.push_back(t);
         for (int r0 = 0; r0 < n; r0 += JAC_APPLY_ROWS) rows.push_back({i, r0, std::min(JAC_APPLY_ROWS, n - r0), 0});
     }

@@ -118,7 +118,7 @@ struct JacTask {
     double2* rot64;    // float64 (tangent of the half angle, s)
     int* done;         // 1: converged
     int* nsw;          // sweeps in the lists of the last launch
-    int* total;        // sweeps performed so far
+    int* total;        // sweeps of the phase so far: [0] of the start, whose [1] is [0] of the polish
     int n;
     int cap;           // sweeps the lists have room for
 };

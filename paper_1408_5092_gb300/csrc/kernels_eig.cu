@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(NT) k_jac_mixed(const JacTask* __restrict__ ta
     if (sh == kNonFinite) {   // no rotation in the start, so that B is not finite either and the polish says so
         if (tid == 0) {
             *t.nsw = 0;
-            *t.total = 0;
+            if (!POLISH) t.total[0] = t.total[1] = 0;
             *t.done = POLISH ? 2 : 0;
         }
         if (t.w)
@@ -223,7 +223,8 @@ __global__ void __launch_bounds__(NT) k_jac_mixed(const JacTask* __restrict__ ta
             stop = q.stop || n < 2 || s >= (POLISH ? min(t.cap, kPolishSweeps) : t.cap);
             if (stop) {
                 *t.nsw = s;
-                *t.total = (POLISH ? *t.total : 0) + s;
+                if (POLISH) *t.total += s;
+                else t.total[0] = s, t.total[1] = 0;
                 *t.done = POLISH && (q.done || n < 2) ? 1 : 0;
             }
         }
