@@ -210,9 +210,9 @@ class DBuf {
     void alloc(size_t bytes, cudaStream_t st) {
         release();
         st_ = st;
-        n_ = bytes;
-        if (bytes) {
+        if (bytes) {   // (n_ stays 0 if the allocation fails)
             MPSPT_CUDA(cudaMallocAsync(&p_, bytes, st));
+            n_ = bytes;
             Registry::get().add(p_, bytes);
         }
     }

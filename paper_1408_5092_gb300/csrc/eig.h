@@ -32,6 +32,7 @@ struct EigSolver {
     //     rotations in float64.  Float32 resolves an off-diagonal part to 1e-7
     //     of itself, so a round that starts below 1e-9 |A| ends at float64
     //     rounding and is the last.  Two rounds are enqueued.
+    // Scratch: up to kEigScratch bytes, less where the device has less to give.
     void run(const std::vector<EigTask>& et, bool fp64_only, cudaStream_t st);
     // With the flags of the last run on the host: false if all are set, else
     // enqueues two more rounds for the matrices that need them (w and flags
@@ -40,20 +41,24 @@ struct EigSolver {
     bool again(const int* flags_host, cudaStream_t st);
 
   private:
+    // matrices that are solved side by side (jac_lists.h): sizes, and the device
+    // lists in blob
+    struct Group {
+        int first = 0, ntask = 0, nsmall = 0, nmax_small = 0, nmax = 0, nrows = 0, nunit = 0, tile = 16;
+        const JacTask *start = nullptr, *polish = nullptr;   // (polish: input B); small matrices first
+        const JacRows* rows = nullptr;
+        const GemmBlk* blk = nullptr;                        // ntask blocks per product
+        const unsigned* unit = nullptr;
+        const GemmOp* ops = nullptr;
+    };
     void fp64(const std::vector<EigTask>& et, cudaStream_t st);
-    void rounds(int n, cudaStream_t st);
-    void product(int j, cudaStream_t st);
-    void count(long long (&acc)[3], const std::vector<JacTask>& jt, cudaStream_t st);
-    DBuf scratch, vt, g, blob;
+    void rounds(const Group& g, int n, cudaStream_t st);
+    void product(const Group& g, int j, cudaStream_t st);
+    void count(long long (&acc)[3], int which, cudaStream_t st);
+    DBuf scratch, blob;
     GemmPlan ge;                // shape of the batched square products
-    // the enqueued batch: device lists in blob, sizes
-    int ntask = 0, nsmall = 0, nmax_small = 0, nmax = 0, nrows = 0, nunit = 0, nround = 0;
-    const JacTask* dtask = nullptr;     // polish tasks (input B); small matrices first
-    const JacRows* drows = nullptr;
-    const GemmBlk* dblk = nullptr;      // ntask blocks per product
-    const unsigned* dunit = nullptr;
-    const GemmOp* dops = nullptr;
-    std::vector<JacTask> polish;
+    std::vector<Group> groups;
+    int nround = 0;
 };
 
 }  // namespace mpspt
