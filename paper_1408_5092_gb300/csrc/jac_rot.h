@@ -101,12 +101,14 @@ __device__ __forceinline__ double jac_sine64(double h) {
 __device__ __forceinline__ double rot_first(double s, double h, double x, double y) { return fma(-s, fma(h, x, y), x); }
 __device__ __forceinline__ double rot_second(double s, double h, double x, double y) { return fma(s, fma(-h, y, x), y); }
 // A symmetric 2 x 2 block [[a, e], [e, b]] under that rotation:
-//   a' = a - u,  b' = b + u,  u = s (2 c e - s (b - a)),
-//   e' = (c^2 - s^2) e - c s (b - a), what a rounded angle leaves of e.
+//   a' = a - u,  b' = b + u,  u = 2 s c e - s^2 (b - a),
+//   e' = (1 - 2 s^2) e - s c (b - a), what a rounded angle leaves of e.
+// (|e| >= 2^-1000, so that twice of it is one exponent up.)
 __device__ __forceinline__ void jac_block64(double s, double h, double& a, double& e, double& b) {
-    const double c = fma(-s, h, 1.0), d = b - a;
-    const double u = s * fma(2.0 * c, e, -(s * d));
-    e = fma(fma(-2.0 * s, s, 1.0), e, -((s * c) * d));
+    const double e2 = __hiloint2double(__double2hiint(e) + (1 << 20), __double2loint(e));
+    const double q = s * fma(-s, h, 1.0), p = s * s, d = b - a;
+    const double u = fma(q, e2, -(p * d));
+    e = fma(-q, d, fma(-p, e2, e));
     a -= u;
     b += u;
 }

@@ -123,18 +123,20 @@ __global__ void __launch_bounds__(NT) k_jac_mixed(const JacTask* __restrict__ ta
     __syncthreads();
     for (int i = warp; i < n; i += NW)
         for (int j = i + lane; j < n; j += 32) {
-            double a = t.A[(size_t)i * n + j];
+            const double a = t.A[(size_t)i * n + j];
             if (j == i) {
                 if constexpr (POLISH) D[i] = ldexp(a, -sh);
                 else D[i] = d2f_scaled(a, sh);
-                continue;
             }
-            // B's two halves are rounded independently: their mean is nearer
-            // (vectors' errors 0.73 of one half's at n = 8, 0.75 at 128; the loads
-            // and additions are 0.1% of a round at n = 173)
-            if constexpr (POLISH) a = 0.5 * (a + t.A[(size_t)j * n + i]);
-            E[tri(m, i, j)] = d2f_scaled(a, sh);
+            else E[tri(m, i, j)] = d2f_scaled(a, POLISH ? sh + 1 : sh);
         }
+    // B's two halves are rounded independently: their mean is nearer (vectors'
+    // errors 0.73 of one half's at n = 8, 0.75 at 128)
+    if constexpr (POLISH) {
+        __syncthreads();
+        for (int i = warp; i < n; i += NW)
+            for (int j = lane; j < i; j += 32) E[tri(m, j, i)] += d2f_scaled(t.A[(size_t)i * n + j], sh + 1);
+    }
     // places of this thread's pair and blocks in a buffer (16 bits each)
     int kl[NC];
     unsigned rd[2][NC], wr[2][NC];
