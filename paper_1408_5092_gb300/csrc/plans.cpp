@@ -307,8 +307,12 @@ std::pair<int, int> Autotuner::choose(const GemmPlan& g, cudaStream_t st) {
                   bucket((long long)g.blocks.size())};
     std::lock_guard<std::mutex> lk(mu);
     auto it = best.find(key);
-    // (a float64 entry of another tile, from an older file, is timed again)
-    if (it != best.end() && (g.kind != GEMM_F64 || it->second.first <= 32)) { ++reused; return it->second; }
+    // (a float64 entry of another tile than its two, from an older file, is timed again)
+    const std::pair<int, int> wide{32, 32}, narrow{16, 128};
+    if (it != best.end() && (g.kind != GEMM_F64 || it->second == wide || it->second == narrow)) {
+        ++reused;
+        return it->second;
+    }
     static const int cand_wide[][2] = {{64, 64}, {32, 64}, {64, 32}, {32, 32}};
     static const int cand_skinny[][2] = {{16, 128}, {32, 64}, {32, 32}};
     static const int cand_f64[][2] = {{32, 32}, {16, 128}};
