@@ -188,7 +188,18 @@ int bucket(long long x) {
 
 void GemmPlan::upload(cudaStream_t st) {
     mpspt::upload(dops, ops, st);
-    if (tuner && !is_tc(kind) && !blocks.empty()) {
+    steps = 0.0;
+    if (kind == GEMM_F64)
+        for (const Blk& b : blocks) {
+            long long q = 0;
+            for (int o = b.op0; o < b.op1; ++o) q += (ops[o].k + 3) / 4;
+            steps += (double)((b.m + 7) / 8) * ((b.n + 7) / 8) * q;
+        }
+    // (float64 plans of few steps take the narrow units: the two differ by the
+    // launch alone there, and their timing would stand for larger plans)
+    const bool few = kind == GEMM_F64 && steps <= kClusterSteps;
+    const bool tune = tuner && !is_tc(kind) && !blocks.empty() && !few;
+    if (tune) {
         const std::pair<int, int> t = tuner->choose(*this, st);
         tm = t.first;
         tn = t.second;
@@ -199,15 +210,7 @@ void GemmPlan::upload(cudaStream_t st) {
     if (kind == GEMM_F64) {
         size_t tk = 0;
         std::vector<long long> cm;
-        steps = 0.0;
-        for (const Blk& b : blocks) {
-            long long q = 0;
-            for (int o = b.op0; o < b.op1; ++o) q += (ops[o].k + 3) / 4;
-            steps += (double)((b.m + 7) / 8) * ((b.n + 7) / 8) * q;
-        }
-        // (plans of few steps take the narrow units whatever the tuner found:
-        // the two differ by the launch alone there)
-        tile64 = steps <= kClusterSteps ? 16 : tuner && !blocks.empty() ? (tm == 32 ? 32 : 16) : tile_rule();
+        tile64 = few ? 16 : tune ? (tm == 32 ? 32 : 16) : tile_rule();
         units(tile64, gblk, unit_blk, &cm, &pe, &tk);
         for (size_t i = 0; i < gblk.size(); ++i) gblk[i].cmap = cm[i] >= 0 ? cbase + cm[i] : nullptr;
         workspace(pe, tk, st);

@@ -33,3 +33,11 @@ def test_entries_of_other_tiles_are_timed_again(tmp_path):
         assert {r[:6] for r in new} >= {r[:6] for r in rows}
         assert all(r[6:] in ((32, 32), (16, 128)) for r in new if r[0] == F64), old
         assert again == e2      # both unit shapes give the same bits
+
+
+def test_small_float64_plans_are_not_timed(tmp_path):
+    """Every float64 plan of the tiny system at M = 3 is below the step count under
+    which the units are narrow whatever the tuner says."""
+    cache = tmp_path / "tiles.txt"
+    _, rows = _run("tiny", 3, cache)
+    assert not [r for r in rows if r[0] == F64]
