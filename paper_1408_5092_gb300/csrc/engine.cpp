@@ -1128,6 +1128,8 @@ struct Sweeper {
         } catch (...) {
             cudaStreamEndCapture(ln.st, &g);
             if (g) cudaGraphDestroy(g);
+            cudaGetLastError();
+            uncount_launches(launch_count_thread() - l0);
             throw;
         }
         MPSPT_CUDA(cudaStreamEndCapture(ln.st, &g));
@@ -1195,9 +1197,12 @@ struct Sweeper {
         // (partition lanes hide the launches behind one another, and 16 whole
         // SMs of one cluster are rarely free beside them: 12 partitions on 8
         // lanes took 164 -> 168 ms with clusters)
-        if (&ln == c.lane0.get() && sig.for_cluster() && cg_cluster_available()) {
+        bool cluster = &ln == c.lane0.get() && sig.for_cluster() && cg_cluster_available();
+        if (cluster) {
             // start, all iterations and the state in one go; with graphs as
-            // one graph launch (whose iterations come in chunks)
+            // one graph launch (whose iterations come in chunks).  Where the
+            // launch is refused, launches per iteration as for larger operators.
+            struct Refused {};
             const bool graph = c.opt.cuda_graphs && ln.st != nullptr;
             const int maxit = graph ? (c.opt.cg_max_iter + kChunk - 1) / kChunk * kChunk : c.opt.cg_max_iter;
             const CgArgs args{sig.g1.lists(), sig.g2.lists(), sig.dmt.as<MixTask>(), sig.dms.as<MixSrc>(),
@@ -1208,22 +1213,30 @@ struct Sweeper {
                 sig.run(ln.st);
                 cg_init(w.r.as<double>(), w.z.as<double>(), w.p.as<double>(), w.b.as<double>(), w.Ap.as<double>(),
                         w.minv.as<double>(), n, S, c.opt.cg_tol, ln.red.as<double>(), ln.cnt.as<unsigned>(), ln.st);
-                if (!launch_cg_cluster(args, ln.st)) throw Error(MPSPT_ERR_CUDA, "cluster solve: launch failed");
+                if (!c.cg_cluster(args, ln.st)) throw Refused{};
             };
             ev_begin();
-            if (graph) {
-                capture(gexec, body);
-                MPSPT_CUDA(cudaGraphLaunch(gexec, ln.st));
-                count_launch();
-            } else {
-                body();
+            try {
+                if (graph) {
+                    capture(gexec, body);
+                    MPSPT_CUDA(cudaGraphLaunch(gexec, ln.st));
+                    count_launch();
+                } else {
+                    body();
+                }
+            } catch (const Refused&) {
+                cluster = false;
             }
-            ev_end(true);
-            sync_state();
-            launched = ln.cg_host->iters;
-            res->sigma64_calls += 1 + launched;
-            res->sigma64_flops += (1 + launched) * sig.flops();
-        } else {
+            if (cluster) {
+                ev_end(true);
+                sync_state();
+                launched = ln.cg_host->iters;
+                res->sigma64_calls += 1 + launched;
+                res->sigma64_flops += (1 + launched) * sig.flops();
+                res->cluster_solves++;
+            }
+        }
+        if (!cluster) {
             MPSPT_CUDA(cudaMemcpyAsync(w.p.get(), x, n * sizeof(double), cudaMemcpyDeviceToDevice, ln.st));
             sigma64();
             cg_init(w.r.as<double>(), w.z.as<double>(), w.p.as<double>(), w.b.as<double>(), w.Ap.as<double>(),

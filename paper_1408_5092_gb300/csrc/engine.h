@@ -77,6 +77,9 @@ struct Ctx {
     bool harvesting = false;
     size_t harvest_max = 0;
     std::vector<float> harvest_x, harvest_t;
+    // launches a small local solve on a cluster; false: not launched, and the
+    // solve takes launches per iteration
+    bool (*cg_cluster)(const CgArgs&, cudaStream_t) = &launch_cg_cluster;
 
     explicit Ctx(const mpspt_options& o);
     ~Ctx();
@@ -109,6 +112,7 @@ struct SweepResult {
     long long launches = 0;
     long long learned_used = 0, learned_rejected = 0;
     long long sigma64_calls = 0;
+    long long cluster_solves = 0;        // local solves in one launch (launch_cg_cluster)
     double sigma64_flops = 0.0, sigma64_ms = 0.0;
     bool converged = false;              // last sweep met e_tol
     std::vector<long long> sigma_cum;    // sigma applications (all precisions) at each sweep end

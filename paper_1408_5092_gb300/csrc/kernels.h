@@ -189,7 +189,8 @@ struct CgArgs {
     size_t n;
     CgState* S;
 };
-// The whole solve in one launch on one cluster; false: not available here.
+// The whole solve in one launch on one cluster; false: not available here, or
+// the launch was refused (nothing runs).
 bool launch_cg_cluster(const CgArgs& a, cudaStream_t st);
 bool cg_cluster_available();
 // Float32 arithmetic on float64 data: grouped GEMM with output tile tm x tn

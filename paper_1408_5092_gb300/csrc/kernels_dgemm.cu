@@ -368,8 +368,12 @@ bool launch_cg_cluster(const CgArgs& a, cudaStream_t st) {
     cf.stream = st;
     cf.attrs = &at;
     cf.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cf, k_cg_cluster, a) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
     count_launch();
-    return cudaLaunchKernelEx(&cf, k_cg_cluster, a) == cudaSuccess;
+    return true;
 }
 bool cg_cluster_available() { return cg_cluster_size() > 0; }
 
