@@ -116,8 +116,12 @@ typedef struct {
     double max_discarded_weight; /* over the last sweep                          */
     long long cg_iters;          /* total CG iterations (all local solves)       */
     long long sigma_calls;       /* applications of A_loc (any precision)        */
-    double sigma_flops;          /* algorithmic flops of those applications      */
-    double sigma_ms;             /* device time inside them (CUDA events)        */
+    double sigma_flops;          /* algorithmic flops of those applications that */
+    double sigma_ms;             /*   were launched by themselves, and their     */
+                                 /*   device time (CUDA events); small float64   */
+                                 /*   local solves that run in one launch, CG    */
+                                 /*   vector work included, are in sigma_calls   */
+                                 /*   alone                                      */
     double wall_ms;              /* wall time of the minimisation                */
     int max_bond_dim;
     double sweep_ms[64];         /* device time at the end of each sweep         */

@@ -1215,7 +1215,6 @@ struct Sweeper {
                         w.minv.as<double>(), n, S, c.opt.cg_tol, ln.red.as<double>(), ln.cnt.as<unsigned>(), ln.st);
                 if (!c.cg_cluster(args, ln.st)) throw Refused{};
             };
-            ev_begin();
             try {
                 if (graph) {
                     capture(gexec, body);
@@ -1228,11 +1227,11 @@ struct Sweeper {
                 cluster = false;
             }
             if (cluster) {
-                ev_end(true);
+                // (counted as calls alone: neither its time nor its flops are
+                // those of the operator by itself)
                 sync_state();
                 launched = ln.cg_host->iters;
                 res->sigma64_calls += 1 + launched;
-                res->sigma64_flops += (1 + launched) * sig.flops();
                 res->cluster_solves++;
             }
         }

@@ -53,3 +53,15 @@ def test_refused_launches_take_the_other_route(runs, M, graphs):
     assert on["clusters"] == solves if M == 3 else 0 < on["clusters"] < solves
     assert off["clusters"] == 0 and off["launches"] > on["launches"]
     assert np.abs(on["e2"] - off["e2"]).max() < 1e-8
+
+
+@pytest.mark.parametrize("M", [3, 40])
+@pytest.mark.parametrize("graphs", [0, 1])
+def test_flops_of_one_launch_solves_are_not_counted(runs, M, graphs):
+    """At M = 3 only the application that evaluates each solve is launched by
+    itself; what refused runs launch by themselves is at least twice that."""
+    res, _ = runs
+    on, off = res[M, graphs, 0], res[M, graphs, 1]
+    assert on["calls"] >= on["iters"] and 0 < on["flops"] < off["flops"]
+    if M == 3:
+        assert off["flops"] > 2 * on["flops"]
