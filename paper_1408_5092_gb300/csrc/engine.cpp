@@ -1532,7 +1532,7 @@ struct Sweeper {
         double* x = w.x.as<double>();
         product(prod, psi, i, X, x);
         const Omega& oA = omega(omA_c, WA, i);
-        sig.build(oA, X, X, bL, bL, bR, bR, LA[i], RA[i + 2], WA.dq[i + 2], w.p.as<double>(),
+        sig.build(oA, X, X, bL, bL, bR, bR, LA[i], RA[i + 2], w.p.as<double>(),
                   w.Ap.as<double>(), ln.st);
         dia.build(oA, X, bL, bR, LA[i], RA[i + 2], WA.dq[i], WA.dq[i + 2], w.dg.as<double>(), ln.st);
         dia.run(ln.st);
@@ -1572,7 +1572,7 @@ struct Sweeper {
         h_prod += since(th); th = clk::now();
         const Omega& oA = omega(omA_c, WA, i);
         const Omega& oV = omega(omV_c, WV, i);
-        rhs.build(oV, X, X0, bL, psi0.bond[i], bR, psi0.bond[i + 2], LV[i], RV[i + 2], WV.dq[i + 2],
+        rhs.build(oV, X, X0, bL, psi0.bond[i], bR, psi0.bond[i + 2], LV[i], RV[i + 2],
                   w.x0.as<double>(), w.g.as<double>(), ln.st);
         h_rhs += since(th);
         if (c.opt.verbose >= 3) MPSPT_CUDA(cudaEventRecord(pev[0], ln.st));
@@ -1581,7 +1581,7 @@ struct Sweeper {
         if (c.opt.verbose >= 2) { MPSPT_CUDA(cudaStreamSynchronize(ln.st)); t_rhs += since(t0); t0 = clk::now(); }
         if (c.opt.verbose >= 3) { float a; cudaEventElapsedTime(&a, pev[0], pev[1]); t_rhs_dev += a; }
         th = clk::now();
-        sig.build(oA, X, X, bL, bL, bR, bR, LA[i], RA[i + 2], WA.dq[i + 2], w.p.as<double>(),
+        sig.build(oA, X, X, bL, bL, bR, bR, LA[i], RA[i + 2], w.p.as<double>(),
                   w.Ap.as<double>(), ln.st);
         dia.build(oA, X, bL, bR, LA[i], RA[i + 2], WA.dq[i], WA.dq[i + 2], w.dg.as<double>(), ln.st);
         dia.run(ln.st);
@@ -1598,7 +1598,7 @@ struct Sweeper {
         if (harvest_here)
             MPSPT_CUDA(cudaMemcpyAsync(w.xw.get(), x, n * sizeof(double), cudaMemcpyDeviceToDevice, ln.st));
         if (lo_kind != GEMM_F64)
-            sig_lo.build(oA, X, X, bL, bL, bR, bR, LA[i], RA[i + 2], WA.dq[i + 2], w.p.as<double>(),
+            sig_lo.build(oA, X, X, bL, bL, bR, bR, LA[i], RA[i + 2], w.p.as<double>(),
                          w.Ap.as<double>(), ln.st);
         h_sig += since(th);
         if (c.opt.verbose >= 2) { MPSPT_CUDA(cudaStreamSynchronize(ln.st)); t_plan += since(t0); t0 = clk::now(); }
@@ -2308,7 +2308,7 @@ void local_apply(Ctx& c, int h0, const MpsD& psi1_in, int i, int op, const doubl
     if (op == MPSPT_LOCAL_SIGMA) {
         sw.omA.build(sw.WA, i);
         TwoSitePlan& pl = (sw.lo_kind == GEMM_F64) ? sw.sig : sw.sig_lo;
-        pl.build(sw.omA, X, X, bL, bL, bR, bR, sw.LA[i], sw.RA[i + 2], sw.WA.dq[i + 2],
+        pl.build(sw.omA, X, X, bL, bL, bR, bR, sw.LA[i], sw.RA[i + 2],
                  sw.w.p.as<double>(), dout, c.st);
         pl.run(c.st);
         sw.check_tc();
@@ -2319,7 +2319,7 @@ void local_apply(Ctx& c, int h0, const MpsD& psi1_in, int i, int op, const doubl
         sw.product(sw.prod0, c.psi0, i, X0, sw.w.x0.as<double>());
         sw.omV.build(sw.WV, i);
         sw.rhs.build(sw.omV, X, X0, bL, c.psi0.bond[i], bR, c.psi0.bond[i + 2], sw.LV[i], sw.RV[i + 2],
-                     sw.WV.dq[i + 2], sw.w.x0.as<double>(), dout, c.st);
+                     sw.w.x0.as<double>(), dout, c.st);
         sw.rhs.run(c.st);
     } else if (op == MPSPT_LOCAL_DIAG) {
         sw.omA.build(sw.WA, i);

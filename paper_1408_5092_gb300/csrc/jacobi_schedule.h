@@ -22,7 +22,8 @@ JAC_HD void rr_pair(int k, int r, int m, int& pa, int& pb) {
 // single index (q = -1) that is not rotated in that round; every index is
 // in exactly one slot per round, so the 2x2 block update over all slot
 // pairs touches every matrix entry once, and every pair meets once per
-// sweep.
+// sweep.  (The kernels work out the same pairs in place; the host check of
+// the ordering goes by this.)
 struct Sched {
     int n, m, half;
     JAC_HD void init(int n_) {

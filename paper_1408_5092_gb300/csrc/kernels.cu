@@ -366,10 +366,6 @@ __global__ void k_scale(double* y, const double* __restrict__ x, double a, size_
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
         y[i] = a * x[i];
 }
-__global__ void k_zero(double* y, size_t n) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        y[i] = 0.0;
-}
 __global__ void k_minv(double* y, const double* __restrict__ d, size_t n) {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
         y[i] = d[i] > 0.0 ? 1.0 / d[i] : 0.0;
@@ -461,14 +457,6 @@ __global__ void __launch_bounds__(RB) k_dav_ritz(double* x, double* ax, double* 
         v[0] = fma(r, r, v[0]);
     }
     if (grid_sum<1>(v, 1, sh, tot, scratch, counter) && threadIdx.x == 0) *out = tot[0];
-}
-__global__ void k_d2f(float* y, const double* __restrict__ x, size_t n) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        y[i] = (float)x[i];
-}
-__global__ void k_f2d(double* y, const float* __restrict__ x, size_t n) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        y[i] = (double)x[i];
 }
 
 inline int ew_grid(size_t n) {
@@ -573,9 +561,6 @@ void launch_diag(const DiagTask* tasks, int ntask, const DiagTerm* terms, cudaSt
 void launch_copy(const CopyTask* tasks, int ntask, cudaStream_t st) {
     if (ntask > 0) { counted(); k_copy<<<ntask, 256, 0, st>>>(tasks); }
 }
-void vec_zero(double* x, size_t n, cudaStream_t st) {
-    if (n) { counted(); k_zero<<<ew_grid(n), 256, 0, st>>>(x, n); }
-}
 void vec_scale_mask(double* y, const double* x, double a, size_t n, cudaStream_t st) {
     if (n) { counted(); k_scale<<<ew_grid(n), 256, 0, st>>>(y, x, a, n); }
 }
@@ -585,12 +570,6 @@ void vec_axpy(double* y, const double* x, double a, size_t n, cudaStream_t st) {
 void vec_dot(const double* x, const double* y, size_t n, double* out, double* scratch,
              unsigned* counter, cudaStream_t st) {
     counted(); k_dot<<<red_grid(n), RB, 0, st>>>(x, y, n, out, scratch, counter);
-}
-void f64_to_f32(float* y, const double* x, size_t n, cudaStream_t st) {
-    if (n) { counted(); k_d2f<<<ew_grid(n), 256, 0, st>>>(y, x, n); }
-}
-void f32_to_f64(double* y, const float* x, size_t n, cudaStream_t st) {
-    if (n) { counted(); k_f2d<<<ew_grid(n), 256, 0, st>>>(y, x, n); }
 }
 namespace {
 inline int dav_grid(size_t n) {   // scratch: DAV_MAX sums of at most 228 blocks

@@ -231,14 +231,11 @@ void launch_jac_apply(const JacTask* tasks, const JacRows* rows, int nblocks, in
 void launch_copy(const CopyTask* tasks, int ntask, cudaStream_t st);
 
 // Vector kernels (n doubles).  Reductions are deterministic (fixed order).
-void vec_zero(double* x, size_t n, cudaStream_t st);
 void vec_scale_mask(double* y, const double* x, double a, size_t n, cudaStream_t st);  // y = a*x
 void vec_axpy(double* y, const double* x, double a, size_t n, cudaStream_t st);       // y += a*x
 // out[slot] = x.y  (partial sums in scratch: 4096 doubles, for all of these)
 void vec_dot(const double* x, const double* y, size_t n, double* out, double* scratch,
              unsigned* counter, cudaStream_t st);
-void f64_to_f32(float* y, const double* x, size_t n, cudaStream_t st);
-void f32_to_f64(double* y, const float* x, size_t n, cudaStream_t st);
 
 // Preconditioned CG building blocks on device scalars.
 // r = b - Ax ; z = Minv r ; p = z ; rz = r.z ; rr = r.r ; bb = b.b

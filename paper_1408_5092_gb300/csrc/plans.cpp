@@ -496,9 +496,7 @@ void mix_pieces(std::vector<MixTask>& tasks, std::vector<unsigned>& piece_task) 
 
 void TwoSitePlan::build(const Omega& om, const TwoT& bra, const TwoT& ket, const Bond& braL,
                         const Bond& ketL, const Bond& braR, const Bond& ketR, const EnvT& L,
-                        const EnvT& R, const std::vector<QN>& dqR, const double* x, double* out,
-                        cudaStream_t st) {
-    (void)dqR; (void)ketL;
+                        const EnvT& R, const double* x, double* out, cudaStream_t st) {
     g1.clear(); g2.clear(); g2s.clear();
     mtasks.clear(); msrc.clear();
     const int np = (int)ket.panels.size();
@@ -771,7 +769,6 @@ void EnvPlan::upload_mix(cudaStream_t st) {
 void EnvPlan::build_left(const MPO& W, int site, const EnvT& L, const SiteT& Abra, const SiteT& Aket,
                          const Bond& braL, const Bond& ketL, const Bond& braR, const Bond& ketR,
                          EnvT& Lnew, cudaStream_t st) {
-    (void)braR;
     g1.clear();
     g2.clear();
     mt.clear();

@@ -184,7 +184,7 @@ struct TwoSitePlan {
     void set_tuner(Autotuner* t) { g1.tuner = t; g2.tuner = t; g2s.tuner = t; }
     void build(const Omega& om, const TwoT& bra, const TwoT& ket, const Bond& braL,
                const Bond& ketL, const Bond& braR, const Bond& ketR, const EnvT& L,
-               const EnvT& R, const std::vector<QN>& dqR, const double* x, double* out,
+               const EnvT& R, const double* x, double* out,
                cudaStream_t st);
     void run(cudaStream_t st) const {
         g1.run(st);
