@@ -23,6 +23,7 @@
 #include <mutex>
 #include <utility>
 
+#include "fconv.h"
 #include "kernels.h"
 
 namespace mpspt {
@@ -117,17 +118,6 @@ __device__ __forceinline__ float d2f_rn(double v) {
     unsigned f = sign | ((unsigned)fe << 23) | mant;
     if (rem > 0x10000000u || (rem == 0x10000000u && (mant & 1u))) f += 1u;   // carry may reach the exponent
     return __uint_as_float(f);
-}
-
-// float32 -> float64 by integer operations (a conversion instruction occupies
-// a sub-partition's float64 unit for 64 clocks: 2 us for a tile of 128 x 64).
-// Subnormal values become signed zero.
-__device__ __forceinline__ double f2d_int(uint32_t b) {
-    const uint32_t mag = b & 0x7FFFFFFFu, sign = b & 0x80000000u;
-    uint32_t hi = (mag >> 3) + (896u << 20);
-    if (mag >= 0x7F800000u) hi = 0x7FF00000u | ((mag & 0x7FFFFFu) >> 3);
-    const bool zero = mag < 0x00800000u;
-    return __hiloint2double((int)(sign | (zero ? 0u : hi)), zero ? 0 : (int)(b << 29));
 }
 
 // hi = round(f), lo = round(f - hi) in the 16-bit type (bf16 or f16)
