@@ -299,30 +299,38 @@ void MPO::index() {
         std::vector<int> fill(in_ptr[p].begin(), in_ptr[p].end() - 1);
         for (int q = 0; q < (int)E.size(); ++q) in_idx[p][fill[E[q].b]++] = q;
     }
-    in_el.assign(nsite, {});
-    out_el.assign(nsite, {});
-    in_at.assign(nsite, {});
-    out_at.assign(nsite, {});
+    std::vector<Lists::Site> in(nsite), out(nsite);
     for (int p = 0; p < nsite; ++p) {
-        const auto& E = W[p];
-        auto fill_rows = [&](int states, const std::vector<int>& ptr, const std::vector<int>* idx, std::vector<El>& el,
-                             std::vector<int>& at) {
-            at.reserve((size_t)states * 4 + 1);
-            for (int x = 0; x < states; ++x)
-                for (int s = 0; s < 4; ++s) {
-                    at.push_back((int)el.size());
-                    for (int q = ptr[x]; q < ptr[x + 1]; ++q) {
-                        const MpoEntry& e = E[idx ? (*idx)[q] : q];
-                        const double* row = &ops[e.op][(size_t)s * 4];
-                        for (int t = 0; t < 4; ++t)
-                            if (row[t] != 0.0) el.push_back({idx ? e.a : e.b, t, e.coef * row[t]});
-                    }
-                }
-            at.push_back((int)el.size());
-        };
-        fill_rows(dim[p + 1], in_ptr[p], &in_idx[p], in_el[p], in_at[p]);
-        fill_rows(dim[p], out_ptr[p], nullptr, out_el[p], out_at[p]);
+        in[p] = {W[p].data(), in_ptr[p].data(), in_idx[p].data(), ops.data(), dim[p + 1]};
+        out[p] = {W[p].data(), out_ptr[p].data(), nullptr, ops.data(), dim[p]};
     }
+    in_el.l = in_at.l = std::make_shared<const Lists>(std::move(in));
+    out_el.l = out_at.l = std::make_shared<const Lists>(std::move(out));
+}
+
+const MPO::Lists::Made& MPO::Lists::get(int p) const {
+    Made& m = made[p];
+    std::call_once(m.once, [&] {
+        const Site& s = src[p];
+        std::vector<El> el;
+        std::vector<int> at;
+        at.reserve((size_t)s.states * 4 + 1);
+        for (int x = 0; x < s.states; ++x)
+            for (int row = 0; row < 4; ++row) {
+                at.push_back((int)el.size());
+                for (int q = s.ptr[x]; q < s.ptr[x + 1]; ++q) {
+                    const MpoEntry& e = s.entry[s.idx ? s.idx[q] : q];
+                    const double* v = &s.ops[e.op][(size_t)row * 4];
+                    for (int t = 0; t < 4; ++t)
+                        if (v[t] != 0.0) el.push_back({s.idx ? e.a : e.b, t, e.coef * v[t]});
+                }
+            }
+        at.push_back((int)el.size());
+        m.el.swap(el);
+        m.at.swap(at);
+        m.done.store(true);
+    });
+    return m;
 }
 
 RunMaps::RunMaps(const MPO& W_) : W(W_) {
