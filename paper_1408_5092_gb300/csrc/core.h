@@ -257,6 +257,7 @@ struct PinnedRing {
     bool used[2] = {false, false};
     cudaEvent_t ev[2] = {nullptr, nullptr};
     cudaStream_t st = 0;
+    std::atomic<bool> taken{false};   // by a RingScope
     PinnedRing(size_t bytes, cudaStream_t s) : st(s) {
         half = bytes / 2;
         MPSPT_CUDA(cudaMallocHost(&base, 2 * half));
@@ -295,10 +296,24 @@ inline PinnedRing*& thread_ring() {
     return r;
 }
 
+// A ring serves one scope at a time: where another thread has it (two E3 calls
+// on one context), this one makes pageable copies.
 struct RingScope {
     PinnedRing* prev;
-    explicit RingScope(PinnedRing* r) : prev(thread_ring()) { thread_ring() = r; }
-    ~RingScope() { thread_ring() = prev; }
+    PinnedRing* held = nullptr;
+    explicit RingScope(PinnedRing* r) : prev(thread_ring()) {
+        if (r && r != prev) {
+            if (r->taken.exchange(true, std::memory_order_acquire)) r = nullptr;
+            else held = r;
+        }
+        thread_ring() = r;
+    }
+    ~RingScope() {
+        thread_ring() = prev;
+        if (held) held->taken.store(false, std::memory_order_release);
+    }
+    RingScope(const RingScope&) = delete;
+    RingScope& operator=(const RingScope&) = delete;
 };
 
 inline void copy_h2d(void* dst, const void* src, size_t bytes, cudaStream_t st) {
