@@ -547,11 +547,17 @@ __device__ __forceinline__ void eig_body(const EigTask& t, double nullrel, int m
                 if (on) {
                     const double a = at(p, p), e = at(p, q), b = at(q, q);
                     const float fd = d2f_trunc(b - a), fe = d2f_trunc(e);
-                    on = fe != 0.f && !jac_negligible(e, a, b) &&
+                    on = !is_zero(e) && !jac_negligible(e, a, b) &&
                          !(abs_below(e, nullv) && abs_below(a, nullv) && abs_below(b, nullv));
-                    if (on) {
+                    double h = 0.0;
+                    if (on && fabsf(fe) >= 0x1p-80f) {
                         const float tn = jac_tan(fd, fe);
-                        const double h = jac_half64(tn, jac_newton(b - a, e, fd, fe, tn));
+                        h = jac_half64(tn, jac_newton(b - a, e, fd, fe, tn));
+                    } else if (on) {
+                        h = jac_half64_tiny(b - a, e);
+                        on = !is_zero(h);
+                    }
+                    if (on) {
                         Hh[k] = h;
                         Ss[k] = jac_sine64(h);
                         Xa[k] = a; Xe[k] = e; Xb[k] = b;
