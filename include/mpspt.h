@@ -391,9 +391,9 @@ mpspt_status mpspt_eigh_batched(int device, void* stream, int batch, const int* 
  * float64 rounding.  A is left unchanged.  Allocates copies of A, V and w
  * and scratch of at most about 1 GiB (17 n^2 doubles a matrix up to n = 590, 4
  * above 1448; a batch that needs more, or more than the device can give, is
- * solved in parts), and returns after the stream has finished the work.  A matrix that does not pass the
- * convergence test (one with an infinity or a NaN among them) gives
- * MPSPT_ERR_NOT_CONVERGED. */
+ * solved in parts), and returns after the stream has finished the work.  A
+ * matrix that does not pass the convergence test (one with an infinity or a
+ * NaN among them) gives MPSPT_ERR_NOT_CONVERGED. */
 mpspt_status mpspt_eigh_batched_ex(int device, void* stream, int batch, const int* n, const double* A,
                                    double* V, double* w, int f32_start);
 

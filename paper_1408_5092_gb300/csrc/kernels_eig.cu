@@ -23,7 +23,9 @@
 // Measured (device time of the truncations of one M = 256 sweep of 8e/8o + 24,
 // sectors up to n = 173): sweeps 240 -> 47 ms, V 159 -> 25 ms against one
 // launch per sweep with float64 polish sweeps and 32 rows of V per CTA; a
-// batch of ten sectors (173 and down by 0.8) 29.7 -> 4.5 ms.
+// batch of ten sectors (173 and down by 0.8) 29.8 -> 6.0 ms a call.  Above n = 236
+// (triangles in global memory): n = 260 102 -> 61 ms, 346 369 -> 148, 500 972 ->
+// 455, sixteen of 300 183 -> 146.
 //
 // k_eig_one / k_eig_cl: the plain float64 solver (float64 sweeps from the
 // identity), all sweeps in one launch, V included.
@@ -400,8 +402,9 @@ __global__ void __launch_bounds__(32 * JAC_APPLY_ROWS) k_jac_apply(const JacTask
 // by the chain rotation - barrier - update - barrier.  A float64 instruction
 // occupies a sub-partition for 64 clocks however few lanes are active, so what
 // counts is their number per warp.  Measured against the one-CTA kernel with
-// divisions and square roots: twelve 13 x 13 350 -> 188 us, seven of 90 and
-// down 25.6 -> 4.1 ms; against the launch-per-sweep cluster form 21 -> 4.2 ms.
+// divisions and square roots: twelve 13 x 13 458 -> 230 us a call, sectors of 90
+// and down 20.6 -> 5.5 ms; against the launch-per-sweep cluster form n = 240 531 ->
+// 53 ms, 346 1664 -> 153, 500 5007 -> 579.
 constexpr int JC = 8;
 
 struct EigFit { size_t head, a, v; };   // shared memory of one CTA: head, triangle share, V rows
