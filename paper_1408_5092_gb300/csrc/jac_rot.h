@@ -98,15 +98,6 @@ __device__ __forceinline__ double jac_sine64(double h) {
     const double e = fma(-(h * h), f2d_exact(rf), f2d_exact(1.f - rf)), r = f2d_exact(2.f * rf);
     return h * fma(r, fma(e, e, e), r);
 }
-// h of a pair whose e is below 2^-80 of the largest entry: the Newton steps'
-// float32 residuals leave their range there, so by division and square roots.
-// Zero where the tangent rounds to zero or e is below 2^-960.
-__device__ __noinline__ double jac_half64_tiny(double d, double e) {
-    if (abs_below(e, 0x1p-960)) return 0.0;
-    const double th = d / (2.0 * e);
-    const double t = (th < 0.0 ? -1.0 : 1.0) / (fabs(th) + sqrt(fma(th, th, 1.0)));
-    return t / (1.0 + sqrt(fma(t, t, 1.0)));
-}
 __device__ __forceinline__ double rot_first(double s, double h, double x, double y) { return fma(-s, fma(h, x, y), x); }
 __device__ __forceinline__ double rot_second(double s, double h, double x, double y) { return fma(s, fma(-h, y, x), y); }
 // A symmetric 2 x 2 block [[a, e], [e, b]] under that rotation:

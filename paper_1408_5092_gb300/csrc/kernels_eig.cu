@@ -425,6 +425,16 @@ inline size_t eig_smem(int n, int C) {
     return f.head + (eig_a_sm(n, C) ? f.a : 0) + (eig_v_sm(n, C) ? f.v : 0);
 }
 
+// h of a pair whose e is below 2^-80 of the largest entry: the Newton steps'
+// float32 residuals leave their range there, so by division and square roots.
+// Zero where the tangent rounds to zero or e is below 2^-960.
+__device__ __noinline__ double jac_half64_tiny(double d, double e) {
+    if (abs_below(e, 0x1p-960)) return 0.0;
+    const double th = d / (2.0 * e);
+    const double t = (th < 0.0 ? -1.0 : 1.0) / (fabs(th) + sqrt(fma(th, th, 1.0)));
+    return t / (1.0 + sqrt(fma(t, t, 1.0)));
+}
+
 template <int C, int NT, bool A_SM>
 __device__ __forceinline__ void eig_body(const EigTask& t, double nullrel, int maxs, int* flag, int rank) {
     namespace cg = cooperative_groups;
